@@ -347,7 +347,9 @@ g2_status g2_bfs_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dep
  * near/far queue of g2_sssp_delta (one bit per source in per-vertex masks).
  * Schedules: PUSH with any frontier load balancing but EDGE_ONLY, or kernel
  * fusion with WM PUSH (the whole loop in one cooperative kernel).  NULL
- * schedule: STRICT PUSH; on a bounded-degree graph (largest out-degree <= 32)
+ * schedule: the distances of a vertex from all sources relaxed together as one
+ * row, in rounds over the vertices whose row changed (delta is not used), or
+ * STRICT PUSH where that has not ended after 32 rounds; on a bounded-degree graph (largest out-degree <= 32)
  * the sources run as single-source fused WM queries, about one per 19 SMs at
  * a time, as g2_bfs_batch does (G2_BATCH_SPLIT_WORKERS = 0: the fused
  * multi-source loop). */

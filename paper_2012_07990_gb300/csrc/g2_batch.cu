@@ -691,7 +691,7 @@ using namespace g2;
 
 // Tuned schedules when the caller passes none: multi-source BFS switches from
 // STRICT PUSH to VERTEX_BASED PULL once the union frontier holds 2% of the
-// vertices; multi-source SSSP relaxes with STRICT PUSH.
+// vertices; multi-source SSSP relaxes distance rows.
 // Tuned multi-source BFS: the direction-optimising hybrid (STRICT PUSH below
 // 2% of n, VERTEX_BASED PULL); on a bounded-degree graph the fused WM PUSH
 // loop (thousands of small levels: launches and host round trips dominate).
@@ -713,8 +713,9 @@ static g2_hybrid tuned_batch_bfs(g2_graph *g, cudaStream_t st) {
     return h;
 }
 
-// Tuned multi-source SSSP: STRICT PUSH; the fused WM PUSH loop on a
-// bounded-degree graph.
+// Tuned multi-source SSSP: distance rows (g2_rows.cu; the STRICT PUSH below is
+// its stand-in where the rows do not apply); the fused WM PUSH loop
+// on a bounded-degree graph.
 static g2_hybrid tuned_batch_sssp(g2_graph *g, cudaStream_t st) {
     int32_t dmax = 0;
     if (max_out_degree(g, st, &dmax) == G2_OK && dmax <= kBoundedDegree) {
@@ -857,6 +858,13 @@ g2_status g2_sssp_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t del
             G2_TRY(split_run(g, srcs, k, delta > 0 ? delta : 1, dist, workers, st));
             return end_call(g, st, d_err);
         }
+    }
+    if (!sched && !h.s1.kernel_fusion) {
+        // rows of distances (RMAT-21, 32 sources: 8.2 ms against 42.7 ms for
+        // STRICT delta-stepping over stacked arrays)
+        bool done = false;
+        G2_TRY(sssp_batch_rows(g, srcs, k, dist, st, d_err, &done));
+        if (done) return end_call(g, st, d_err);
     }
     G2_TRY(sssp_batch_run(g, srcs, k, delta, dist, h, st, d_err));
     return end_call(g, st, d_err);

@@ -449,6 +449,23 @@ __device__ __forceinline__ int block_incl_scan(int x, int *s_warp, int *total) {
     return incl + off;
 }
 
+// The last i in [0, size) with scan[i] <= k, given scan[0] <= k < scan[size]
+// (scan not decreasing): 32 probes a step, by a whole warp.
+__device__ __forceinline__ int32_t scan_owner(const int32_t *scan, int32_t size, int32_t k) {
+    const int lane = threadIdx.x & 31;
+    int32_t lo = 0, hi = size;  // scan[lo] <= k < scan[hi]
+    while (hi - lo > 1) {
+        const int32_t step = (int32_t)(((int64_t)hi - lo + 31) / 32);
+        const int64_t p = (int64_t)lo + (int64_t)(lane + 1) * step;
+        const unsigned below = __ballot_sync(G2_FULL, p < hi && scan[p] <= k);
+        const int c = __popc(below);  // the probes at or below k come first
+        const int64_t top = (int64_t)lo + (int64_t)(c + 1) * step;
+        lo += c * step;
+        if (top < hi) hi = (int32_t)top;
+    }
+    return lo;
+}
+
 // Per-warp count of examined arcs into a 64-bit device counter (stats mode).
 __device__ __forceinline__ void count_arcs(unsigned long long *ctr, int k) {
     if (!ctr) return;

@@ -618,6 +618,8 @@ g2_status ensure_coo(g2_graph *g, cudaStream_t st) {
     G2_CK(dmalloc(&t->coo_src, (size_t)t->m * sizeof(int32_t), st));
     k_coo_src<<<grid_for(g, (int64_t)t->n * 32, kCta), kCta, 0, st>>>(t->rowptr, t->n, t->coo_src);
     G2_CK(cudaGetLastError());
+    // built once; a call on another view may use it on its own stream next
+    G2_CK(cudaStreamSynchronize(st));
     return G2_OK;
 }
 
@@ -959,6 +961,7 @@ g2_status g2_load_csr(int32_t n, int64_t m, const int32_t *rowptr, const int32_t
     t->eb_N = 0; t->eb_nseg = 0; t->eb_src = t->eb_dst = nullptr; t->eb_seg = nullptr;
     t->h_eb_seg = nullptr;
     t->max_out_deg = -1;
+    t->max_w = -1;
     t->pr_hot = -1; t->pr_hot_min_deg = 0; t->pr_slot_of = t->pr_ccol = nullptr;
     t->seg_head = nullptr; t->seg_nzrow = t->seg_chunk_rank = nullptr; t->seg_nnzrow = 0;
     t->blk_S = 0; t->blk_nb = 0; t->blk_nchunks = 0; t->blk_nruns = 0; t->blk_nact = 0;

@@ -56,6 +56,7 @@ enum Buf {
     B_I0, B_I1,                    // int32 arrays of n
     B_BIG,                         // dedup-disabled overflow queue (capacity m + n)
     B_MS0, B_MS1, B_MS2,           // multi-source masks (uint64[n])
+    B_ROWS,                        // multi-source distance rows (int32[n][8, 16 or 32])
     B_COUNT
 };
 
@@ -122,6 +123,7 @@ struct Topology {
     // PageRank share-cache layout: the share slot of every vertex, the least
     // out-degree of the cached vertices, the CSC column ids as share slots
     int32_t max_out_deg;  // largest out-degree (-1: not computed yet)
+    int32_t max_w;        // largest arc weight (-1: not computed yet)
     int32_t pr_hot;
     int32_t pr_hot_min_deg;
     int32_t *pr_slot_of, *pr_ccol;
@@ -239,6 +241,11 @@ g2_status pagerank_blk_run(g2_graph *g, float damping, int32_t iters, float *ran
 // thread, releases its handle and stream; returns its status).
 g2_status pr_prepare_start(g2_graph *g, cudaStream_t load_stream);
 g2_status pr_prepare_wait(Topology *t);
+
+// Multi-source SSSP over distance rows (g2_rows.cu); *done tells whether the
+// form applied.
+g2_status sssp_batch_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist,
+                          cudaStream_t st, int32_t *d_err, bool *done);
 
 // Largest out-degree of the graph (computed on the device once, then kept).
 g2_status max_out_degree(g2_graph *g, cudaStream_t st, int32_t *out);
