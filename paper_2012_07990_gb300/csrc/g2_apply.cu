@@ -14,6 +14,15 @@
 namespace g2 {
 
 // ---------------------------------------------------------- kernel wrappers
+// val[u] copied to snap[u] for the members u of the input vertexset
+__global__ void k_snapshot(FrontierIn fin, int32_t fsize, const int32_t *val, int32_t *snap) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < fsize;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t u = fin.vertex((int32_t)i);
+        snap[u] = val[u];
+    }
+}
+
 template <class P, int G>
 __global__ void __launch_bounds__(kCta) k_pull(DevGraph g, const int32_t *cand, int32_t ncand,
                                                Member mem, P op, OutCtx out,
@@ -140,13 +149,15 @@ g2_status apply_round(g2_graph *g, const g2_schedule &s, const OpArgs &a, const 
     KTime kt;
     ktime_begin(kt, s.direction == G2_PUSH ? push_names[a.kind] : pull_names[a.kind], st);
     g2_status r = G2_OK;
+    const int32_t *from = a.from ? a.from : a.i0;
     if (s.direction == G2_PUSH) {
         switch (a.kind) {
             case K_BFS: r = push_round(g, s, OpBFS{a.i0, a.i1}, in, out, ctr, st); break;
             case K_RELAX:
-                r = push_round(g, s, OpRelaxMin{a.i0, dg.w, a.err, a.threshold}, in, out, ctr, st);
+                r = push_round(g, s, OpRelaxMin{a.i0, from, dg.w, a.err, a.threshold}, in, out, ctr,
+                               st);
                 break;
-            case K_LABEL: r = push_round(g, s, OpLabelMin{a.i0}, in, out, ctr, st); break;
+            case K_LABEL: r = push_round(g, s, OpLabelMin{a.i0, from}, in, out, ctr, st); break;
             case K_PR: r = push_round(g, s, OpPRAdd{a.f0, a.f1}, in, out, ctr, st); break;
             case K_SIGMA: r = push_round(g, s, OpBCSigma{a.i0, a.d0}, in, out, ctr, st); break;
             case K_HOOK: r = push_round(g, s, OpHook{a.i0}, in, out, ctr, st); break;
@@ -289,6 +300,17 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         case K_PR: a.f0 = (const float *)vdata; a.f1 = (float *)vdata2; break;
         case K_SIGMA: case K_DELTA: a.i0 = (int32_t *)vdata; a.d0 = (double *)vdata2; break;
         default: break;
+    }
+    // A PUSH round lowers values that are sources' values too.  It relaxes
+    // with the values from before the round (a copy of the sources' values:
+    // 2 us), so that the result does not depend on which CTAs run first.
+    if (s.direction == G2_PUSH && (kind == K_RELAX || kind == K_LABEL) && use.size > 0) {
+        int32_t *snap;
+        G2_TRY(ws(g, B_I0, (size_t)std::max(n, 1), &snap));
+        const FrontierIn fin{use.rep == -1 ? nullptr : use.q, use.size, nullptr};
+        k_snapshot<<<grid_for(g, use.size, kCta), kCta, 0, st>>>(fin, use.size, a.i0, snap);
+        stats().launches += 1;
+        a.from = snap;
     }
     G2_TRY(apply_round(g, s, a, use, o, st));
     s.direction == G2_PUSH ? stats().push_rounds++ : stats().pull_rounds++;

@@ -29,14 +29,22 @@ struct OpMsBfs {
     const u64 *fcur;
     u64 *fnext;
     typedef u64 S;
+    struct Pre {
+        u64 seen, next;
+    };
+    typedef u64 Old;
+    static constexpr int kFlight = 4;
     __device__ __forceinline__ S load(int32_t u) const { return fcur[u]; }
     __device__ __forceinline__ bool skip(S m) const { return m == 0; }
-    __device__ __forceinline__ int relax(int32_t, S fm, int32_t v, int32_t) const {
-        u64 m = fm & ~visit[v];
-        if (m == 0) return 0;
-        if ((fnext[v] & m) == m) return 0;
-        u64 old = atomicOr(&fnext[v], m);
-        return old == 0 ? 1 : 0;
+    __device__ __forceinline__ Pre pre(int32_t v, int32_t) const {
+        return Pre{visit[v], fnext[v]};
+    }
+    __device__ __forceinline__ Old act(int32_t, S fm, int32_t v, int32_t, Pre p) const {
+        const u64 m = fm & ~p.seen;
+        return (p.next & m) == m ? ~0ull : atomicOr(&fnext[v], m);
+    }
+    __device__ __forceinline__ int fin(int32_t, S, int32_t, Pre, Old old) const {
+        return old == 0;
     }
 };
 
@@ -322,9 +330,14 @@ struct OpMsRelax {
     int32_t T;
     int32_t *err;
     typedef unsigned S;
+    typedef int32_t Pre;
+    typedef int Old;
+    static constexpr int kFlight = 1;  // a loop over the mask's bits per arc
     __device__ __forceinline__ S load(int32_t u) const { return mcur[u]; }
     __device__ __forceinline__ bool skip(S m) const { return m == 0; }
-    __device__ __forceinline__ int relax(int32_t u, S mu, int32_t v, int32_t e) const {
+    __device__ __forceinline__ Pre pre(int32_t, int32_t) const { return 0; }
+    __device__ __forceinline__ int fin(int32_t, S, int32_t, Pre, Old code) const { return code; }
+    __device__ __forceinline__ Old act(int32_t u, S mu, int32_t v, int32_t e, Pre) const {
         const int32_t wt = w[e];
         unsigned nb = 0, fb = 0;
         while (mu) {

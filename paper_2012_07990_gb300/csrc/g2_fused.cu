@@ -103,8 +103,9 @@ struct FusedDoBfsArgs {
     int32_t push_below;  // PUSH while the frontier holds fewer vertices
     int32_t *scan;       // STRICT: prefix sums of a PUSH level's degrees (n + 1) ...
     int32_t *ctasum;     // ... and the slice totals of the CTAs (one per CTA)
-    EtwcEntry<int32_t> *spq;  // ETWC: a level's entries of kEtwcSpill arcs or more ...
+    EtwcEntry<int32_t> *spq;  // ETWC: a level's CTA-stage pieces (room for spcap) ...
     int32_t *spcnt;           // ... and their counts per level parity, 0 at launch
+    int32_t spcap;
     int32_t *result;     // [0] levels, [1] PULL levels
     GridBarrier bar;
     int32_t *err;
@@ -214,15 +215,15 @@ __global__ void __launch_bounds__(kCta) k_bfs_fused_do(FusedDoBfsArgs a) {
             out.q = a.q[(d + 1) & 1];
             out.cnt = a.cnt + (d + 1) % 3;
             if (LB == G2_LB_ETWC && a.spcnt) {
-                // Algorithm 3 with the CTA-stage entries of kEtwcSpill arcs or
-                // more handed to a grid-wide pass after the barrier (a hub
-                // would otherwise keep one CTA busy while the rest wait)
+                // Algorithm 3 with the CTA-stage entries handed to a grid-wide
+                // pass after the barrier (a hub would otherwise keep one CTA
+                // busy while the rest wait)
                 int32_t *spc = a.spcnt + (d & 1);
-                lb_etwc(a.g, fin, size, op, out, blockIdx.x, gridDim.x, a.ctr,
-                        EtwcSpill<int32_t>{a.spq, spc});
+                const EtwcSpill<int32_t> spill{a.spq, spc, a.spcap};
+                lb_etwc(a.g, fin, size, op, out, blockIdx.x, gridDim.x, a.ctr, spill);
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
                 if (ld_relaxed_i32(spc) > 0) {
-                    lb_etwc_spill(a.g, a.spq, spc, op, out, blockIdx.x, gridDim.x);
+                    lb_etwc_spill(a.g, spill, op, out, blockIdx.x, gridDim.x);
                     if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
                 }
             } else if (LB == G2_LB_STRICT) {
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kCta) k_sssp_fused(FusedSsspArgs a) {
     for (;;) {
         int32_t size = ld_relaxed_i32(a.ncnt + d % 3);
         if (size > 0) {
-            OpRelaxMin op{a.dist, a.g.w, a.err, (int32_t)(T < G2_INF32 ? T : G2_INF32)};
+            OpRelaxMin op{a.dist, a.dist, a.g.w, a.err, (int32_t)(T < G2_INF32 ? T : G2_INF32)};
             FrontierIn fin{a.nq[d & 1], size, nullptr};
             out.q = a.nq[(d + 1) & 1];
             out.cnt = a.ncnt + (d + 1) % 3;
@@ -1026,6 +1027,7 @@ g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent
     a.bcnt = ctrs + 46;  // [46..48]
     a.spq = nullptr;
     a.spcnt = nullptr;
+    a.spcap = 0;
     a.scan = nullptr;
     a.ctasum = nullptr;
     if (h.s1.load_balance == G2_LB_STRICT) {
@@ -1034,9 +1036,8 @@ g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent
         G2_TRY(ws(g, B_SCANTMP, (size_t)t->sm_count * (2048 / kCta) + 1, &a.ctasum));
     }
     if (h.s1.load_balance == G2_LB_ETWC) {
-        // every handed-off entry has at least kEtwcSpill arcs
-        const size_t cap = (size_t)t->m / kEtwcSpill + 1;
-        G2_TRY(ws(g, B_TWC_L, cap, &a.spq));
+        a.spcap = (int32_t)etwc_spill_cap(n, t->m);
+        G2_TRY(ws(g, B_TWC_L, (size_t)a.spcap, &a.spq));
         a.spcnt = ctrs + 54;  // [54..55]
     }
     const double pb = (double)h.threshold * (double)n;

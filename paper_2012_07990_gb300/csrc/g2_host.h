@@ -322,6 +322,7 @@ struct OpArgs {
     OpKind kind;
     int32_t *i0;       // depth / dist / label
     int32_t *i1;       // parent
+    const int32_t *from;  // RELAX, LABEL: the sources' values (null: read from i0)
     const float *f0;   // contrib
     float *f1;         // acc
     double *d0;        // sigma

@@ -18,10 +18,57 @@ __device__ __forceinline__ T shfl_xor_acc(T x, int d) {
 }
 
 // --------------------------------------------------------------- VERTEX_BASED
+// Every lane walks every stride-th of the len arcs from beg, kFlight a step
+// (len may be negative: none).
+template <class Op>
+__device__ __forceinline__ void walk_lists(const DevGraph &g, const Op &op, const OutCtx &out,
+                                           Stage &st, int32_t u, typename Op::S s, int32_t beg,
+                                           int32_t len, int stride = 1) {
+    constexpr int N = Op::kFlight;
+    const int maxlen = (int)__reduce_max_sync(G2_FULL, (unsigned)max(len, 0));
+    for (int k = 0; k < maxlen; k += N * stride) {
+        int32_t us[N], e[N];
+        typename Op::S ss[N];
+        bool on[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            us[j] = u;
+            ss[j] = s;
+            e[j] = beg + k + j * stride;
+            on[j] = k + j * stride < len;
+        }
+        apply_arcs<N>(op, out, st, us, ss, g.col, e, on);
+    }
+}
+
+// A group of `width` threads (this one is number `t` of it) walks the arcs
+// [beg, end) of one vertex, kFlight steps of `width` arcs at a time.
+template <class Op>
+__device__ __forceinline__ void walk_group(const DevGraph &g, const Op &op, const OutCtx &out,
+                                           Stage &st, int32_t u, typename Op::S s, int32_t beg, int32_t end,
+                                           int t, int width) {
+    constexpr int N = Op::kFlight;
+    for (int64_t e0 = beg; e0 < end; e0 += N * width) {
+        int32_t us[N], e[N];
+        typename Op::S ss[N];
+        bool on[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int64_t k = e0 + j * width + t;
+            us[j] = u;
+            ss[j] = s;
+            on[j] = k < end;
+            e[j] = on[j] ? (int32_t)k : 0;
+        }
+        apply_arcs<N>(op, out, st, us, ss, g.col, e, on);
+    }
+}
+
 // One thread per active vertex, serial walk of its arcs.
 template <class Op>
 __device__ void lb_vertex(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
                           const OutCtx &out, int bid, int nb, unsigned long long *ctr) {
+    Stage st = stage_begin();
     const int lane = threadIdx.x & 31;
     const int gw = bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int nw = nb * (blockDim.x >> 5);
@@ -38,26 +85,21 @@ __device__ void lb_vertex(const DevGraph &g, const FrontierIn &fin, int32_t fsiz
             }
         }
         count_arcs(ctr, len);
-        int maxlen = (int)__reduce_max_sync(G2_FULL, (unsigned)len);
-        for (int k = 0; k < maxlen; ++k) {
-            int code = 0;
-            int32_t v = 0;
-            if (k < len) {
-                v = g.col[beg + k];
-                code = op.relax(u, s, v, beg + k);
-            }
-            emit(out, v, code);
-        }
+        walk_lists(g, op, out, st, u, s, beg, len);
     }
+    stage_end(out, st);
 }
 
 // ------------------------------------------------------------------------ WM
 // A warp takes 32 active vertices, prefix-sums their degrees with shuffles and
-// walks the combined arc range 32 arcs at a time; each lane finds the owner of
-// its arc by a 5-step binary search over the lanes' prefix sums.
+// walks the combined arc range 32 arcs at a time, kFlight such steps in
+// flight; each lane finds the owner of its arc by a 5-step binary search over
+// the lanes' prefix sums.
 template <class Op>
 __device__ void lb_warp(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
                         const OutCtx &out, int bid, int nb, unsigned long long *ctr) {
+    Stage st = stage_begin();
+    constexpr int N = Op::kFlight;
     const int lane = threadIdx.x & 31;
     const int gw = bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int nw = nb * (blockDim.x >> 5);
@@ -76,40 +118,43 @@ __device__ void lb_warp(const DevGraph &g, const FrontierIn &fin, int32_t fsize,
         count_arcs(ctr, len);
         int incl = warp_incl_scan(len);
         int total = __shfl_sync(G2_FULL, incl, 31);
-        int excl = incl - len;
-        for (int k0 = 0; k0 < total; k0 += 32) {
-            int k = k0 + lane;
-            int lo = 0, hi = 31;
+        int off = beg - (incl - len);  // arc k of the range sits at off + k
+        for (int k0 = 0; k0 < total; k0 += 32 * N) {
+            int32_t us[N], e[N];
+            typename Op::S ss[N];
+            bool on[N];
 #pragma unroll
-            for (int st = 0; st < 5; ++st) {
-                int mid = (lo + hi) >> 1;
-                int im = __shfl_sync(G2_FULL, incl, mid);
-                if (im > k) hi = mid;
-                else lo = mid + 1;
+            for (int j = 0; j < N; ++j) {
+                int k = k0 + 32 * j + lane;
+                int lo = 0, hi = 31;
+#pragma unroll
+                for (int b = 0; b < 5; ++b) {
+                    int mid = (lo + hi) >> 1;
+                    int im = __shfl_sync(G2_FULL, incl, mid);
+                    if (im > k) hi = mid;
+                    else lo = mid + 1;
+                }
+                lo &= 31;  // past the range: any lane
+                us[j] = __shfl_sync(G2_FULL, u, lo);
+                ss[j] = shfl(s, lo);
+                e[j] = __shfl_sync(G2_FULL, off, lo) + k;
+                on[j] = k < total;
             }
-            int owner = lo;
-            int32_t ou = __shfl_sync(G2_FULL, u, owner);
-            typename Op::S os = shfl(s, owner);
-            int32_t ob = __shfl_sync(G2_FULL, beg, owner);
-            int oe = __shfl_sync(G2_FULL, excl, owner);
-            int code = 0;
-            int32_t v = 0;
-            if (k < total) {
-                int32_t e = ob + (k - oe);
-                v = g.col[e];
-                code = op.relax(ou, os, v, e);
-            }
-            emit(out, v, code);
+            apply_arcs<N>(op, out, st, us, ss, g.col, e, on);
         }
     }
+    stage_end(out, st);
 }
 
 // ------------------------------------------------------------------------ CM
 // A CTA takes kCta active vertices, block-scans their degrees in shared memory
-// and walks the combined arc range kCta arcs at a time.
+// and walks the combined arc range kCta arcs at a time, kFlight such steps in
+// flight.
 template <class Op>
 __device__ void lb_cta(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
                        const OutCtx &out, int bid, int nb, unsigned long long *ctr) {
+    Stage st = stage_begin();
+    constexpr int N = Op::kFlight;
     __shared__ int s_incl[kCta];
     __shared__ int32_t s_u[kCta];
     __shared__ int32_t s_beg[kCta];
@@ -136,86 +181,155 @@ __device__ void lb_cta(const DevGraph &g, const FrontierIn &fin, int32_t fsize, 
         s_beg[tid] = beg - (incl - len);  // arc index = s_beg[owner] + k
         s_s[tid] = s;
         __syncthreads();
-        for (int k0 = 0; k0 < total; k0 += kCta) {
-            int k = k0 + tid;
-            int code = 0;
-            int32_t v = 0;
-            if (k < total) {
-                int lo = 0, hi = kCta - 1;
+        for (int k0 = 0; k0 < total; k0 += kCta * N) {
+            int32_t us[N], e[N];
+            typename Op::S ss[N];
+            bool on[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const int k = k0 + kCta * j + tid;
+                on[j] = k < total;
+                int lo = 0, hi = on[j] ? kCta - 1 : 0;
                 while (lo < hi) {
                     int mid = (lo + hi) >> 1;
                     if (s_incl[mid] > k) hi = mid;
                     else lo = mid + 1;
                 }
-                int32_t e = s_beg[lo] + k;
-                v = g.col[e];
-                code = op.relax(s_u[lo], s_s[lo], v, e);
+                us[j] = s_u[lo];
+                ss[j] = s_s[lo];
+                e[j] = s_beg[lo] + k;
             }
-            emit(out, v, code);
+            apply_arcs<N>(op, out, st, us, ss, g.col, e, on);
         }
         __syncthreads();
     }
+    stage_end(out, st);
 }
 
 // -------------------------------------------------------------------- STRICT
 // Every thread gets the same number of arcs: arc k of the frontier-wide arc
 // sequence belongs to the active vertex i with scan[i] <= k < scan[i+1]
 // (scan = exclusive prefix sum of the active vertices' degrees, computed by a
-// separate pass); found by binary search per arc.
+// separate pass).  A CTA takes runs of up to kStrictRun consecutive tiles of
+// kTile arcs: a run's first owner by a 32-way search of every warp, the
+// owners of a tile read into shared memory in one pass (each with its source
+// value and arc base, so that an arc reads nothing of its owner from global
+// memory) and found there by binary search, kFlight arcs per thread at
+// once; the next tile starts at the last owner.  A tile with more owners than
+// fit (vertices without arcs in the list) searches the scan itself.
+constexpr int kStrictRun = 8;
+
 template <class Op>
 __device__ void lb_strict(const DevGraph &g, const FrontierIn &fin, int32_t fsize,
                           const int32_t *scan, const Op &op, const OutCtx &out, int bid, int nb,
                           unsigned long long *ctr) {
+    Stage st = stage_begin();
+    constexpr int N = Op::kFlight;
+    constexpr int kTile = kCta * N;
+    constexpr int kOwn = kTile + kCta;  // a tile of one-arc owners and the last one's
+    __shared__ int32_t s_at[kOwn];    // first arc of the owner, from the tile's start
+    __shared__ int32_t s_base[kOwn];  // arc k of the tile sits at s_base[owner] + k
+    __shared__ int32_t s_u[kOwn];
+    __shared__ typename Op::S s_s[kOwn];
+    const int tid = threadIdx.x;
     const int32_t total = scan[fsize];
-    constexpr int kPer = 4;  // arcs per thread per tile
-    const int64_t tile = (int64_t)kCta * kPer;
-    __shared__ int32_t s_lo, s_hi;
-    for (int64_t t0 = (int64_t)bid * tile; t0 < total; t0 += (int64_t)nb * tile) {
-        if (threadIdx.x == 0) {
-            // owners of the first and last arc of the tile
-            int64_t t1 = t0 + tile - 1 < total ? t0 + tile - 1 : total - 1;
-            int lo = 0, hi = fsize - 1;
-            while (lo < hi) {
-                int mid = (lo + hi + 1) >> 1;
-                if (scan[mid] <= t0) lo = mid;
-                else hi = mid - 1;
-            }
-            s_lo = lo;
-            int lo2 = lo, hi2 = fsize - 1;
-            while (lo2 < hi2) {
-                int mid = (lo2 + hi2 + 1) >> 1;
-                if (scan[mid] <= t1) lo2 = mid;
-                else hi2 = mid - 1;
-            }
-            s_hi = lo2;
+    // (tile numbers fit: total < 2^31)
+    const int32_t tiles = (int32_t)(((int64_t)total + kTile - 1) / kTile);
+    // runs of one to kStrictRun tiles, four or more per CTA where there are
+    // as many: neighbouring arcs (a hub's) go to several CTAs
+    int32_t run = tiles / (nb * 4);
+    run = run < 1 ? 1 : run > kStrictRun ? kStrictRun : run;
+    int32_t own0 = 0;
+    int left = 0;  // tiles of the current run
+    for (int32_t it = run * bid; it < tiles; ++it) {
+        const int64_t t0 = (int64_t)it * kTile;
+        if (left == 0) {
+            own0 = scan_owner(scan, fsize, (int32_t)t0);
+            left = run;
         }
-        __syncthreads();
-        const int32_t vlo = s_lo, vhi = s_hi;
-        int cnt = 0;
+        const int len = (int)(total - t0 < kTile ? total - t0 : kTile);
+        // owners of the tile: the entries from own0 on that start before its end
+        int no = 0;
+        bool more = true;
+        while (more && no < kOwn) {
+            const int64_t i = (int64_t)own0 + no + tid;
+            int32_t at = 0;
+            bool in = i < fsize;
+            if (in) {
+                at = (int32_t)((int64_t)scan[i] - t0);
+                in = at < len;
+            }
+            if (in) {
+                const int32_t u = fin.vertex((int32_t)i);
+                s_at[no + tid] = at;
+                s_u[no + tid] = u;
+                s_s[no + tid] = op.load(u);
+                s_base[no + tid] = g.rowptr[u] - at;
+            }
+            const int c = __syncthreads_count(in);
+            more = c == kCta;
+            no += c;
+        }
+        if (!more) {
+            // shared search, the thread's arcs side by side
+            int top = 1;
+            while (top < no) top <<= 1;
+            int lo[N];
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) {
-            int64_t k = t0 + (int64_t)j * kCta + threadIdx.x;
-            int code = 0;
-            int32_t v = 0;
-            if (k < total) {
-                int lo = vlo, hi = vhi;
-                while (lo < hi) {
-                    int mid = (lo + hi + 1) >> 1;
-                    if (scan[mid] <= k) lo = mid;
-                    else hi = mid - 1;
+            for (int j = 0; j < N; ++j) lo[j] = 0;
+            for (int d = top >> 1; d > 0; d >>= 1) {
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    const int m = lo[j] + d;
+                    if (m < no && s_at[m] <= j * kCta + tid) lo[j] = m;
                 }
-                int32_t u = fin.vertex(lo);
-                typename Op::S s = op.load(u);
-                int32_t e = g.rowptr[u] + (int32_t)(k - scan[lo]);
-                v = g.col[e];
-                code = op.relax(u, s, v, e);
-                ++cnt;
             }
-            emit(out, v, code);
+            int cnt = 0;
+            int32_t us[N], e[N];
+            typename Op::S ss[N];
+            bool on[N];
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const int k = j * kCta + tid;
+                on[j] = k < len;
+                us[j] = s_u[lo[j]];
+                ss[j] = s_s[lo[j]];
+                e[j] = s_base[lo[j]] + k;
+                cnt += on[j];
+            }
+            apply_arcs<N>(op, out, st, us, ss, g.col, e, on);
+            count_arcs(ctr, cnt);
+            // the last owner of this tile may reach into the next one
+            own0 += no - 1;
+        } else {
+            int cnt = 0;
+#pragma unroll 1
+            for (int j = 0; j < N; ++j) {
+                const int64_t k = t0 + j * kCta + tid;
+                int32_t us[1] = {0}, e[1] = {0};
+                typename Op::S ss[1] = {};
+                bool on[1] = {k < t0 + len};
+                if (on[0]) {
+                    int32_t lo = own0, hi = fsize - 1;
+                    while (lo < hi) {
+                        const int32_t mid = lo + (hi - lo + 1) / 2;
+                        if (scan[mid] <= k) lo = mid;
+                        else hi = mid - 1;
+                    }
+                    us[0] = fin.vertex(lo);
+                    ss[0] = op.load(us[0]);
+                    e[0] = g.rowptr[us[0]] + (int32_t)(k - scan[lo]);
+                    ++cnt;
+                }
+                apply_arcs<1>(op, out, st, us, ss, g.col, e, on);
+            }
+            count_arcs(ctr, cnt);
+            own0 = scan_owner(scan, fsize, (int32_t)(t0 + len - 1));
         }
-        count_arcs(ctr, cnt);
+        if (--left == 0) it += run * (nb - 1);
         __syncthreads();
     }
+    stage_end(out, st);
 }
 
 // ---------------------------------------------------------------------- ETWC
@@ -230,34 +344,47 @@ struct EtwcEntry {
     S s;
 };
 
-// Frontier-wide hand-off of ETWC's largest CTA-stage entries: a vertex whose
-// CTA-granularity part reaches kEtwcSpill arcs would otherwise keep one CTA
-// busy while the others idle (a hub on a power-law graph: RMAT-22's first
-// round is one 163K-arc vertex); such entries go to a list that a second
-// pass spreads over every CTA (k_push_etwc_spill).  q == null: no hand-off,
-// every entry stays with its CTA, as in Algorithm 3.
-constexpr int32_t kEtwcSpill = 4096;
+// Frontier-wide hand-off of the CTA-stage entries: on a power-law graph a few
+// CTAs hold most of them (RMAT-22's first BFS round is one 163K-arc vertex; a
+// frontier in vertex order puts the hubs into its first CTAs), and the rest
+// of the grid waits.  Such entries go, in pieces of kEtwcPiece arcs, to a
+// list that a second pass spreads over every CTA (k_push_etwc_spill).  q ==
+// null: no hand-off, every entry stays with its CTA, as in Algorithm 3.  An
+// entry that no longer fits the list stays with its CTA too.
+constexpr int32_t kEtwcPiece = 4 * kCta;
 template <class S>
 struct EtwcSpill {
     EtwcEntry<S> *q;
     int32_t *cnt;
+    int32_t cap;
 };
+
+// Room for the hand-off of a frontier without repeats: every entry has at
+// least kCta arcs and one piece that is not full.
+__host__ __device__ inline int64_t etwc_spill_cap(int64_t fsize, int64_t m) {
+    const int64_t big = m / kCta;
+    return (fsize < big ? fsize : big) + m / kEtwcPiece + 1;
+}
 
 template <class Op>
 __device__ void lb_etwc(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
                         const OutCtx &out, int bid, int nb, unsigned long long *ctr,
-                        EtwcSpill<typename Op::S> spill = {nullptr, nullptr}) {
+                        EtwcSpill<typename Op::S> spill = {nullptr, nullptr, 0}) {
+    Stage st = stage_begin();
     typedef typename Op::S S;
     __shared__ EtwcEntry<S> q0[kCta], q1[kCta], q2[kCta];
     __shared__ int n0, n1, n2;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    for (int64_t base = (int64_t)bid * kCta; base < fsize; base += (int64_t)nb * kCta) {
+    // the list in groups of 32, group x to CTA x mod nb: neighbours in the
+    // list (hubs, where it is in vertex order) go to different CTAs
+    const int64_t groups = ((int64_t)fsize + 31) / 32;
+    for (int64_t base = 0; base + bid < groups; base += (int64_t)nb * kWarps) {
         if (tid == 0) n0 = n1 = n2 = 0;
         __syncthreads();
-        int32_t i = (int32_t)base + tid;
+        const int64_t i = (base + (int64_t)wid * nb + bid) * 32 + lane;
         int len0 = 0;
         if (i < fsize) {
-            int32_t u = fin.vertex(i);
+            int32_t u = fin.vertex((int32_t)i);
             S s = op.load(u);
             if (!op.skip(s)) {
                 int32_t beg = g.rowptr[u], end = g.rowptr[u + 1];
@@ -265,9 +392,18 @@ __device__ void lb_etwc(const DevGraph &g, const FrontierIn &fin, int32_t fsize,
                 len0 = size;
                 int32_t c = (size / kCta) * kCta;  // CTA-granularity part
                 if (c > 0) {
-                    if (spill.q && c >= kEtwcSpill) {
-                        spill.q[atomicAdd(spill.cnt, 1)] = EtwcEntry<S>{beg, beg + c, u, s};
-                    } else {
+                    bool keep = true;
+                    if (spill.q) {
+                        const int32_t np = (c + kEtwcPiece - 1) / kEtwcPiece;
+                        const int32_t p = atomicAdd(spill.cnt, np);
+                        keep = p > spill.cap - np;
+                        for (int32_t x = 0; x < np && p + x < spill.cap && p >= 0; ++x) {
+                            const int32_t b = keep ? beg + c : beg + x * kEtwcPiece;
+                            const int32_t e = beg + c - b < kEtwcPiece ? beg + c : b + kEtwcPiece;
+                            spill.q[p + x] = EtwcEntry<S>{b, e, u, s};
+                        }
+                    }
+                    if (keep) {
                         int p = atomicAdd(&n2, 1);
                         q2[p] = EtwcEntry<S>{beg, beg + c, u, s};
                     }
@@ -289,72 +425,51 @@ __device__ void lb_etwc(const DevGraph &g, const FrontierIn &fin, int32_t fsize,
         }
         count_arcs(ctr, len0);
         __syncthreads();
-        // stage 0: one thread per entry
+        // stage 0: four neighbouring threads per entry (one thread per entry
+        // leaves most of a CTA idle behind its longest remainder, and its
+        // reads of the arcs uncoalesced)
         {
-            int32_t beg = 0, len = 0, u = 0;
-            S s{};
-            if (tid < n0) {
-                beg = q0[tid].beg;
-                len = q0[tid].end - beg;
-                u = q0[tid].u;
-                s = q0[tid].s;
-            }
-            int maxlen = (int)__reduce_max_sync(G2_FULL, (unsigned)len);
-            for (int k = 0; k < maxlen; ++k) {
-                int code = 0;
-                int32_t v = 0;
-                if (k < len) {
-                    v = g.col[beg + k];
-                    code = op.relax(u, s, v, beg + k);
+            const int sub = lane & 3;
+            for (int j0 = wid * 8; j0 < n0; j0 += kWarps * 8) {
+                const int j = j0 + (lane >> 2);
+                int32_t beg = 0, len = 0, u = 0;
+                S s{};
+                if (j < n0) {
+                    beg = q0[j].beg;
+                    len = q0[j].end - beg;
+                    u = q0[j].u;
+                    s = q0[j].s;
                 }
-                emit(out, v, code);
+                walk_lists(g, op, out, st, u, s, beg + sub, len - sub, 4);
             }
         }
         // stage 1: one warp per entry, lanes cyclic
         for (int j = wid; j < n1; j += kWarps) {
             EtwcEntry<S> en = q1[j];
-            for (int32_t e = en.beg + lane; e < en.end; e += 32) {
-                int32_t v = g.col[e];
-                emit(out, v, op.relax(en.u, en.s, v, e));
-            }
+            walk_group(g, op, out, st, en.u, en.s, en.beg, en.end, lane, 32);
         }
         // stage 2: the whole CTA per entry
         for (int j = 0; j < n2; ++j) {
             EtwcEntry<S> en = q2[j];
-            for (int32_t e = en.beg + tid; e < en.end; e += kCta) {
-                int32_t v = g.col[e];
-                emit(out, v, op.relax(en.u, en.s, v, e));
-            }
+            walk_group(g, op, out, st, en.u, en.s, en.beg, en.end, tid, kCta);
         }
         __syncthreads();
     }
+    stage_end(out, st);
 }
 
-// The handed-off entries, spread over the grid: entry j's arcs in chunks of
-// kCta arcs, chunk c of every entry taken by CTA c mod gridDim.x.
+// The handed-off pieces, one CTA each in turn.
 template <class Op>
-__device__ void lb_etwc_spill(const DevGraph &g, const EtwcEntry<typename Op::S> *q,
-                              const int32_t *cnt, const Op &op, const OutCtx &out, int bid,
-                              int nb) {
-    const int32_t k = *cnt;
-    const int lane = threadIdx.x & 31;
-    for (int32_t j = 0; j < k; ++j) {
-        const EtwcEntry<typename Op::S> en = q[j];
-        // a warp takes 32 consecutive arcs a step, lanes past the entry's end
-        // emit nothing, so every lane reaches the warp-wide append (entries
-        // are whole multiples of kCta arcs, but the loop does not rely on it)
-        for (int64_t base = en.beg + (int64_t)bid * kCta + (threadIdx.x & ~31); base < en.end;
-             base += (int64_t)nb * kCta) {
-            const int64_t e = base + lane;
-            int32_t v = 0;
-            int code = 0;
-            if (e < en.end) {
-                v = g.col[e];
-                code = op.relax(en.u, en.s, v, (int32_t)e);
-            }
-            emit(out, v, code);
-        }
+__device__ void lb_etwc_spill(const DevGraph &g, const EtwcSpill<typename Op::S> &spill,
+                              const Op &op, const OutCtx &out, int bid, int nb) {
+    Stage st = stage_begin();
+    int32_t k = *spill.cnt;
+    if (k > spill.cap || k < 0) k = spill.cap;
+    for (int32_t j = bid; j < k; j += nb) {
+        const EtwcEntry<typename Op::S> en = spill.q[j];
+        walk_group(g, op, out, st, en.u, en.s, en.beg, en.end, (int)threadIdx.x, kCta);
     }
+    stage_end(out, st);
 }
 
 // ----------------------------------------------------------------------- TWC
@@ -386,6 +501,7 @@ template <class Op>
 __device__ void lb_twc_process(const DevGraph &g, const int32_t *qs, const int32_t *qm,
                                const int32_t *ql, const int32_t *counts, const Op &op,
                                const OutCtx &out, int bid, int nb, unsigned long long *ctr) {
+    Stage st = stage_begin();
     typedef typename Op::S S;
     const int tid = threadIdx.x, lane = tid & 31;
     const int gw = bid * kWarps + (tid >> 5);
@@ -403,51 +519,23 @@ __device__ void lb_twc_process(const DevGraph &g, const int32_t *qs, const int32
             len = g.rowptr[u + 1] - beg;
         }
         count_arcs(ctr, len);
-        int maxlen = (int)__reduce_max_sync(G2_FULL, (unsigned)len);
-        for (int k = 0; k < maxlen; ++k) {
-            int code = 0;
-            int32_t v = 0;
-            if (k < len) {
-                v = g.col[beg + k];
-                code = op.relax(u, s, v, beg + k);
-            }
-            emit(out, v, code);
-        }
+        walk_lists(g, op, out, st, u, s, beg, len);
     }
     // medium: warp per vertex
     for (int32_t j = gw; j < nm; j += nw) {
         int32_t u = qm[j];
-        S s = op.load(u);
         int32_t beg = g.rowptr[u], end = g.rowptr[u + 1];
         if (ctr && lane == 0) atomicAdd(ctr, (unsigned long long)(end - beg));
-        for (int32_t e0 = beg; e0 < end; e0 += 32) {
-            int32_t e = e0 + lane;
-            int code = 0;
-            int32_t v = 0;
-            if (e < end) {
-                v = g.col[e];
-                code = op.relax(u, s, v, e);
-            }
-            emit(out, v, code);
-        }
+        walk_group(g, op, out, st, u, op.load(u), beg, end, lane, 32);
     }
     // large: CTA per vertex
     for (int32_t j = bid; j < nl; j += nb) {
         int32_t u = ql[j];
-        S s = op.load(u);
         int32_t beg = g.rowptr[u], end = g.rowptr[u + 1];
         if (ctr && tid == 0) atomicAdd(ctr, (unsigned long long)(end - beg));
-        for (int32_t e0 = beg; e0 < end; e0 += kCta) {
-            int32_t e = e0 + tid;
-            int code = 0;
-            int32_t v = 0;
-            if (e < end) {
-                v = g.col[e];
-                code = op.relax(u, s, v, e);
-            }
-            emit(out, v, code);
-        }
+        walk_group(g, op, out, st, u, op.load(u), beg, end, tid, kCta);
     }
+    stage_end(out, st);
 }
 
 // ----------------------------------------------------------------- EDGE_ONLY
@@ -457,24 +545,36 @@ template <class Op>
 __device__ void lb_edges(const int32_t *src, const int32_t *dst, int64_t e0, int64_t e1,
                          const Op &op, const OutCtx &out, int bid, int nb,
                          unsigned long long *ctr) {
+    Stage st = stage_begin();
+    constexpr int N = Op::kFlight;
     const int lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nw = (int64_t)nb * (blockDim.x >> 5);
     int cnt = 0;
-    for (int64_t base = e0 + gw * 32; base < e1; base += nw * 32) {
-        int64_t e = base + lane;
-        int code = 0;
-        int32_t v = 0;
-        if (e < e1) {
-            int32_t u = src[e];
-            v = dst[e];
-            typename Op::S s = op.load(u);
-            if (!op.skip(s)) code = op.relax(u, s, v, (int32_t)e);
-            ++cnt;
+    for (int64_t base = e0 + gw * 32 * N; base < e1; base += nw * 32 * N) {
+        int32_t us[N], e[N];
+        typename Op::S ss[N];
+        bool on[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int64_t k = base + 32 * j + lane;
+            on[j] = k < e1;
+            e[j] = on[j] ? (int32_t)k : 0;
+            us[j] = on[j] ? src[e[j]] : 0;
+            cnt += on[j];
         }
-        emit(out, v, code);
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            ss[j] = typename Op::S{};
+            if (on[j]) {
+                ss[j] = op.load(us[j]);
+                on[j] = !op.skip(ss[j]);
+            }
+        }
+        apply_arcs<N>(op, out, st, us, ss, dst, e, on);
     }
     count_arcs(ctr, cnt);
+    stage_end(out, st);
 }
 
 // ---------------------------------------------------------------- PULL side

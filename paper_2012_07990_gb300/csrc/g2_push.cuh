@@ -32,9 +32,9 @@ __global__ void __launch_bounds__(kCta) k_push_etwc(DevGraph g, FrontierIn fin, 
 }
 template <class Op>
 __global__ void __launch_bounds__(kCta) k_push_etwc_spill(DevGraph g,
-                                                          const EtwcEntry<typename Op::S> *q,
-                                                          const int32_t *cnt, Op op, OutCtx out) {
-    lb_etwc_spill(g, q, cnt, op, out, blockIdx.x, gridDim.x);
+                                                          EtwcSpill<typename Op::S> spill, Op op,
+                                                          OutCtx out) {
+    lb_etwc_spill(g, spill, op, out, blockIdx.x, gridDim.x);
 }
 template <class Op>
 __global__ void __launch_bounds__(kCta) k_push_strict(DevGraph g, FrontierIn fin, int32_t fsize,
@@ -92,21 +92,27 @@ inline g2_status push_round(g2_graph *g, const g2_schedule &s, const Op &op, con
             k_push_cta<<<grid_for(g, fsize, kCta), kCta, 0, st>>>(dg, fin, fsize, op, out, ctr);
             break;
         case G2_LB_ETWC: {
-            // entries of kEtwcSpill arcs or more are handed to a second pass
-            // over the whole grid, where the graph has such vertices
+            // CTA-stage entries are handed to a second pass over the whole
+            // grid, where the graph has vertices with that many arcs (RMAT-20,
+            // 52K sorted frontier vertices, 1.64M arcs: 1,079 us with entries
+            // of 4,096 arcs and more handed over, 100 us so)
             int32_t maxdeg = 0;
             G2_TRY(max_out_degree(g, st, &maxdeg));
-            EtwcSpill<typename Op::S> spill{nullptr, nullptr};
-            if (maxdeg >= kEtwcSpill) {
+            EtwcSpill<typename Op::S> spill{nullptr, nullptr, 0};
+            if (maxdeg >= kCta) {
                 int32_t *ctrs;
                 G2_TRY(ws(g, B_CTR, 64, &ctrs));
                 spill.cnt = ctrs + 45;
-                G2_TRY(ws(g, B_TWC_L, (size_t)fsize, &spill.q));
+                spill.cap = (int32_t)etwc_spill_cap(fsize, t->m);
+                G2_TRY(ws(g, B_TWC_L, (size_t)spill.cap, &spill.q));
                 G2_CK(cudaMemsetAsync(spill.cnt, 0, sizeof(int32_t), st));
             }
-            k_push_etwc<<<grid_for(g, fsize, kCta), kCta, 0, st>>>(dg, fin, fsize, op, out, ctr, spill);
+            // two groups of 32 vertices per CTA, so that a small frontier still
+            // fills the chip
+            k_push_etwc<<<grid_for(g, fsize, 64), kCta, 0, st>>>(dg, fin, fsize, op, out, ctr,
+                                                                 spill);
             if (spill.q) {
-                k_push_etwc_spill<<<t->sm_count * 8, kCta, 0, st>>>(dg, spill.q, spill.cnt, op, out);
+                k_push_etwc_spill<<<t->sm_count * 8, kCta, 0, st>>>(dg, spill, op, out);
                 stats().launches += 1;
             }
             break;
@@ -117,8 +123,11 @@ inline g2_status push_round(g2_graph *g, const g2_schedule &s, const Op &op, con
             G2_TRY(ws(g, B_SCAN, (size_t)fsize + 1, &scan));
             k_frontier_degrees<<<grid_for(g, fsize, kCta), kCta, 0, st>>>(dg, fin, fsize, op, deg);
             G2_TRY(exclusive_scan_i32(g, deg, scan, fsize, st));
-            // one tile per kCta*4 arcs; the arc total is on the device, so size
-            // the grid for the resident CTAs and stride
+            // the arc total is on the device: size the grid for the resident
+            // CTAs and stride.  RMAT of 1,300,003 vertices, 107M arcs over 29
+            // delta-stepping rounds: 2,876 us with a serial owner search per
+            // tile, one arc in flight per thread and an append per 32 arcs;
+            // 1,529 us so (latency: 4 CTAs per SM, L2 22%, DRAM 11%)
             k_push_strict<<<t->sm_count * 8, kCta, 0, st>>>(dg, fin, fsize, scan, op, out, ctr);
             stats().launches += 1;
             break;
