@@ -10,17 +10,27 @@
 // vertices of one level can differ by more than the fp64 range, so sigma is an
 // extended-range number: a 64-bit integer mantissa and an int32 exponent per
 // vertex.  The dependency sum delta_v = sum_w sigma_v / sigma_w (1 + delta_w)
-// is formed as m_v * sum_w c_w 2^(e_v - e_w) with c_w = (1 + delta_w) / m_w
-// kept per vertex (one fp64 division per vertex, when its sigma is known),
-// so an arc costs a power-of-two scaling and an add (fp64 is slow on this
-// GPU).
+// is formed as sigma_v * sum_w C_w with C_w = (1 + delta_w) / sigma_w kept per
+// vertex in the same form, so both passes add integers per arc: GB300's fp64
+// units take 16 cycles for a warp's add (delta's pass over RMAT-21: 618 us a
+// source with an fp64 scaling and add per arc and the fp64 finish in one lane
+// of a warp, 583 us so, before the rest below).  fp64 is left to one finish
+// per vertex, 32 vertices at a time.
+//
+// A vertex's mantissa, exponent and level lie in one 16-byte record, so that a
+// neighbour costs one aligned load (one 32-byte sector) whether it counts or
+// not.  The backward pass replaces sigma by C.
 //
 // Schedules: each level's discovery is one edgeset.apply round (PUSH or PULL
-// per the hybrid schedule); with kernel fusion the whole source runs in one
-// persistent cooperative kernel with one grid barrier per level and pass.
-// The sigma and delta pulls give a warp to every vertex and a whole CTA to
-// the vertices with at least kBigDeg arcs, or a thread to every vertex on a
-// symmetric bounded-degree graph.
+// per the hybrid schedule; the tuned schedule finds all depths of a source in
+// one launch of the fused hybrid when there are several sources), then the
+// reached vertices are grouped by level and degree, and sigma and delta are
+// pulled level by level over the groups: a thread, eight lanes, a warp or a
+// CTA per vertex by its degree.  With kernel fusion the whole source runs in
+// one persistent cooperative kernel with one grid barrier per level and pass;
+// there the pulls give a warp to every vertex and a whole CTA to the vertices
+// with at least kBigDeg arcs, or a thread to every vertex on a symmetric
+// bounded-degree graph.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -32,6 +42,9 @@
 #include "g2_lb.cuh"
 
 namespace g2 {
+
+g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
+                       const g2_hybrid &h, cudaStream_t st, int32_t *d_err);
 
 constexpr int32_t kBigDeg = 4096;    // a CTA per vertex from this many arcs
 constexpr int32_t kThreadDeg = 32;   // a thread per vertex below this many arcs
@@ -50,12 +63,19 @@ __device__ __forceinline__ double bf_mant(unsigned long long m) {
     return (double)m * 0x1p-63;
 }
 
-// x * 2^k for k <= 1023, by a multiply with the power of two built from its
-// exponent bits; 0 below 2^-1022 (a term that small is below the rounding of
-// every sum it joins).
-__device__ __forceinline__ double scale2(double x, int k) {
-    if (k < -1022) return 0.0;
-    return x * __hiloint2double((k + 1023) << 20, 0);
+// The value x * 2^e (x > 0 normal) as an extended-range number.
+__device__ __forceinline__ BigF bf_from(double x, int e) {
+    const long long b = __double_as_longlong(x);
+    const int ex = (int)(b >> 52) - 1023;
+    const unsigned long long f = ((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull;
+    return BigF{f << 10, ex + 1 + e};
+}
+
+// a * 2^k as fp64; 0 below 2^-1022 (below the rounding of what it is added to)
+__device__ __forceinline__ double bf_value(BigF a, int k) {
+    const int e = a.e + k;
+    if (a.m == 0 || e < -1021) return 0.0;
+    return bf_mant(a.m) * __hiloint2double((e + 1023) << 20, 0);
 }
 
 // a + b: the smaller mantissa shifted to the larger one's exponent (the
@@ -83,218 +103,374 @@ __device__ __forceinline__ BigF bf_shfl_xor(BigF a, int d) {
     return BigF{__shfl_xor_sync(G2_FULL, a.m, d), __shfl_xor_sync(G2_FULL, a.e, d)};
 }
 
+// What the pulls need of a vertex.
+struct __align__(16) BcRec {
+    unsigned long long m;  // sigma (BigF); C once delta is known
+    int e;
+    int d;                 // level, -1 before sigma is known
+};
+
 struct BcState {
     DevGraph g;
     int32_t *depth;
-    unsigned long long *sm;  // sigma mantissas (BigF)
-    int32_t *se; // sigma exponents
-    // (1 + delta_v) / m_v: 1 / m_v once sigma_v is known, then (1 + delta_v) /
-    // m_v once delta_v is, so that delta_u = m_u * sum over successors w of
-    // coef_w * 2^(e_u - e_w): per arc a scaling and an add, no division
-    double *coef;
+    BcRec *rec;
     double *bc;
     int32_t *lvl;  // all levels, in order
     int32_t src;
-    // level-pass granularity: one thread per vertex on a symmetric
+    // fused kernels' granularity: one thread per vertex on a symmetric
     // bounded-degree graph (every list short), else one warp per vertex and,
     // when some vertex may have kBigDeg or more arcs (`big`), one CTA for those
     int32_t per_thread;
     int32_t big;
 };
 
-// sigma of vertex w at level d+1: sum over in-neighbours u at level d
-__device__ __forceinline__ BigF bc_sigma_part(const BcState &s, int32_t w, int32_t d, int32_t b,
-                                              int32_t e, int32_t step, int32_t off) {
+// One 16-byte load, written out: left to the compiler it became two of 8
+// bytes, and the pulls are bound by the L1 tag look-ups of their loads.
+__device__ __forceinline__ BcRec bc_load(const BcState &s, int32_t v) {
+    unsigned m0, m1;
+    BcRec r;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(m0), "=r"(m1), "=r"(r.e), "=r"(r.d)
+                 : "l"(s.rec + v)
+                 : "memory");
+    r.m = (unsigned long long)m0 | (unsigned long long)m1 << 32;
+    return r;
+}
+
+__device__ __forceinline__ void bc_store(const BcState &s, int32_t v, BigF a, int32_t d) {
+    *reinterpret_cast<int4 *>(s.rec + v) =
+        make_int4((int)(unsigned)a.m, (int)(unsigned)(a.m >> 32), a.e, d);
+}
+
+// A thread's part of a vertex's sum: every step-th arc of list[b, e) from
+// b + off, N records in flight, those of level `want` added in arc order.
+// sigma: the in-neighbours one level up; delta: the out-neighbours one level
+// down.
+template <int N>
+__device__ __forceinline__ BigF bc_part(const BcState &s, const int32_t *list, int32_t want, int32_t b,
+                                        int32_t e, int step, int off) {
     BigF acc{0, 0};
-    for (int32_t k = b + off; k < e; k += step) {
-        int32_t u = s.g.ccol[k];
-        if (s.depth[u] == d) acc = bf_add(acc, BigF{s.sm[u], s.se[u]});
-    }
-    return acc;
-}
-
-// delta of vertex v at level d, over its out-neighbours w at level d+1:
-// the sum of coef_w * 2^(e_v - e_w) (bc_finish_delta multiplies by m_v)
-__device__ __forceinline__ double bc_delta_part(const BcState &s, int32_t v, int32_t d, int32_t b,
-                                                int32_t e, int32_t step, int32_t off) {
-    const int ev = s.se[v];
-    double acc = 0.0;
-    for (int32_t k = b + off; k < e; k += step) {
-        int32_t w = s.g.col[k];
-        if (s.depth[w] == d + 1) acc += scale2(s.coef[w], ev - s.se[w]);
-    }
-    return acc;
-}
-
-// delta_v from the sum of its successors' terms: added to bc (but for the
-// source) and kept as the coefficient the level above uses
-__device__ __forceinline__ void bc_finish_delta(const BcState &s, int32_t v, double sum) {
-    const double dl = bf_mant(s.sm[v]) * sum;
-    if (v != s.src) s.bc[v] += dl;
-    s.coef[v] *= 1.0 + dl;
-}
-
-// sigma_v found: stored, and 1 / m_v as the first coefficient
-__device__ __forceinline__ void bc_finish_sigma(const BcState &s, int32_t v, BigF a) {
-    s.sm[v] = a.m;
-    s.se[v] = a.e;
-    s.coef[v] = 1.0 / bf_mant(a.m);
-}
-
-// The same sums for one thread over a whole (short) list, four arcs' loads in
-// flight at a time and the terms added in arc order, so the result is the
-// one bc_sigma_part / bc_delta_part give with step 1.
-__device__ __forceinline__ BigF bc_sigma_thread(const BcState &s, int32_t w, int32_t d) {
-    const int32_t b = s.g.crowptr[w], e = s.g.crowptr[w + 1];
-    BigF acc{0, 0};
-    for (int32_t k = b; k < e; k += 4) {
-        int32_t u[4], du[4];
+    for (int64_t k0 = (int64_t)b + off; k0 < e; k0 += (int64_t)N * step) {
+        int32_t u[N];
+        BcRec r[N];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) u[j] = k + j < e ? s.g.ccol[k + j] : -1;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) du[j] = u[j] >= 0 ? s.depth[u[j]] : -2;
-        BigF t[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            t[j] = du[j] == d ? BigF{s.sm[u[j]], s.se[u[j]]} : BigF{0, 0};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc = bf_add(acc, t[j]);
-    }
-    return acc;
-}
-
-__device__ __forceinline__ double bc_delta_thread(const BcState &s, int32_t v, int32_t d) {
-    const int32_t b = s.g.rowptr[v], e = s.g.rowptr[v + 1];
-    const int ev = s.se[v];
-    double acc = 0.0;
-    for (int32_t k = b; k < e; k += 4) {
-        int32_t w[4], dw[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = k + j < e ? s.g.col[k + j] : -1;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) dw[j] = w[j] >= 0 ? s.depth[w[j]] : -2;
-        double cw[4];
-        int ew[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool on = dw[j] == d + 1;
-            cw[j] = on ? s.coef[w[j]] : 0.0;
-            ew[j] = on ? s.se[w[j]] : 0;
+        for (int j = 0; j < N; ++j) {
+            const int64_t x = k0 + (int64_t)j * step;
+            u[j] = x < e ? list[x] : -1;
         }
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (dw[j] == d + 1) acc += scale2(cw[j], ev - ew[j]);
+        for (int j = 0; j < N; ++j)
+            if (u[j] >= 0) r[j] = bc_load(s, u[j]);
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+            if (u[j] >= 0 && r[j].d == want) acc = bf_add(acc, BigF{r[j].m, r[j].e});
     }
     return acc;
 }
 
-// Level pass over list[0, cnt): small vertices one per warp, big ones one per
-// CTA.  `bid`/`nb` as in the load-balancing library (plain or fused).
+// sigma_v, v at level d
+__device__ __forceinline__ void bc_finish_sigma(const BcState &s, int32_t v, BigF a, int32_t d) {
+    bc_store(s, v, a, d);
+}
+
+// delta_v from the sum of its successors' C: added to bc (but for the source)
+// and kept as the C that the level above uses
+__device__ __forceinline__ void bc_finish_delta(const BcState &s, int32_t v, BigF sum) {
+    const BcRec r = bc_load(s, v);
+    const double m = bf_mant(r.m), dl = m * bf_value(sum, r.e);
+    if (v != s.src) s.bc[v] += dl;
+    bc_store(s, v, bf_from((1.0 + dl) / m, -r.e), r.d);
+}
+
+template <bool SIGMA>
+__device__ __forceinline__ void bc_finish(const BcState &s, int32_t v, BigF a, int32_t d) {
+    if (SIGMA) bc_finish_sigma(s, v, a, d + 1);
+    else bc_finish_delta(s, v, a);
+}
+
+// The sums for one thread over a whole (short) list.
+__device__ __forceinline__ BigF bc_sigma_thread(const BcState &s, int32_t w, int32_t d) {
+    return bc_part<4>(s, s.g.ccol, d, s.g.crowptr[w], s.g.crowptr[w + 1], 1, 0);
+}
+
+__device__ __forceinline__ BigF bc_delta_thread(const BcState &s, int32_t v, int32_t d) {
+    return bc_part<4>(s, s.g.col, d + 1, s.g.rowptr[v], s.g.rowptr[v + 1], 1, 0);
+}
+
+// Sum of a group's parts (the lanes of a group of G, G a power of two).
+template <int G>
+__device__ __forceinline__ BigF bc_group_sum(BigF a) {
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) a = bf_add(a, bf_shfl_xor(a, o));
+    return a;
+}
+
+// The sum of the CTA's parts, in thread 0.
+__device__ __forceinline__ BigF bc_cta_sum(BigF a) {
+    __shared__ unsigned long long s_m[kWarps];
+    __shared__ int s_e[kWarps];
+    a = bc_group_sum<32>(a);
+    if ((threadIdx.x & 31) == 0) {
+        s_m[threadIdx.x >> 5] = a.m;
+        s_e[threadIdx.x >> 5] = a.e;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int k = 1; k < kWarps; ++k) a = bf_add(a, BigF{s_m[k], s_e[k]});
+    __syncthreads();
+    return a;
+}
+
+// The whole CTA on vertex v.
+template <bool SIGMA>
+__device__ void bc_cta_vertex(const BcState &s, int32_t v, int32_t d) {
+    const int32_t *rp = SIGMA ? s.g.crowptr : s.g.rowptr;
+    const BigF a = bc_cta_sum(bc_part<4>(s, SIGMA ? s.g.ccol : s.g.col, SIGMA ? d : d + 1, rp[v],
+                                         rp[v + 1], kCta, (int)threadIdx.x));
+    if (threadIdx.x == 0) bc_finish<SIGMA>(s, v, a, d);
+}
+
+// Groups of G lanes, a vertex each, over list[0, cnt) (PICK: those with
+// lo <= degree < hi only).  The sums of delta's pass wait in shared memory
+// until 32 can be finished at once (its fp64 takes a warp's time however few
+// lanes it has).
+template <bool SIGMA, int G, int N, bool PICK>
+__device__ __forceinline__ void bc_groups(const BcState &s, const int32_t *list, int32_t cnt,
+                                          int32_t d, int32_t lo, int32_t hi, int bid, int nb) {
+    constexpr bool kWait = !SIGMA && G > 1;
+    __shared__ int32_t s_v[kWait ? kWarps : 1][32];
+    __shared__ int s_e[kWait ? kWarps : 1][32];
+    __shared__ unsigned long long s_m[kWait ? kWarps : 1][32];
+    const int32_t *rp = SIGMA ? s.g.crowptr : s.g.rowptr;
+    const int32_t *arcs = SIGMA ? s.g.ccol : s.g.col;
+    const int lane = threadIdx.x & 31, sub = lane % G, wid = kWait ? threadIdx.x >> 5 : 0;
+    const int64_t gw = (int64_t)bid * kWarps + (threadIdx.x >> 5), nw = (int64_t)nb * kWarps;
+    int waiting = 0;
+    auto flush = [&]() {
+        __syncwarp();
+        if (lane < waiting) bc_finish<SIGMA>(s, s_v[wid][lane], BigF{s_m[wid][lane], s_e[wid][lane]}, d);
+        __syncwarp();
+        waiting = 0;
+    };
+    for (int64_t base = gw * (32 / G); base < cnt; base += nw * (32 / G)) {
+        const int64_t i = base + lane / G;
+        int32_t v = 0, b = 0, e = 0;
+        bool on = i < cnt;
+        if (on) {
+            v = list[i];
+            b = rp[v];
+            e = rp[v + 1];
+            if (PICK) on = e - b >= lo && e - b < hi;
+        }
+        if (!on) b = e = 0;
+        BigF a = bc_part<N>(s, arcs, SIGMA ? d : d + 1, b, e, G, sub);
+        if (G > 1) __syncwarp();
+        a = bc_group_sum<G>(a);
+        const bool lead = on && sub == 0;
+        if (!kWait) {
+            if (lead) bc_finish<SIGMA>(s, v, a, d);
+        } else {
+            const unsigned mask = __ballot_sync(G2_FULL, lead);
+            if (waiting + 32 / G > 32) flush();
+            if (lead) {
+                const int p = waiting + __popc(mask & lanemask_lt());
+                s_v[wid][p] = v;
+                s_m[wid][p] = a.m;
+                s_e[wid][p] = a.e;
+            }
+            waiting += __popc(mask);
+        }
+    }
+    if (kWait) flush();
+}
+
+// Level pass of the fused kernels over list[0, cnt): small vertices one per
+// thread or warp, big ones one per CTA.  The backward pass of the deepest
+// level has no successors to look for (`deepest`).
 template <bool SIGMA>
 __device__ void bc_level_pass(const BcState &s, const int32_t *list, int32_t cnt, int32_t d,
-                              int bid, int nb) {
-    if (s.per_thread) {  // uniform over the grid
+                              int bid, int nb, bool deepest = false) {
+    if (s.per_thread || deepest) {  // uniform over the grid
         const int64_t nt = (int64_t)nb * blockDim.x;
         for (int64_t i = (int64_t)bid * blockDim.x + threadIdx.x; i < cnt; i += nt) {
             const int32_t v = list[i];
-            if (SIGMA) bc_finish_sigma(s, v, bc_sigma_thread(s, v, d));
-            else bc_finish_delta(s, v, bc_delta_thread(s, v, d));
+            if (SIGMA) bc_finish_sigma(s, v, bc_sigma_thread(s, v, d), d + 1);
+            else bc_finish_delta(s, v, deepest ? BigF{0, 0} : bc_delta_thread(s, v, d));
         }
         return;
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int gw = bid * kWarps + wid, nw = nb * kWarps;
-    // threads: vertices with fewer than kThreadDeg arcs (on a power-law
-    // graph most of a level, whose few arcs would leave a warp nearly idle)
-    {
-        const int64_t nt = (int64_t)nb * blockDim.x;
-        for (int64_t i = (int64_t)bid * blockDim.x + threadIdx.x; i < cnt; i += nt) {
-            const int32_t v = list[i];
-            const int32_t deg = SIGMA ? s.g.crowptr[v + 1] - s.g.crowptr[v]
-                                      : s.g.rowptr[v + 1] - s.g.rowptr[v];
-            if (deg >= kThreadDeg) continue;
-            if (SIGMA) bc_finish_sigma(s, v, bc_sigma_thread(s, v, d));
-            else bc_finish_delta(s, v, bc_delta_thread(s, v, d));
-        }
-    }
-    // warps: vertices with kThreadDeg .. kBigDeg - 1 arcs
-    for (int32_t i = gw; i < cnt; i += nw) {
-        int32_t v = list[i];
-        int32_t b = SIGMA ? s.g.crowptr[v] : s.g.rowptr[v];
-        int32_t e = SIGMA ? s.g.crowptr[v + 1] : s.g.rowptr[v + 1];
-        if (e - b < kThreadDeg || e - b >= kBigDeg) continue;
-        if (SIGMA) {
-            BigF a = bc_sigma_part(s, v, d, b, e, 32, lane);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a = bf_add(a, bf_shfl_xor(a, o));
-            if (lane == 0) bc_finish_sigma(s, v, a);
-        } else {
-            double a = bc_delta_part(s, v, d, b, e, 32, lane);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(G2_FULL, a, o);
-            if (lane == 0) bc_finish_delta(s, v, a);
-        }
-    }
-    // CTAs: vertices with at least kBigDeg arcs
-    __shared__ double s_m[kWarps];
-    __shared__ unsigned long long s_mu[kWarps];
-    __shared__ int s_e[kWarps];
+    bc_groups<SIGMA, 1, 4, true>(s, list, cnt, d, 0, kThreadDeg, bid, nb);
+    bc_groups<SIGMA, 32, 4, true>(s, list, cnt, d, kThreadDeg, kBigDeg, bid, nb);
     if (!s.big) return;  // uniform: no vertex has that many arcs
+    const int32_t *rp = SIGMA ? s.g.crowptr : s.g.rowptr;
     for (int32_t i = bid; i < cnt; i += nb) {
-        int32_t v = list[i];
-        int32_t b = SIGMA ? s.g.crowptr[v] : s.g.rowptr[v];
-        int32_t e = SIGMA ? s.g.crowptr[v + 1] : s.g.rowptr[v + 1];
-        if (e - b < kBigDeg) continue;
-        if (SIGMA) {
-            BigF a = bc_sigma_part(s, v, d, b, e, kCta, threadIdx.x);
+        const int32_t v = list[i];
+        if (rp[v + 1] - rp[v] >= kBigDeg) bc_cta_vertex<SIGMA>(s, v, d);
+    }
+}
+
+// --------------------------------------------------- levels grouped by degree
+// The reached vertices sorted by (class, level) into one list: class 0 below
+// 9 arcs (a thread per vertex), 1 below 129 (eight lanes), 2 below kBcPiece (a
+// warp), 3 the rest (a CTA per piece of kBcPiece arcs), so that no pass reads
+// a vertex it does not work on and no CTA walks a hub alone (RMAT-21: a level
+// of three hubs took one CTA 149 us).  Counting sort: k_bc_sort twice, with a
+// scan of the counts between.  The first kBcKeys keys are counted in shared
+// memory (a power-law graph has a dozen levels), one global atomic per key
+// and CTA.
+constexpr int kBcKeys = 256;
+constexpr int kBcPiece = 2048;
+
+__device__ __forceinline__ int bc_class(int32_t deg) {
+    return deg < 9 ? 0 : deg < 129 ? 1 : deg < kBcPiece ? 2 : 3;
+}
+
+template <bool PLACE>
+__global__ void __launch_bounds__(kCta) k_bc_sort(const int32_t *depth, const int32_t *rowptr,
+                                                  int32_t n, int32_t levels, int32_t *cnt,
+                                                  const int32_t *off, int32_t *order) {
+    __shared__ int32_t s_cnt[kBcKeys], s_base[kBcKeys];
+    constexpr int kPer = 8;
+    const int64_t tile = (int64_t)kCta * kPer;
+    for (int64_t t0 = (int64_t)blockIdx.x * tile; t0 < n; t0 += (int64_t)gridDim.x * tile) {
+        for (int i = threadIdx.x; i < kBcKeys; i += kCta) s_cnt[i] = 0;
+        __syncthreads();
+        int key[kPer], pos[kPer];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a = bf_add(a, bf_shfl_xor(a, o));
-            if (lane == 0) {
-                s_mu[wid] = a.m;
-                s_e[wid] = a.e;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                BigF t{0, 0};
-                for (int k = 0; k < kWarps; ++k) t = bf_add(t, BigF{s_mu[k], s_e[k]});
-                bc_finish_sigma(s, v, t);
-            }
-        } else {
-            double a = bc_delta_part(s, v, d, b, e, kCta, threadIdx.x);
+        for (int j = 0; j < kPer; ++j) {
+            const int64_t v = t0 + j * kCta + threadIdx.x;
+            const int32_t dv = v < n ? depth[v] : -1;
+            key[j] = dv < 0 ? -1 : bc_class(rowptr[v + 1] - rowptr[v]) * levels + dv;
+        }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(G2_FULL, a, o);
-            if (lane == 0) s_m[wid] = a;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double t = 0.0;
-                for (int k = 0; k < kWarps; ++k) t += s_m[k];
-                bc_finish_delta(s, v, t);
-            }
+        for (int j = 0; j < kPer; ++j) {
+            // one atomic per key of a warp
+            const unsigned same = __match_any_sync(G2_FULL, key[j]);
+            const int lead = __ffs(same) - 1;
+            int p = 0;
+            if (key[j] >= 0 && (int)(threadIdx.x & 31) == lead)
+                p = atomicAdd(key[j] < kBcKeys ? &s_cnt[key[j]] : &cnt[key[j]], __popc(same));
+            pos[j] = __shfl_sync(G2_FULL, p, lead) + __popc(same & lanemask_lt());
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kBcKeys; i += kCta)
+            if (s_cnt[i]) s_base[i] = atomicAdd(&cnt[i], s_cnt[i]);
+        __syncthreads();
+        if (PLACE) {
+#pragma unroll
+            for (int j = 0; j < kPer; ++j)
+                if (key[j] >= 0)
+                    order[off[key[j]] + (key[j] < kBcKeys ? s_base[key[j]] : 0) + pos[j]] =
+                        (int32_t)(t0 + j * kCta + threadIdx.x);
         }
         __syncthreads();
     }
 }
 
-template <bool SIGMA>
-__global__ void __launch_bounds__(kCta) k_bc_level(BcState s, const int32_t *list, int32_t cnt,
-                                                   int32_t d) {
-    bc_level_pass<SIGMA>(s, list, cnt, d, blockIdx.x, gridDim.x);
+// pieces of the class 3 vertices, and nothing of them done yet
+__global__ void k_bc_pieces(const int32_t *rowptr, const int32_t *hubs, int32_t cnt, int32_t *np,
+                            int32_t *done) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t v = hubs[i];
+        np[i] = (rowptr[v + 1] - rowptr[v] + kBcPiece - 1) / kBcPiece;
+        done[i] = 0;
+    }
 }
 
+// One level's vertices: `list` and the length of each class' part of it.
+struct BcLevel {
+    const int32_t *list[4];
+    int32_t cnt[4];
+    // class 3: first piece of each vertex (cnt[3] + 1 entries; numbers of the
+    // whole graph's pieces), pieces done of each vertex, results of the pieces
+    const int32_t *piece;
+    int32_t *done;
+    int4 *part;
+};
+
+// sigma of the vertices at level d + 1 (SIGMA), or delta of those at level d.
+// The largest first, each class by the whole grid.  Bound: one L1 tag look-up
+// per gathered record (84% of L1's peak with two 8-byte loads a record).  Six
+// CTAs per SM: delta's pass needs 70 registers unbounded (17.4 ms for 16
+// sources of RMAT-21 against 19.4, 17.7 with five, 18.9 with eight); two
+// records in flight per lane instead of four 18.9 ms.
+template <bool SIGMA>
+__global__ void __launch_bounds__(kCta, 6) k_bc_level(BcState s, BcLevel l, int32_t d,
+                                                   int32_t deepest) {
+    if (deepest) {
+        for (int c = 0; c < 4; ++c)
+            for (int64_t i = (int64_t)blockIdx.x * kCta + threadIdx.x; i < l.cnt[c];
+                 i += (int64_t)gridDim.x * kCta)
+                bc_finish_delta(s, l.list[c][i], BigF{0, 0});
+        return;
+    }
+    if (l.cnt[3] > 0) {
+        __shared__ int s_last;
+        const int32_t *rp = SIGMA ? s.g.crowptr : s.g.rowptr;
+        const int32_t p1 = l.piece[l.cnt[3]];
+        for (int32_t p = l.piece[0] + (int32_t)blockIdx.x; p < p1; p += gridDim.x) {
+            const int32_t h = scan_owner(l.piece, l.cnt[3], p);
+            const int32_t v = l.list[3][h], first = l.piece[h], np = l.piece[h + 1] - first;
+            const int32_t e = rp[v + 1], b = rp[v] + (p - first) * kBcPiece;
+            BigF a = bc_cta_sum(bc_part<4>(s, SIGMA ? s.g.ccol : s.g.col, SIGMA ? d : d + 1, b,
+                                           e - b < kBcPiece ? e : b + kBcPiece, kCta,
+                                           (int)threadIdx.x));
+            if (threadIdx.x == 0) {
+                __stcg(l.part + p, make_int4((int)(unsigned)a.m, (int)(unsigned)(a.m >> 32), a.e, 0));
+                __threadfence();
+                s_last = atomicAdd(l.done + h, 1) == np - 1;
+            }
+            __syncthreads();
+            if (s_last) {
+                // the last piece to end sums the results, always in one order
+                __threadfence();
+                a = BigF{0, 0};
+                for (int32_t j = threadIdx.x; j < np; j += kCta) {
+                    const int4 r = __ldcg(l.part + first + j);
+                    a = bf_add(a, BigF{(unsigned long long)(unsigned)r.x |
+                                           (unsigned long long)(unsigned)r.y << 32,
+                                       r.z});
+                }
+                a = bc_cta_sum(a);
+                if (threadIdx.x == 0) {
+                    l.done[h] = 0;  // for the backward pass
+                    bc_finish<SIGMA>(s, v, a, d);
+                }
+            }
+            __syncthreads();
+        }
+    }
+    bc_groups<SIGMA, 32, 4, false>(s, l.list[2], l.cnt[2], d, 0, 0, blockIdx.x, gridDim.x);
+    bc_groups<SIGMA, 8, 4, false>(s, l.list[1], l.cnt[1], d, 0, 0, blockIdx.x, gridDim.x);
+    bc_groups<SIGMA, 1, 4, false>(s, l.list[0], l.cnt[0], d, 0, 0, blockIdx.x, gridDim.x);
+}
+
+// depths and records before the source's search (its own set)
 __global__ void k_bc_init(BcState s, int32_t n, int32_t *cnt3) {
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
          v += (int64_t)gridDim.x * blockDim.x) {
-        bool is_src = v == s.src;
+        const bool is_src = v == s.src;
         s.depth[v] = is_src ? 0 : -1;
-        s.sm[v] = is_src ? (1ull << 62) : 0ull;  // sigma(src) = 1 = 2^62 * 2^(1 - 63)
-        s.se[v] = is_src ? 1 : 0;
-        s.coef[v] = is_src ? 2.0 : 0.0;  // 1 / m_src
+        // sigma(src) = 1 = 2^62 * 2^(1 - 63)
+        bc_finish_sigma(s, (int32_t)v, BigF{is_src ? 1ull << 62 : 0ull, is_src ? 1 : 0},
+                        is_src ? 0 : -1);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         s.lvl[0] = s.src;
         if (cnt3) {
             cnt3[0] = cnt3[1] = cnt3[2] = 0;
         }
+    }
+}
+
+// the records alone
+__global__ void k_bc_init_rec(BcState s, int32_t n) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const bool is_src = v == s.src;
+        bc_finish_sigma(s, (int32_t)v, BigF{is_src ? 1ull << 62 : 0ull, is_src ? 1 : 0},
+                        is_src ? 0 : -1);
     }
 }
 
@@ -309,8 +485,9 @@ struct BcFusedArgs {
     int32_t fwd;     // 1: forward phases from level d0, whose list is lvl[b0, e0)
     int32_t d0, b0, e0;
     int32_t lo;      // > 0: after a phase, stop before a level of fewer vertices
-    int32_t bwd;     // 1: backward pass after the forward pass (levels D-2 .. 0)
+    int32_t bwd;     // 1: backward pass after the forward pass (levels D-1 .. 0)
     int32_t Lhi, Llo;  // without the forward pass: backward over levels Lhi down to Llo
+    int32_t deepest;   // ... of which this one is the deepest (no successors)
     int32_t *result; // out: [0] 1 if stopped for the cluster loop, [1] levels found (or
                      // the next level), [2] its start in lvl, [3] its size
 };
@@ -318,7 +495,7 @@ struct BcFusedArgs {
 template <int LB>
 __global__ void __launch_bounds__(kCta) k_bc_fused(BcFusedArgs a) {
     const BcState &s = a.s;
-    int32_t Lhi = a.Lhi;
+    int32_t Lhi = a.Lhi, deepest = a.deepest;
     const int32_t Llo = a.Llo;
     if (a.fwd) {
         OpBFS op{s.depth, nullptr};
@@ -364,11 +541,11 @@ __global__ void __launch_bounds__(kCta) k_bc_fused(BcFusedArgs a) {
             a.result[1] = d + 1;
         }
         if (!a.bwd) return;
-        Lhi = d - 1;  // levels 0..d: from the deepest but one
+        Lhi = deepest = d;  // levels 0..d
     }
     for (int32_t L = Lhi; L >= Llo; --L) {
         const int32_t lb0 = ld_relaxed_i32(a.off + L), lb1 = ld_relaxed_i32(a.off + L + 1);
-        bc_level_pass<false>(s, s.lvl + lb0, lb1 - lb0, L, blockIdx.x, gridDim.x);
+        bc_level_pass<false>(s, s.lvl + lb0, lb1 - lb0, L, blockIdx.x, gridDim.x, L == deepest);
         if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
     }
 }
@@ -398,6 +575,7 @@ struct ClusterBcArgs {
     int32_t d0, start0, n0;
     int32_t hi;       // stop before a level with more vertices
     int32_t Lhi, Llo; // without the forward pass: backward over levels Lhi down to Llo
+    int32_t deepest;  // ... of which this one is the deepest (no successors)
     int32_t *result;  // out: [0] CL_DONE / CL_TO_GRID / CL_OVERFLOW, [1] levels found (or
                       // the level handed over), [2] its start in lvl, [3] its size
 };
@@ -420,7 +598,7 @@ __global__ void __launch_bounds__(kClCta, 1) k_bc_cluster(ClusterBcArgs a) {
             const int32_t hi = (int32_t)((int64_t)cnt * (rank + 1) / CL);
             for (int32_t i = lo + threadIdx.x; i < hi; i += kClCta) {
                 const int32_t v = s.lvl[b0 + i];
-                bc_finish_delta(s, v, bc_delta_thread(s, v, L));
+                bc_finish_delta(s, v, L == a.deepest ? BigF{0, 0} : bc_delta_thread(s, v, L));
             }
             cl_barrier();  // level L's dependencies visible to level L-1
         }
@@ -486,7 +664,7 @@ __global__ void __launch_bounds__(kClCta, 1) k_bc_cluster(ClusterBcArgs a) {
                 }
                 beg = __ldg(rowptr + u);
                 deg = __ldg(rowptr + u + 1) - beg;
-                if (d > 0) bc_finish_sigma(s, u, bc_sigma_thread(s, u, d - 1));
+                if (d > 0) bc_finish_sigma(s, u, bc_sigma_thread(s, u, d - 1), d);
             }
             int32_t incl = deg;
 #pragma unroll
@@ -533,8 +711,9 @@ __global__ void __launch_bounds__(kClCta, 1) k_bc_cluster(ClusterBcArgs a) {
 }
 
 // ------------------------------------------------------------------- host
-static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h,
-                              std::vector<int32_t> &off, cudaStream_t st, int32_t *d_err) {
+// The source's depths by one edgeset.apply round per level.  *levels: how many.
+static g2_status bc_depths(g2_graph *g, const BcState &s, const g2_hybrid &h, int32_t *levels,
+                           cudaStream_t st, int32_t *d_err) {
     Topology *t = g->topo;
     const int32_t n = t->n;
     int32_t *ctrs = d_err - 62;
@@ -542,13 +721,9 @@ static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h,
     uint8_t *bo;
     G2_TRY(ws(g, B_BM0, (size_t)(n + 31) / 32 + 1, &bm));
     G2_TRY(ws(g, B_BOOL0, (size_t)std::max(n, 1), &bo));
-    k_bc_init<<<grid_for(g, n, kCta), kCta, 0, st>>>(s, n, nullptr);
-    stats().launches += 1;
-    off.assign(1, 0);
-    off.push_back(1);
+    int32_t b = 0, e = 1;
     for (int d = 0;; ++d) {
-        int32_t b = off[d], e = off[d + 1];
-        int32_t size = e - b;
+        const int32_t size = e - b;
         const g2_schedule &sc = pick_schedule(h, size, n);
         G2_TRY(check_schedule(g, sc, K_BFS, false));
         if (sc.load_balance == G2_LB_EDGE_ONLY)
@@ -568,7 +743,7 @@ static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h,
         a.threshold = G2_INF32;
         OutArgs o;
         memset(&o, 0, sizeof(o));
-        o.rep = OUT_SPARSE;  // the level lists are needed for the backward pass
+        o.rep = OUT_SPARSE;
         o.q = s.lvl + e;
         o.qcap = n - e;
         o.cnt = ctrs + 3;
@@ -577,20 +752,112 @@ static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h,
         G2_TRY(apply_round(g, sc, a, in, o, st));
         sc.direction == G2_PUSH ? stats().push_rounds++ : stats().pull_rounds++;
         G2_TRY(read_counters(g, ctrs, 4, st, d_err));
-        int32_t nn = g->h_ctr[3];
-        if (nn == 0) break;
-        k_bc_level<true><<<grid_for(g, (int64_t)nn * 32, kCta), kCta, 0, st>>>(s, s.lvl + e, nn, d);
-        stats().launches += 1;
+        const int32_t nn = g->h_ctr[3];
+        if (nn == 0) {
+            *levels = d + 1;
+            return G2_OK;
+        }
         stats().iterations++;
-        off.push_back(e + nn);
+        b = e;
+        e += nn;
     }
-    const int D = (int)off.size() - 1;  // number of levels
-    for (int L = D - 2; L >= 0; --L) {
-        int32_t cnt = off[L + 1] - off[L];
-        k_bc_level<false><<<grid_for(g, (int64_t)cnt * 32, kCta), kCta, 0, st>>>(s, s.lvl + off[L],
-                                                                                cnt, L);
+}
+
+// A source's levels grouped by class (bc_group): bounds on the host.
+struct BcGroups {
+    std::vector<int32_t> off;  // class c of level L: order[off[c * levels + L], off[c * levels + L + 1])
+    int32_t levels;
+    const int32_t *piece;
+    int32_t *done;
+    int4 *part;
+};
+
+// The vertices of every level grouped by class of their degree in `rowptr`
+// into s.lvl.
+static g2_status bc_group(g2_graph *g, const BcState &s, const int32_t *rowptr, int32_t levels,
+                          BcGroups &gr, cudaStream_t st, int32_t *d_err) {
+    const int32_t n = g->topo->n, keys = std::max(4 * levels, kBcKeys);
+    int32_t *cnt, *doff;
+    G2_TRY(ws(g, B_I1, (size_t)keys, &cnt));
+    G2_TRY(ws(g, B_SCAN, (size_t)keys + 1, &doff));
+    const int grid = grid_for(g, n, kCta * 8);
+    G2_CK(cudaMemsetAsync(cnt, 0, (size_t)keys * 4, st));
+    k_bc_sort<false><<<grid, kCta, 0, st>>>(s.depth, rowptr, n, levels, cnt, nullptr, nullptr);
+    G2_TRY(exclusive_scan_i32(g, cnt, doff, keys, st));
+    G2_CK(cudaMemsetAsync(cnt, 0, (size_t)keys * 4, st));
+    k_bc_sort<true><<<grid, kCta, 0, st>>>(s.depth, rowptr, n, levels, cnt, doff, s.lvl);
+    stats().launches += 2;
+    gr.levels = levels;
+    gr.off.resize((size_t)4 * levels + 1);
+    G2_CK(cudaMemcpyAsync(gr.off.data(), doff, gr.off.size() * 4, cudaMemcpyDeviceToHost, st));
+    G2_TRY(sync_and_check(g, st, d_err));
+    const int32_t h0 = gr.off[(size_t)3 * levels], hubs = gr.off[(size_t)4 * levels] - h0;
+    gr.piece = nullptr;
+    gr.done = nullptr;
+    gr.part = nullptr;
+    if (hubs > 0) {
+        int32_t *np, *piece;
+        G2_TRY(ws(g, B_TWC_S, (size_t)hubs, &np));
+        G2_TRY(ws(g, B_TWC_M, (size_t)hubs + 1, &piece));
+        G2_TRY(ws(g, B_TWC_L, (size_t)hubs, &gr.done));
+        // every piece but a vertex's last is full
+        G2_TRY(ws(g, B_D1, (size_t)g->topo->m / kBcPiece + (size_t)hubs, &gr.part));
+        k_bc_pieces<<<grid_for(g, hubs, kCta), kCta, 0, st>>>(rowptr, s.lvl + h0, hubs, np, gr.done);
+        G2_TRY(exclusive_scan_i32(g, np, piece, hubs, st));
         stats().launches += 1;
+        gr.piece = piece;
     }
+    return G2_OK;
+}
+
+// One level's pass over the groups.
+template <bool SIGMA>
+static void launch_level(g2_graph *g, const BcState &s, const BcGroups &gr, int32_t level, int32_t d,
+                         bool deepest, cudaStream_t st) {
+    BcLevel l;
+    for (int c = 0; c < 4; ++c) {
+        const int32_t *o = gr.off.data() + (size_t)c * gr.levels + level;
+        l.list[c] = s.lvl + o[0];
+        l.cnt[c] = o[1] - o[0];
+    }
+    const int32_t h = gr.off[(size_t)3 * gr.levels + level] - gr.off[(size_t)3 * gr.levels];
+    l.piece = gr.piece ? gr.piece + h : nullptr;
+    l.done = gr.done ? gr.done + h : nullptr;
+    l.part = gr.part;
+    // enough CTAs for every class at once, of hubs with a few dozen pieces
+    const int64_t want = (int64_t)l.cnt[3] * 32 + (l.cnt[2] + kWarps - 1) / kWarps +
+                         (l.cnt[1] + kCta / 8 - 1) / (kCta / 8) + (l.cnt[0] + kCta - 1) / kCta;
+    k_bc_level<SIGMA><<<grid_for(g, want, 1), kCta, 0, st>>>(s, l, d, deepest);
+    stats().launches += 1;
+}
+
+// One source: depths (one fused launch with `fused_depths`, else a round per
+// level), the levels grouped, sigma level by level, delta from the deepest.
+static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h, bool fused_depths,
+                              BcGroups &gr, cudaStream_t st, int32_t *d_err) {
+    Topology *t = g->topo;
+    const int32_t n = t->n;
+    int32_t levels = 0;
+    if (fused_depths) {
+        const int32_t it = stats().iterations, push = stats().push_rounds, pull = stats().pull_rounds;
+        // the hybrid's counters, zero at the start of a call, lie in ctrs[20, 56)
+        G2_CK(cudaMemsetAsync(d_err - 62 + 20, 0, 36 * 4, st));
+        G2_TRY(bfs_fused_do(g, s.src, s.depth, nullptr, h, st, d_err));
+        levels = stats().iterations;
+        stats().iterations += it - 1;
+        stats().push_rounds += push;
+        stats().pull_rounds += pull;
+        k_bc_init_rec<<<grid_for(g, n, kCta), kCta, 0, st>>>(s, n);
+    } else {
+        k_bc_init<<<grid_for(g, n, kCta), kCta, 0, st>>>(s, n, nullptr);
+        G2_TRY(bc_depths(g, s, h, &levels, st, d_err));
+    }
+    stats().launches += 1;
+    G2_TRY(bc_group(g, s, s.g.crowptr, levels, gr, st, d_err));
+    for (int32_t L = 1; L < levels; ++L) launch_level<true>(g, s, gr, L, L - 1, false, st);
+    if (!t->symmetric) G2_TRY(bc_group(g, s, s.g.rowptr, levels, gr, st, d_err));
+    for (int32_t L = levels - 1; L >= 0; --L)
+        launch_level<false>(g, s, gr, L, L, L == levels - 1, st);
     G2_CK(cudaGetLastError());
     return G2_OK;
 }
@@ -749,12 +1016,13 @@ static g2_status bc_one_cluster(g2_graph *g, const BcState &s, const g2_schedule
     }
     stats().iterations += D;
     stats().barriers += 2 * D;
-    // backward over levels D-2 .. 0, by ranges of small / large levels
-    if (D < 2) return G2_OK;
+    // backward over levels D-1 .. 0, by ranges of small / large levels
+    if (D < 2) return G2_OK;  // (the source alone)
+    c.deepest = a.deepest = D - 1;
     std::vector<int32_t> offs((size_t)D + 1);
     G2_CK(cudaMemcpyAsync(offs.data(), off, ((size_t)D + 1) * 4, cudaMemcpyDeviceToHost, st));
     G2_TRY(sync_and_check(g, st, d_err));
-    for (int32_t L = D - 2; L >= 0;) {
+    for (int32_t L = D - 1; L >= 0;) {
         const bool small = offs[L + 1] - offs[L] <= c.hi;
         int32_t Llo = L;
         while (Llo > 0 && (offs[Llo] - offs[Llo - 1] <= c.hi) == small) --Llo;
@@ -775,7 +1043,7 @@ static g2_status bc_one_cluster(g2_graph *g, const BcState &s, const g2_schedule
 }
 
 g2_status bc_run(g2_graph *g, const int32_t *srcs, int32_t k, double *bc, const g2_hybrid &h,
-                 cudaStream_t st, int32_t *d_err) {
+                 bool fused_depths, cudaStream_t st, int32_t *d_err) {
     Topology *t = g->topo;
     const int32_t n = t->n;
     BcState s;
@@ -787,11 +1055,9 @@ g2_status bc_run(g2_graph *g, const int32_t *srcs, int32_t k, double *bc, const 
     s.big = !(t->symmetric && dmax < kBigDeg);
     G2_TRY(ws(g, B_I0, (size_t)std::max(n, 1), &s.depth));
     G2_TRY(ws(g, B_LVL, (size_t)std::max(n, 1), &s.lvl));
-    G2_TRY(ws(g, B_D0, (size_t)std::max(n, 1), &s.sm));
-    G2_TRY(ws(g, B_D1, (size_t)std::max(n, 1), &s.coef));
-    G2_TRY(ws(g, B_F2, (size_t)std::max(n, 1), &s.se));
+    G2_TRY(ws(g, B_D0, (size_t)std::max(n, 1), &s.rec));
     G2_CK(cudaMemsetAsync(bc, 0, (size_t)n * 8, st));
-    std::vector<int32_t> off;
+    BcGroups groups;
     // fused WM sources on a symmetric bounded-degree graph use the cluster
     const int cl = h.s1.kernel_fusion && h.s1.load_balance == G2_LB_WM && s.per_thread
                        ? cluster_size(2, k_bc_cluster<16>, k_bc_cluster<8>, kBcSmem)
@@ -800,7 +1066,7 @@ g2_status bc_run(g2_graph *g, const int32_t *srcs, int32_t k, double *bc, const 
         s.src = srcs[i];
         if (cl) G2_TRY(bc_one_cluster(g, s, h.s1, cl, st, d_err));
         else if (h.s1.kernel_fusion) G2_TRY(bc_one_fused(g, s, h.s1, st, d_err));
-        else G2_TRY(bc_one_plain(g, s, h, off, st, d_err));
+        else G2_TRY(bc_one_plain(g, s, h, fused_depths, groups, st, d_err));
         G2_TRY(sync_and_check(g, st, d_err));
     }
     return G2_OK;
@@ -844,6 +1110,11 @@ extern "C" g2_status g2_bc(g2_graph *g, const int32_t *srcs, int32_t k, double *
         return fail(G2_EUNSUPPORTED, "kernel fusion must be set on both hybrid schedules");
     int32_t *d_err;
     G2_TRY(begin_call(g, st, &d_err));
-    G2_TRY(bc_run(g, srcs, k, bc, h, st, d_err));
+    // Tuned, several sources on a power-law graph: each source's depths in one
+    // launch of the fused direction-optimising hybrid.  (A single source keeps
+    // the rounds: that cooperative launch needs every SM at once, and a server
+    // runs single sources beside other streams.)
+    const bool fused_depths = !sched && !h.s1.kernel_fusion && k > 1;
+    G2_TRY(bc_run(g, srcs, k, bc, h, fused_depths, st, d_err));
     return end_call(g, st, d_err);
 }
