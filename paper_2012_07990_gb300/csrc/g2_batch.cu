@@ -48,51 +48,257 @@ struct OpMsBfs {
     }
 };
 
-// PULL: v ORs the frontier masks of its in-neighbours, stops once every
-// source has reached it.
-struct PullMsBfs {
-    u64 *visit;
-    const u64 *fcur;
-    u64 *fnext;
-    int32_t *depth;
+// Where the levels of a search go.  Up to kMsPlanes levels' bits are kept as
+// bit planes: bit b of plane[j][v] is bit j of the depth of v from source b, so
+// that a round writes 8 bytes a plane and vertex, and k_ms_out writes every
+// depth once, in order.  (Written to depth[b][v] round by round, the 64 arrays
+// took 446 us of RMAT-21's rounds in part lines, beside 80 us to clear them.)
+// A search of more levels goes on writing its depths directly.
+constexpr int kMsPlanes = 5;  // depths up to 31
+struct MsLevels {
+    u64 *plane[kMsPlanes];
+    int32_t *depth;  // null while the planes are used
     int32_t n;
-    int32_t level;  // depth assigned this round
-    u64 full;
-    typedef u64 Ctx;
-    typedef u64 Acc;
-    __device__ __forceinline__ Ctx ctx(int32_t v) const { return visit[v]; }
-    __device__ __forceinline__ bool filter(Ctx c) const { return c != full; }
-    __device__ __forceinline__ Acc identity() const { return 0ull; }
-    __device__ __forceinline__ Acc edge(Ctx, int32_t u, int32_t) const { return fcur[u]; }
-    __device__ __forceinline__ Acc combine(Acc a, Acc b) const { return a | b; }
-    __device__ __forceinline__ bool stop(Acc a) const { return (a & full) == full; }
-    __device__ __forceinline__ int finish(int32_t v, Ctx c, Acc a) const {
-        u64 nm = a & ~c & full;
-        if (!nm) return 0;
-        fnext[v] = nm;
-        visit[v] = c | nm;
-        while (nm) {
-            int i = __ffsll((long long)nm) - 1;
-            nm &= nm - 1;
-            depth[(int64_t)i * n + v] = level;
-        }
-        return 1;
-    }
 };
 
-// after a PUSH round: newly reached bits become visited, depths written
-__global__ void k_ms_commit(const int32_t *touched, int32_t cnt, u64 *visit, const u64 *fnext,
-                            int32_t *depth, int32_t n, int32_t level) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int32_t v = touched[i];
-        u64 nm = fnext[v];
-        visit[v] |= nm;
-        while (nm) {
-            int b = __ffsll((long long)nm) - 1;
-            nm &= nm - 1;
-            depth[(int64_t)b * n + v] = level;
+// The lanes' vertices v (nm: new bits) at `level`.  Called by all 32 lanes.
+__device__ __forceinline__ void ms_set_level(const MsLevels &l, int32_t v, u64 nm, int32_t level) {
+    if (!l.depth) {
+#pragma unroll
+        for (int j = 0; j < kMsPlanes; ++j)
+            if (nm && ((level >> j) & 1)) l.plane[j][v] |= nm;
+        return;
+    }
+    u64 any = (u64)__reduce_or_sync(G2_FULL, (unsigned)nm) |
+              (u64)__reduce_or_sync(G2_FULL, (unsigned)(nm >> 32)) << 32;
+    while (any) {
+        const int b = __ffsll((long long)any) - 1;
+        any &= any - 1;
+        if ((nm >> b) & 1u) l.depth[(int64_t)b * l.n + v] = level;
+    }
+}
+
+// depth[b][v] of every source b < k from the first `planes` planes (-1 where
+// visit has not the bit).
+__global__ void __launch_bounds__(kCta) k_ms_out(MsLevels l, const u64 *visit, int32_t planes,
+                                                 int32_t k, int32_t *depth) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < l.n;
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const u64 seen = visit[v];
+        u64 p[kMsPlanes];
+#pragma unroll
+        for (int j = 0; j < kMsPlanes; ++j) p[j] = j < planes ? l.plane[j][v] : 0;
+#pragma unroll 8
+        for (int b = 0; b < k; ++b) {
+            int32_t d = 0;
+#pragma unroll
+            for (int j = 0; j < kMsPlanes; ++j) d |= (int32_t)((p[j] >> b) & 1u) << j;
+            depth[(int64_t)b * l.n + v] = (seen >> b) & 1u ? d : -1;
         }
+    }
+}
+
+// the bits of the warp's new masks into *active.  Called by all 32 lanes.
+__device__ __forceinline__ void ms_note_active(u64 *active, u64 nm) {
+    const u64 any = (u64)__reduce_or_sync(G2_FULL, (unsigned)nm) |
+                    (u64)__reduce_or_sync(G2_FULL, (unsigned)(nm >> 32)) << 32;
+    if ((threadIdx.x & 31) == 0 && (any & ~*active)) atomicOr(active, any);
+}
+
+// PULL: every vertex ORs the frontier masks of its in-neighbours and stops
+// once it has every bit it can still get: those not yet visited of the sources
+// whose frontier is not empty (`active`; a source in a small component ends
+// after a level or two, and waiting for its bit made every vertex read its
+// whole list).  Three kernels by the length of the list: k_ms_pull_pieces for
+// kMsPiece arcs and more, k_ms_pull for the first kMsThread arcs of the rest, a
+// thread each, k_ms_pull_rest for what those threads leave, a warp each from a
+// list (left to the warp that found them, the low ids of a power-law graph
+// held it for half a millisecond).  They only collect fnext; k_ms_commit_all
+// then passes over the vertices in order.  RMAT-21, 64 sources: the four pull
+// rounds took 1.99 ms with a thread per vertex waiting for every source (6 ms
+// where one source lay in a small component), 0.35 ms so, 0.15 ms to commit.
+struct MsPullArgs {
+    DevGraph g;
+    const u64 *visit;
+    const u64 *fcur;
+    u64 *fnext;
+    const u64 *active;  // sources with a frontier
+    int32_t *rest, *rest_cnt;
+    int32_t *err;
+    unsigned long long *ctr;
+};
+
+constexpr int32_t kMsThread = 32;   // arcs a thread walks alone
+constexpr int32_t kMsPiece = 2048;  // arcs of a big vertex a CTA takes
+
+// the OR of up to four masks, in flight together, at arcs e, e + step, ...
+__device__ __forceinline__ u64 ms_gather(const MsPullArgs &a, int64_t e, int step, int64_t end) {
+    int32_t u[4];
+    u64 m = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) u[j] = e + (int64_t)j * step < end ? a.g.ccol[e + (int64_t)j * step] : -1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (u[j] >= 0) m |= a.fcur[u[j]];
+    return m;
+}
+
+__global__ void __launch_bounds__(kCta) k_ms_pull(MsPullArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const u64 active = *a.active;
+    const int32_t n = a.g.n;
+    OutCtx out;
+    memset(&out, 0, sizeof(out));
+    out.mode = OUT_SPARSE;
+    out.q = a.rest;
+    out.cnt = a.rest_cnt;
+    out.cap = n;
+    out.err = a.err;
+    Stage st = stage_begin();
+    for (int64_t base = gw * 32; base < n; base += nw * 32) {
+        const int64_t v = base + lane;
+        u64 need = v < n ? active & ~a.visit[v] : 0, acc = 0;
+        int32_t b = 0, e = 0;
+        int cnt = 0;
+        if (need) {
+            b = a.g.crowptr[v];
+            e = a.g.crowptr[v + 1];
+            if (e - b < kMsPiece) {
+                const int32_t e1 = e - b > kMsThread ? b + kMsThread : e;
+                for (; b < e1 && (acc & need) != need; b += 4) {
+                    acc |= ms_gather(a, b, 1, e1);
+                    cnt += e1 - b < 4 ? e1 - b : 4;
+                }
+                if (acc & need) a.fnext[v] = acc & need;
+            } else {
+                b = e;
+            }
+        }
+        count_arcs(a.ctr, cnt);
+        const int32_t vs[1] = {(int32_t)v};
+        const int code[1] = {b < e && (acc & need) != need};
+        emit_n<1>(out, st, vs, code);
+    }
+    stage_end(out, st);
+}
+
+__global__ void __launch_bounds__(kCta) k_ms_pull_rest(MsPullArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const u64 active = *a.active;
+    const int32_t cnt = *a.rest_cnt;
+    for (int64_t i = gw; i < cnt; i += nw) {
+        const int32_t v = a.rest[i];
+        const u64 need = active & ~a.visit[v], have = a.fnext[v];
+        const int64_t e = a.g.crowptr[v + 1];
+        u64 got = have;
+        int64_t k = (int64_t)a.g.crowptr[v] + kMsThread;
+        for (; k < e && (got & need) != need; k += 128) {
+            const u64 m = ms_gather(a, k + lane, 32, e);
+            got |= (u64)__reduce_or_sync(G2_FULL, (unsigned)m) |
+                   (u64)__reduce_or_sync(G2_FULL, (unsigned)(m >> 32)) << 32;
+        }
+        if (lane == 0) {
+            got &= need;
+            if (got != have) a.fnext[v] = got;
+            if (a.ctr) atomicAdd(a.ctr, (u64)((k < e ? k : e) - a.g.crowptr[v] - kMsThread));
+        }
+    }
+}
+
+// Piece p belongs to the vertex big[i] with piece[i] <= p < piece[i + 1].
+__global__ void __launch_bounds__(kCta) k_ms_pull_pieces(MsPullArgs a, const int32_t *big,
+                                                         int32_t nbig, const int32_t *piece) {
+    __shared__ u64 s_m[kWarps];
+    const u64 active = *a.active;
+    const int32_t total = piece[nbig];
+    for (int32_t p = blockIdx.x; p < total; p += gridDim.x) {
+        const int32_t i = scan_owner(piece, nbig, p), v = big[i];
+        const u64 need = active & ~a.visit[v];
+        const int64_t b = (int64_t)a.g.crowptr[v] + (int64_t)(p - piece[i]) * kMsPiece;
+        const int64_t e1 = a.g.crowptr[v + 1], e = e1 - b < kMsPiece ? e1 : b + kMsPiece;
+        u64 m = 0;
+        if (need && (*(volatile u64 *)&a.fnext[v] & need) != need) {
+            for (int64_t k = b + threadIdx.x; k < e; k += 4 * kCta) m |= ms_gather(a, k, kCta, e);
+            if (a.ctr && threadIdx.x == 0) atomicAdd(a.ctr, (u64)(e - b));
+        }
+        m = (u64)__reduce_or_sync(G2_FULL, (unsigned)m) |
+            (u64)__reduce_or_sync(G2_FULL, (unsigned)(m >> 32)) << 32;
+        if ((threadIdx.x & 31) == 0) s_m[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int w = 1; w < kWarps; ++w) m |= s_m[w];
+            if (m & need) atomicOr(&a.fnext[v], m & need);
+        }
+        __syncthreads();
+    }
+}
+
+// The new masks of all vertices become visited, depths written, and the
+// vertices with one the new frontier.
+__global__ void __launch_bounds__(kCta) k_ms_commit_all(u64 *visit, const u64 *fnext, MsLevels l,
+                                                        int32_t level, u64 *active_next, int32_t *q,
+                                                        int32_t *qcnt, int32_t *err) {
+    const int lane = threadIdx.x & 31;
+    const int32_t n = l.n;
+    OutCtx out;
+    memset(&out, 0, sizeof(out));
+    out.mode = OUT_SPARSE;
+    out.q = q;
+    out.cnt = qcnt;
+    out.cap = n;
+    out.err = err;
+    Stage st = stage_begin();
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; base < n;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = base + lane;
+        const u64 nm = v < n ? fnext[v] : 0;
+        if (!__any_sync(G2_FULL, nm != 0)) continue;
+        if (nm) visit[v] |= nm;
+        ms_set_level(l, (int32_t)v, nm, level);
+        ms_note_active(active_next, nm);
+        const int32_t vs[1] = {(int32_t)v};
+        const int code[1] = {nm != 0};
+        emit_n<1>(out, st, vs, code);
+    }
+    stage_end(out, st);
+}
+
+// the vertices of at least `big` in-arcs, and their numbers of pieces
+__global__ void k_ms_big(const int32_t *crowptr, int32_t n, int32_t big, int32_t *list, int32_t *np,
+                         int32_t *cnt) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+         v += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t d = crowptr[v + 1] - crowptr[v];
+        if (d >= big) {
+            const int32_t i = atomicAdd(cnt, 1);
+            list[i] = (int32_t)v;
+            np[i] = (d + kMsPiece - 1) / kMsPiece;
+        }
+    }
+}
+
+// after a PUSH round: the new masks of the listed vertices (their number on
+// the device) become visited, their levels noted
+__global__ void k_ms_commit(const int32_t *touched, const int32_t *cnt_ptr, u64 *visit,
+                            const u64 *fnext, MsLevels l, int32_t level, u64 *active_next) {
+    const int lane = threadIdx.x & 31;
+    const int32_t cnt = *cnt_ptr;
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; base < cnt;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = base + lane;
+        int32_t v = 0;
+        u64 nm = 0;
+        if (i < cnt) {
+            v = touched[i];
+            nm = fnext[v];
+            visit[v] |= nm;
+        }
+        ms_set_level(l, v, nm, level);
+        ms_note_active(active_next, nm);
     }
 }
 
@@ -109,7 +315,7 @@ __global__ void k_ms_seed(const int32_t *srcs, int32_t k, u64 *visit, u64 *fcur,
         int32_t s = srcs[i];
         atomicOr(&visit[s], 1ull << i);
         u64 old = atomicOr(&fcur[s], 1ull << i);
-        depth[(int64_t)i * n + s] = 0;
+        if (depth) depth[(int64_t)i * n + s] = 0;
         if (old == 0) list[atomicAdd(cnt, 1)] = s;
     }
 }
@@ -123,13 +329,6 @@ __global__ void __launch_bounds__(kCta) k_ms_push(DevGraph g, FrontierIn fin, in
         case G2_LB_ETWC: lb_etwc(g, fin, fsize, op, out, blockIdx.x, gridDim.x, ctr); break;
         default: lb_vertex(g, fin, fsize, op, out, blockIdx.x, gridDim.x, ctr); break;
     }
-}
-
-template <class P, int G>
-__global__ void __launch_bounds__(kCta) k_ms_pull(DevGraph g, P op, OutCtx out,
-                                                  unsigned long long *ctr) {
-    Member all{MEM_ALL, nullptr, nullptr};
-    lb_pull<P, G>(g, nullptr, g.n, all, op, out, blockIdx.x, gridDim.x, ctr);
 }
 
 // ------------------------------------------- multi-source BFS, fused
@@ -261,48 +460,91 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
     G2_CK(cudaMemsetAsync(visit, 0, (size_t)n * 8, st));
     G2_CK(cudaMemsetAsync(F[0], 0, (size_t)n * 8, st));
     G2_CK(cudaMemsetAsync(F[1], 0, (size_t)n * 8, st));
-    G2_CK(cudaMemsetAsync(depth, 0xFF, (size_t)k * n * 4, st));
+    MsLevels lv;
+    u64 *planes;
+    G2_TRY(ws(g, B_ROWS, (size_t)kMsPlanes * std::max(n, 1), &planes));
+    for (int j = 0; j < kMsPlanes; ++j) lv.plane[j] = planes + (size_t)j * n;
+    lv.depth = nullptr;
+    lv.n = n;
+    int nplanes = 0;  // cleared so far
     G2_TRY(put_array(dsrc, srcs, k, st));
-    k_ms_seed<<<1, 64, 0, st>>>(dsrc, k, visit, F[0], depth, n, list[0], ctrs + 0);
-    stats().launches += 1;
-    G2_TRY(read_counters(g, ctrs, 4, st, d_err));
-    int32_t size = g->h_ctr[0];
+    // ctrs: [0..1] list lengths, [2] big vertices, [3] a pull's rest, [8..11] active masks of the
+    // even and odd levels (all zero at the start of the call)
+    u64 *active[2] = {reinterpret_cast<u64 *>(ctrs + 8), reinterpret_cast<u64 *>(ctrs + 10)};
+    k_ms_seed<<<1, 64, 0, st>>>(dsrc, k, visit, F[0], nullptr, n, list[0], ctrs + 0);
     const u64 full = k == 64 ? ~0ull : ((1ull << k) - 1);
+    G2_TRY(put_i32(st, {{ctrs + 8, (int32_t)(uint32_t)full}, {ctrs + 9, (int32_t)(uint32_t)(full >> 32)}}));
+    stats().launches += 1;
+    // PULL: the vertices whose lists go to the grid in pieces
+    int32_t *big = nullptr, *piece = nullptr, *rest = nullptr;
+    int32_t nbig = 0;
+    const bool pulls = h.s1.direction == G2_PULL ||
+                       (h.criteria == G2_INPUT_VERTEXSET_SIZE && h.s2.direction == G2_PULL);
+    if (pulls) {
+        int32_t *np;
+        const size_t room = (size_t)t->m / kMsPiece + 1;  // vertices of kMsPiece arcs or more
+        G2_TRY(ws(g, B_F0, room, &big));
+        G2_TRY(ws(g, B_F1, room, &np));
+        k_ms_big<<<grid_for(g, n, kCta), kCta, 0, st>>>(t->crowptr, n, kMsPiece, big, np, ctrs + 2);
+        stats().launches += 1;
+        G2_TRY(read_counters(g, ctrs, 4, st, d_err));
+        nbig = g->h_ctr[2];
+        G2_TRY(ws(g, B_F2, (size_t)std::max(n, 1), &rest));
+        if (nbig > 0) {
+            G2_TRY(ws(g, B_LVL, (size_t)nbig + 1, &piece));
+            G2_TRY(exclusive_scan_i32(g, np, piece, nbig, st));
+        }
+    } else {
+        G2_TRY(read_counters(g, ctrs, 4, st, d_err));
+    }
+    int32_t size = g->h_ctr[0];
     unsigned long long *ctr = nullptr;
     if (count_arcs_enabled()) G2_TRY(ws(g, B_ARCS, 2, &ctr));
-    const DevGraph dg = t->view();
     int p = 0;
     for (int level = 1; size > 0; ++level) {
         const g2_schedule &s = pick_schedule(h, size, n);
         G2_TRY(batch_lb(s));
         int q = 1 - p;
-        OutCtx out;
-        memset(&out, 0, sizeof(out));
-        out.mode = OUT_SPARSE;
-        out.q = list[q];
-        out.cnt = ctrs + q;
-        out.cap = n;
-        out.err = d_err;
+        u64 *act = active[(level - 1) & 1], *act_next = active[level & 1];
         G2_CK(cudaMemsetAsync(ctrs + q, 0, 4, st));
+        G2_CK(cudaMemsetAsync(act_next, 0, 8, st));
+        if (!lv.depth && level == 1 << nplanes) {
+            if (nplanes < kMsPlanes) {
+                G2_CK(cudaMemsetAsync(lv.plane[nplanes++], 0, (size_t)n * 8, st));
+            } else {
+                k_ms_out<<<grid_for(g, n, kCta), kCta, 0, st>>>(lv, visit, nplanes, k, depth);
+                stats().launches += 1;
+                lv.depth = depth;
+            }
+        }
         if (s.direction == G2_PUSH) {
+            OutCtx out;
+            memset(&out, 0, sizeof(out));
+            out.mode = OUT_SPARSE;
+            out.q = list[q];
+            out.cnt = ctrs + q;
+            out.cap = n;
+            out.err = d_err;
             VSet in{OUT_SPARSE, list[p], n, ctrs + p, nullptr, nullptr, size};
             G2_TRY(push_round(g, s, OpMsBfs{visit, F[p], F[q]}, in, out, ctr, st));
-            G2_TRY(read_counters(g, ctrs, 4, st, d_err));
-            int32_t nt = g->h_ctr[q];
-            if (nt > 0)
-                k_ms_commit<<<grid_for(g, nt, kCta), kCta, 0, st>>>(list[q], nt, visit, F[q], depth,
-                                                                   n, level);
+            k_ms_commit<<<t->sm_count * 8, kCta, 0, st>>>(list[q], ctrs + q, visit, F[q], lv, level,
+                                                        act_next);
             stats().push_rounds++;
             stats().launches += 2;
         } else {
-            PullMsBfs op{visit, F[p], F[q], depth, n, level, full};
-            if (s.load_balance == G2_LB_WM)
-                k_ms_pull<PullMsBfs, 32><<<grid_for(g, (int64_t)n * 32, kCta), kCta, 0, st>>>(
-                    dg, op, out, ctr);
-            else
-                k_ms_pull<PullMsBfs, 1><<<grid_for(g, n, kCta), kCta, 0, st>>>(dg, op, out, ctr);
+            // (the schedule's VERTEX_BASED and WM run the same kernel)
+            MsPullArgs a{t->view(), visit, F[p], F[q], act, rest, ctrs + 3, d_err, ctr};
+            G2_CK(cudaMemsetAsync(ctrs + 3, 0, 4, st));
+            if (nbig > 0)
+                k_ms_pull_pieces<<<grid_for(g, (int64_t)t->m / kMsPiece + nbig, 1), kCta, 0, st>>>(
+                    a, big, nbig, piece);
+            k_ms_pull<<<grid_for(g, n, kCta), kCta, 0, st>>>(a);
+            k_ms_pull_rest<<<t->sm_count * 16, kCta, 0, st>>>(a);
+            k_ms_commit_all<<<grid_for(g, n, kCta), kCta, 0, st>>>(visit, F[q], lv, level, act_next,
+                                                                 list[q], ctrs + q, d_err);
+            G2_CK(cudaGetLastError());
             stats().pull_rounds++;
-            stats().launches += 1;
+            stats().launches += nbig > 0 ? 4 : 3;
         }
         // the current frontier masks become the (all-zero) next-next array
         k_ms_clear<<<grid_for(g, size, kCta), kCta, 0, st>>>(list[p], size, F[p]);
@@ -311,6 +553,11 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
         size = g->h_ctr[q];
         p = q;
         stats().iterations++;
+    }
+    if (!lv.depth) {
+        k_ms_out<<<grid_for(g, n, kCta), kCta, 0, st>>>(lv, visit, nplanes, k, depth);
+        stats().launches += 1;
+        G2_CK(cudaGetLastError());
     }
     return G2_OK;
 }

@@ -88,7 +88,8 @@ class GraphPool:
                                              np.nonzero(G.degrees() > 0)[0].astype(np.int32))
 
     def footprint_bytes(self) -> int:
-        return sum(4 * (g.host.n + 1) + 8 * g.host.m for g in self.graphs.values())
+        # row offsets; arc heads, weights and (batched SSSP) tails
+        return sum(4 * (g.host.n + 1) + 12 * g.host.m for g in self.graphs.values())
 
 
 def make_trace(pool, rate: float, duration: float, mix=(0.6, 0.3, 0.1), seed: int = 1):
@@ -145,6 +146,10 @@ def batch_bytes(kind: str, k: int, n: int) -> int:
     """Device bytes a batch holds while it runs: outputs + workspace estimate."""
     out = {"bfs": 4 * k * n, "sssp": 4 * k * n, "bc": 8 * n}[kind]
     work = {"bfs": 40 * n, "sssp": 48 * n, "bc": 44 * n}[kind]
+    if k > 1 and kind == "bfs":     # the depths' bit planes
+        work += 40 * n
+    if k > 1 and kind == "sssp":    # the distance rows of 8, 16 or 32 sources
+        work += 4 * n * (8 if k <= 8 else 16 if k <= 16 else 32)
     return out + work
 
 
