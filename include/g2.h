@@ -286,8 +286,8 @@ g2_status g2_cc(g2_graph *g, int32_t *label, const g2_hybrid *sched, void *strea
  * WM, buckets run inside one thread-block cluster (near lists and far piles in
  * shared memory) while near rounds hold at most 1,024 vertices per cluster CTA,
  * and in the grid-wide kernel otherwise (back at a bucket boundary with a
- * small far pile), one launch per hand-over.  NULL schedule: STRICT PUSH,
- * unfused; fused WM PUSH on a bounded-degree graph (largest out-degree <= 32). */
+ * small far pile), one launch per hand-over.  NULL schedule: STRICT PUSH
+ * in one cooperative launch; fused WM PUSH on a bounded-degree graph (largest out-degree <= 32). */
 g2_status g2_sssp_delta(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
                         const g2_hybrid *sched, void *stream);
 

@@ -155,8 +155,28 @@ __device__ bool fused_strict_scan(const DevGraph &g, const int32_t *q, int32_t s
     return grid_sync(bar, err, limit_ns);
 }
 
+// CTAs per SM of the fused STRICT kernels (64 registers; a fifth gains BFS 3%
+// on RMAT-22 and costs RMAT-14 and delta-stepping 4-5%).
+constexpr int kFusedStrictCtas = 4;
+
+// One STRICT round of a fused loop (no barrier after it).  False: a barrier
+// wait gave up.
+template <class Op>
+__device__ __forceinline__ bool fused_strict(const DevGraph &g, const FrontierIn &fin, int32_t size,
+                                             const Op &op, const OutCtx &out, int32_t *scan,
+                                             int32_t *ctasum, const GridBarrier &bar, int32_t *err,
+                                             uint64_t limit_ns, unsigned long long *ctr) {
+    if (size <= kStrictSmall) {
+        lb_strict_small(g, fin, size, op, out, blockIdx.x, gridDim.x, ctr);
+        return true;
+    }
+    if (!fused_strict_scan(g, fin.q, size, scan, ctasum, bar, err, limit_ns)) return false;
+    lb_strict(g, fin, size, scan, op, out, blockIdx.x, gridDim.x, ctr);
+    return true;
+}
+
 template <int LB>
-__global__ void __launch_bounds__(kCta) k_bfs_fused_do(FusedDoBfsArgs a) {
+__global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 1) k_bfs_fused_do(FusedDoBfsArgs a) {
     OpBFS op{a.depth, a.parent};
     PullBFS pop{a.depth, a.parent};
     const int lane = threadIdx.x & 31;
@@ -228,10 +248,9 @@ __global__ void __launch_bounds__(kCta) k_bfs_fused_do(FusedDoBfsArgs a) {
                 }
             } else if (LB == G2_LB_STRICT) {
                 // the same number of arcs for every thread of the grid
-                if (!fused_strict_scan(a.g, a.q[d & 1], size, a.scan, a.ctasum, a.bar, a.err,
-                                       a.limit_ns))
+                if (!fused_strict(a.g, fin, size, op, out, a.scan, a.ctasum, a.bar, a.err, a.limit_ns,
+                                  a.ctr))
                     return;
-                lb_strict(a.g, fin, size, a.scan, op, out, blockIdx.x, gridDim.x, a.ctr);
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             } else {
                 run_lb<LB>(a.g, fin, size, op, out, a.ctr);
@@ -308,6 +327,8 @@ struct FusedSsspArgs {
     int32_t T0;        // threshold of the bucket at launch (clamped to G2_INF32)
     int32_t lo_far;    // after a near round, stop at a bucket boundary whose
                        // pile holds at most this many entries (0: never)
+    int32_t *scan;     // STRICT: prefix sums of a near list's degrees (n + 1) ...
+    int32_t *ctasum;   // ... and the slice totals of the CTAs (one per CTA)
     int32_t *result;   // [0] near rounds, [1] buckets, [2] 1 if stopped for the
                        // cluster loop, [3] threshold, [4] live pile, [5] epochs
     GridBarrier bar;
@@ -322,7 +343,7 @@ struct FusedSsspArgs {
 // smallest live far distance picks the next bucket and the far pile is split
 // (stale entries, already settled, are dropped).
 template <int LB>
-__global__ void __launch_bounds__(kCta) k_sssp_fused(FusedSsspArgs a) {
+__global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 1) k_sssp_fused(FusedSsspArgs a) {
     const int32_t n = a.g.n;
     int64_t T = a.T0;
     int d = 0, fp = 0, epoch = 0, buckets = 0, handover = 0;
@@ -348,7 +369,13 @@ __global__ void __launch_bounds__(kCta) k_sssp_fused(FusedSsspArgs a) {
             out.cnt2 = a.fcnt + fp;
             out.round2 = a.epoch0 + epoch;
             if (blockIdx.x == 0 && threadIdx.x == 0) a.ncnt[(d + 2) % 3] = 0;
-            run_lb<LB>(a.g, fin, size, op, out, a.ctr);
+            if (LB == G2_LB_STRICT) {
+                if (!fused_strict(a.g, fin, size, op, out, a.scan, a.ctasum, a.bar, a.err, a.limit_ns,
+                                  a.ctr))
+                    return;
+            } else {
+                run_lb<LB>(a.g, fin, size, op, out, a.ctr);
+            }
             if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             ++d;
             continue;
@@ -1072,9 +1099,11 @@ g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent
     return G2_OK;
 }
 
+// (STRICT is the tuned schedule on power-law graphs; the caller checks that a
+// schedule of its user's does not ask for it.)
 g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
                      const g2_schedule &s, cudaStream_t st, int32_t *d_err) {
-    G2_TRY(check_fused_lb(s));
+    if (s.load_balance != G2_LB_STRICT) G2_TRY(check_fused_lb(s));
     if (s.frontier_creation != G2_FUSED || s.dedup != G2_DEDUP_ENABLED)
         return fail(G2_EUNSUPPORTED, "the fused near/far queue uses FUSED lists with deduplication");
     Topology *t = g->topo;
@@ -1101,6 +1130,13 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     }
     a.round0 = g->round + 1;
     a.epoch0 = g->round2 + 1;
+    a.scan = nullptr;
+    a.ctasum = nullptr;
+    if (s.load_balance == G2_LB_STRICT) {
+        // one slice total per CTA: at most 2,048 threads, so 8 CTAs, per SM
+        G2_TRY(ws(g, B_SCAN, (size_t)n + 1, &a.scan));
+        G2_TRY(ws(g, B_SCANTMP, (size_t)t->sm_count * (2048 / kCta) + 1, &a.ctasum));
+    }
     a.ncnt = ctrs + 20;
     a.fcnt = ctrs + 23;
     a.dmin = ctrs + 25;
@@ -1186,6 +1222,11 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
                 case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st)); break;
                 case G2_LB_CM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_CM>, a, st)); break;
                 case G2_LB_ETWC: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_ETWC>, a, st)); break;
+                case G2_LB_STRICT:
+                    // rounds of millions of arcs: as many CTAs as fit
+                    G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_STRICT>, a, st,
+                                       env_i32("G2_FUSED_DO_CTAS_PER_SM", 4)));
+                    break;
                 default: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_VERTEX_BASED>, a, st)); break;
             }
             G2_TRY(read_counters(g, ctrs + 30, 6, st, d_err));

@@ -219,18 +219,33 @@ __device__ void lb_cta(const DevGraph &g, const FrontierIn &fin, int32_t fsize, 
 // fit (vertices without arcs in the list) searches the scan itself.
 constexpr int kStrictRun = 8;
 
+// The owners of a tile, in shared memory (one copy for both forms below: what
+// it takes comes out of L1).
+template <class Op>
+struct StrictOwners {
+    static constexpr int kTile = kCta * Op::kFlight;
+    static constexpr int kOwn = kTile + kCta;  // a tile of one-arc owners and the last one's
+    int32_t at[kOwn];    // first arc of the owner, from the tile's start
+    int32_t base[kOwn];  // arc k of the tile sits at base[owner] + k
+    int32_t u[kOwn];
+    typename Op::S s[kOwn];
+};
+template <class Op>
+__device__ __forceinline__ StrictOwners<Op> &strict_owners() {
+    __shared__ StrictOwners<Op> x;
+    return x;
+}
+
 template <class Op>
 __device__ void lb_strict(const DevGraph &g, const FrontierIn &fin, int32_t fsize,
                           const int32_t *scan, const Op &op, const OutCtx &out, int bid, int nb,
                           unsigned long long *ctr) {
     Stage st = stage_begin();
     constexpr int N = Op::kFlight;
-    constexpr int kTile = kCta * N;
-    constexpr int kOwn = kTile + kCta;  // a tile of one-arc owners and the last one's
-    __shared__ int32_t s_at[kOwn];    // first arc of the owner, from the tile's start
-    __shared__ int32_t s_base[kOwn];  // arc k of the tile sits at s_base[owner] + k
-    __shared__ int32_t s_u[kOwn];
-    __shared__ typename Op::S s_s[kOwn];
+    constexpr int kTile = StrictOwners<Op>::kTile, kOwn = StrictOwners<Op>::kOwn;
+    StrictOwners<Op> &own = strict_owners<Op>();
+    int32_t *s_at = own.at, *s_base = own.base, *s_u = own.u;
+    typename Op::S *s_s = own.s;
     const int tid = threadIdx.x;
     const int32_t total = scan[fsize];
     // (tile numbers fit: total < 2^31)
@@ -330,6 +345,85 @@ __device__ void lb_strict(const DevGraph &g, const FrontierIn &fin, int32_t fsiz
         __syncthreads();
     }
     stage_end(out, st);
+}
+
+// STRICT for a list of up to kStrictSmall entries in a fused loop, without a
+// scan of the whole grid before it: every CTA scans the list's degrees itself
+// (1 us, against two grid barriers and a pass over the list) and takes every
+// nb-th tile of its arcs.
+constexpr int kStrictSmall = 4 * kCta;
+
+template <class Op>
+__device__ void lb_strict_small(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
+                                const OutCtx &out, int bid, int nb, unsigned long long *ctr) {
+    typedef typename Op::S S;
+    constexpr int N = Op::kFlight, kTile = kCta * N, kPer = kStrictSmall / kCta;
+    Stage st = stage_begin();
+    static_assert(kStrictSmall <= StrictOwners<Op>::kOwn, "the list fits");
+    StrictOwners<Op> &own = strict_owners<Op>();
+    int32_t *s_at = own.at, *s_base = own.base, *s_u = own.u;
+    S *s_s = own.s;
+    __shared__ int s_warp[kWarps];
+    const int tid = threadIdx.x;
+    int32_t u[kPer], b[kPer], deg[kPer];
+    int sum = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int i = tid * kPer + j;
+        u[j] = i < fsize ? fin.vertex(i) : -1;
+    }
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        b[j] = deg[j] = 0;
+        if (u[j] >= 0) {
+            b[j] = g.rowptr[u[j]];
+            deg[j] = g.rowptr[u[j] + 1] - b[j];
+            s_s[tid * kPer + j] = op.load(u[j]);
+        }
+        sum += deg[j];
+    }
+    int total;
+    int at = block_incl_scan(sum, s_warp, &total) - sum;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int i = tid * kPer + j;
+        s_at[i] = at;
+        s_u[i] = u[j];
+        s_base[i] = b[j] - at;
+        at += deg[j];
+    }
+    __syncthreads();
+    int top = 1;
+    while (top < fsize) top <<= 1;
+    for (int64_t t0 = (int64_t)bid * kTile; t0 < total; t0 += (int64_t)nb * kTile) {
+        int lo[N];
+#pragma unroll
+        for (int j = 0; j < N; ++j) lo[j] = 0;
+        for (int d = top >> 1; d > 0; d >>= 1) {
+#pragma unroll
+            for (int j = 0; j < N; ++j) {
+                const int m = lo[j] + d;
+                if (m < fsize && s_at[m] <= t0 + j * kCta + tid) lo[j] = m;
+            }
+        }
+        int32_t us[N], e[N];
+        S ss[N];
+        bool on[N];
+        int cnt = 0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) {
+            const int64_t k = t0 + j * kCta + tid;
+            on[j] = k < total;
+            us[j] = s_u[lo[j]];
+            ss[j] = s_s[lo[j]];
+            e[j] = s_base[lo[j]] + (int32_t)k;
+            cnt += on[j];
+        }
+        apply_arcs<N>(op, out, st, us, ss, g.col, e, on);
+        count_arcs(ctr, cnt);
+    }
+    stage_end(out, st);
+    __syncthreads();  // the next call writes the arrays
 }
 
 // ---------------------------------------------------------------------- ETWC

@@ -165,16 +165,17 @@ class GpuExecutor:
         self.streams = [torch.cuda.Stream() for _ in range(slots)]
         self.views = [{name: g.handle.view() for name, g in pool.graphs.items()} for _ in range(slots)]
         self.fused = g2.schedule("WM", kernel_fusion=True)
-        # A single BFS on a power-law graph: with several slots, the tuned
-        # hybrid's schedules as per-level launches, whose small kernels
+        # A single BFS or SSSP on a power-law graph: with several slots, the
+        # tuned schedules as launches per level or round, whose small kernels
         # interleave with the other slots' work (the fused form's cooperative
         # launch needs every SM at once, so the slots' launches would run one
         # at a time); with one slot, the library's tuned schedule (NULL).
-        self.powerlaw_bfs = None
+        self.powerlaw_bfs = self.powerlaw_sssp = None
         if slots > 1:
             pull = g2.schedule("VERTEX_BASED", direction=g2.G2_PULL, pull_frontier=g2.G2_BITMAP,
                                frontier_creation=g2.G2_UNFUSED_BITMAP, dedup=False)
             self.powerlaw_bfs = g2.hybrid(g2.schedule("STRICT"), pull, 0.02)
+            self.powerlaw_sssp = g2.schedule("STRICT")
 
     def execute(self, slot: int, batch: list[Request]) -> dict:
         import torch
@@ -197,7 +198,8 @@ class GpuExecutor:
             elif r0.kind == "sssp":
                 out = torch.empty(k * n, dtype=torch.int32, device="cuda")
                 if k == 1:
-                    g2.g2_sssp_delta(view, int(srcs[0]), pg.spec.delta, out, single)
+                    g2.g2_sssp_delta(view, int(srcs[0]), pg.spec.delta, out,
+                                     single if pg.spec.road else self.powerlaw_sssp)
                 else:
                     g2.g2_sssp_batch(view, srcs, pg.spec.delta, out, None)
             else:
