@@ -59,6 +59,29 @@ __device__ __forceinline__ void cta_append(int32_t *q, int32_t *cnt, int32_t cap
     if (pred && pos < cap) q[pos] = v;
 }
 
+// N such appends with one shared atomic.
+template <int N>
+__device__ __forceinline__ void cta_append_n(int32_t *q, int32_t *cnt, int32_t cap,
+                                             const int32_t (&v)[N], const bool (&pred)[N], int lane) {
+    unsigned mask[N];
+    int total = 0;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        mask[j] = __ballot_sync(G2_FULL, pred[j]);
+        total += __popc(mask[j]);
+    }
+    if (total == 0) return;
+    int32_t base = 0;
+    if (lane == 0) base = atomicAdd(cnt, total);
+    base = __shfl_sync(G2_FULL, base, 0);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const int32_t pos = base + __popc(mask[j] & lanemask_lt());
+        if (pred[j] && pos < cap) q[pos] = v[j];
+        base += __popc(mask[j]);
+    }
+}
+
 // The cluster CTA that holds entry i of the concatenated list, where CTA r
 // holds entries [off[r], off[r + 1]) (off: the CL + 1 prefix sums of the
 // CTAs' list lengths).
@@ -84,10 +107,10 @@ static __global__ void k_level_list(const int32_t *depth, int32_t n, int32_t lvl
 }
 
 // ------------------------------------------------------------------ host
-// Whether one cluster of CL CTAs of `kernel` (kClCta threads, `smem` bytes
+// Whether one cluster of CL CTAs of `kernel` (`threads` each, `smem` bytes
 // of dynamic shared memory) fits on the current device.
 template <class K>
-inline bool cluster_fits(K kernel, int CL, size_t smem) {
+inline bool cluster_fits(K kernel, int CL, size_t smem, int threads) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -95,7 +118,7 @@ inline bool cluster_fits(K kernel, int CL, size_t smem) {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(CL);
-    cfg.blockDim = dim3(kClCta);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -116,7 +139,7 @@ inline bool cluster_fits(K kernel, int CL, size_t smem) {
 // none fits or G2_FUSED_CLUSTER=0 (read on every call; G2_FUSED_CLUSTER=8 or
 // 16 asks for that size).  k16 / k8 are the kernel's two instances.
 template <class K16, class K8>
-inline int cluster_size(int slot, K16 k16, K8 k8, size_t smem) {
+inline int cluster_size(int slot, K16 k16, K8 k8, size_t smem, int threads = kClCta) {
     const char *e = getenv("G2_FUSED_CLUSTER");
     const int want = e ? atoi(e) : -1;
     if (want == 0) return 0;
@@ -131,8 +154,8 @@ inline int cluster_size(int slot, K16 k16, K8 k8, size_t smem) {
     }
     std::lock_guard<std::mutex> lock(mu);
     int *f = fits[dev][slot];
-    if (f[0] == 0) f[0] = cluster_fits(k16, 16, smem) ? 1 : 2;
-    if (f[1] == 0) f[1] = cluster_fits(k8, 8, smem) ? 1 : 2;
+    if (f[0] == 0) f[0] = cluster_fits(k16, 16, smem, threads) ? 1 : 2;
+    if (f[1] == 0) f[1] = cluster_fits(k8, 8, smem, threads) ? 1 : 2;
     if (want != 8 && f[0] == 1) return 16;
     if (want != 16 && f[1] == 1) return 8;
     return 0;
@@ -146,7 +169,8 @@ inline int32_t env_i32(const char *name, int32_t dflt) {
 
 // One cluster of CL CTAs of `kernel` on `st`.
 template <class K, class A>
-inline g2_status launch_cluster(K kernel, int CL, size_t smem, const A &a, cudaStream_t st) {
+inline g2_status launch_cluster(K kernel, int CL, size_t smem, const A &a, cudaStream_t st,
+                                int threads = kClCta) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -154,7 +178,7 @@ inline g2_status launch_cluster(K kernel, int CL, size_t smem, const A &a, cudaS
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(CL);
-    cfg.blockDim = dim3(kClCta);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;

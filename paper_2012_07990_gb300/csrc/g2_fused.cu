@@ -460,6 +460,8 @@ __global__ void k_fill_dist(int32_t *a, int32_t n) {
 // its lanes (a warp-wide scan of the degrees and a shuffle search for each
 // arc's source), four arcs per lane in flight, so a level costs one chain of
 // dependent accesses: queue entry, row offsets, column ids, compare-and-swap.
+// One warp reads the CL lengths for its CTA (every warp for itself, without the
+// CTA barrier, was 15% slower: the reads of a peer's memory queue up).
 // Every CTA reads the same lengths and takes the same decisions, so all
 // threads pass the same sequence of cluster barriers.
 //
@@ -472,6 +474,11 @@ __global__ void k_fill_dist(int32_t *a, int32_t n) {
 // all labelled, so the host rebuilds that frontier from the depths.
 constexpr int kClQcap = 28672;    // queue entries per CTA and buffer (2 buffers: 224 KiB)
 constexpr int kClArcs = 4;        // arcs per lane in flight
+// Threads per CTA: a level of 1,400 vertices is one step of 44 warps, and a
+// barrier of 256 warps is cheaper than one of 512 (1024^2 grid 2.20 against 2.28
+// ms, 2000^2 5.45 against 5.59); the levels of larger grids fill 512 warps (4096^2
+// 18.3 against 17.4 ms).
+inline int bfs_cluster_threads(int32_t n) { return n > (1 << 22) ? kClCta : kClCta / 2; }
 
 struct ClusterBfsArgs {
     DevGraph g;
@@ -495,10 +502,7 @@ __global__ void __launch_bounds__(kClCta, 1) k_bfs_cluster(ClusterBfsArgs a) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int32_t *__restrict__ rowptr = a.g.rowptr;
     const int32_t *__restrict__ col = a.g.col;
-    if (threadIdx.x == 0) {
-        s_cnt[0] = 0;
-        s_cnt[1] = 0;
-    }
+    if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
     const int32_t *qg = (a.d0 & 1) ? a.q[1] : a.q[0];
     int32_t total = ld_relaxed_i32(a.cnt + a.d0 % 3);
     int reason = CL_DONE;
@@ -535,7 +539,7 @@ __global__ void __launch_bounds__(kClCta, 1) k_bfs_cluster(ClusterBfsArgs a) {
                 // hand the level to the grid loop: this CTA's part of the list
                 int32_t *dst = (cb ? a.q[1] : a.q[0]) + s_off[rank];
                 const int32_t mine = s_off[rank + 1] - s_off[rank];
-                for (int32_t j = threadIdx.x; j < mine; j += kClCta) dst[j] = s_q[cb * kClQcap + j];
+                for (int32_t j = threadIdx.x; j < mine; j += (int)blockDim.x) dst[j] = s_q[cb * kClQcap + j];
                 reason = CL_TO_GRID;
                 break;
             }
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__(kClCta, 1) k_bfs_cluster(ClusterBfsArgs a) {
         int32_t *nxt = s_q + nb * kClQcap;
         const int32_t lo = (int32_t)((int64_t)total * rank / CL);
         const int32_t hi = (int32_t)((int64_t)total * (rank + 1) / CL);
-        for (int32_t base = lo + warp * 32; base < hi; base += kClCta) {
+        for (int32_t base = lo + warp * 32; base < hi; base += (int)blockDim.x) {
             const int32_t i = base + lane;
             int32_t u = 0, beg = 0, deg = 0;
             if (i < hi) {
@@ -568,6 +572,7 @@ __global__ void __launch_bounds__(kClCta, 1) k_bfs_cluster(ClusterBfsArgs a) {
             arcs += (unsigned)tot;
             for (int32_t k0 = 0; k0 < tot; k0 += 32 * kClArcs) {
                 int32_t v[kClArcs], ou[kClArcs], dv[kClArcs];
+                bool disc[kClArcs];
 #pragma unroll
                 for (int j = 0; j < kClArcs; ++j) {
                     const int32_t k = k0 + 32 * j + lane;
@@ -588,12 +593,12 @@ __global__ void __launch_bounds__(kClCta, 1) k_bfs_cluster(ClusterBfsArgs a) {
                     dv[j] = v[j] >= 0 ? atomicCAS(a.depth + v[j], -1, d + 1) : 0;
 #pragma unroll
                 for (int j = 0; j < kClArcs; ++j) {
-                    const bool disc = v[j] >= 0 && dv[j] == -1;
+                    disc[j] = v[j] >= 0 && dv[j] == -1;
                     // the smallest source among this level's arcs into v
-                    if (a.parent && v[j] >= 0 && (disc || dv[j] == d + 1))
+                    if (a.parent && v[j] >= 0 && (disc[j] || dv[j] == d + 1))
                         atomicMin(reinterpret_cast<unsigned *>(a.parent + v[j]), (unsigned)ou[j]);
-                    cta_append(nxt, &s_cnt[nb], kClQcap, v[j], disc, lane);
                 }
+                cta_append_n<kClArcs>(nxt, &s_cnt[nb], kClQcap, v, disc, lane);
             }
         }
         cl_barrier();  // level d complete: queues nb filled, queues cb no longer read
@@ -809,16 +814,18 @@ __global__ void __launch_bounds__(kClCta, 1) k_sssp_cluster(ClusterSsspArgs a) {
 #pragma unroll
                     for (int j = 0; j < kClArcs; ++j)
                         old[j] = v[j] >= 0 ? atomicMin(a.dist + v[j], nv[j]) : 0;
+                    bool to_near[kClArcs], to_far[kClArcs];
 #pragma unroll
                     for (int j = 0; j < kClArcs; ++j) {
                         const bool better = v[j] >= 0 && nv[j] < old[j];
-                        bool to_near = better && nv[j] < T;
-                        bool to_far = better && nv[j] >= T;
-                        if (to_near && a.dedup_near) to_near = atomicExch(a.stamp + v[j], rid) != rid;
-                        if (to_far) to_far = atomicExch(a.stamp2 + v[j], eid) != eid;
-                        cta_append(nxt, &s_ncnt[nb], kCsQn, v[j], to_near, lane);
-                        cta_append(far, &s_fcnt[fp], kCsQf, v[j], to_far, lane);
+                        to_near[j] = better && nv[j] < T;
+                        to_far[j] = better && nv[j] >= T;
+                        if (to_near[j] && a.dedup_near)
+                            to_near[j] = atomicExch(a.stamp + v[j], rid) != rid;
+                        if (to_far[j]) to_far[j] = atomicExch(a.stamp2 + v[j], eid) != eid;
                     }
+                    cta_append_n<kClArcs>(nxt, &s_ncnt[nb], kCsQn, v, to_near, lane);
+                    cta_append_n<kClArcs>(far, &s_fcnt[fp], kCsQf, v, to_far, lane);
                 }
             }
             first = false;
@@ -983,8 +990,10 @@ g2_status bfs_fused(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
     for (;;) {
         if (in_cluster) {
             c.d0 = level;
-            if (cl == 16) G2_TRY(launch_cluster(k_bfs_cluster<16>, 16, 2 * (size_t)kClQcap * 4, c, st));
-            else G2_TRY(launch_cluster(k_bfs_cluster<8>, 8, 2 * (size_t)kClQcap * 4, c, st));
+            if (cl == 16) G2_TRY(launch_cluster(k_bfs_cluster<16>, 16, 2 * (size_t)kClQcap * 4, c, st,
+                                            bfs_cluster_threads(n)));
+            else G2_TRY(launch_cluster(k_bfs_cluster<8>, 8, 2 * (size_t)kClQcap * 4, c, st,
+                                         bfs_cluster_threads(n)));
             G2_TRY(read_counters(g, ctrs + 32, 2, st, d_err));
             const int32_t reached = g->h_ctr[0], why = g->h_ctr[1];
             if (reached <= level) return fail(G2_ECUDA, "cluster BFS made no progress");
@@ -1164,9 +1173,14 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     c.delta = delta;
     c.stamp = a.stamp;
     c.stamp2 = a.stamp2;
-    c.hi = env_i32("G2_CLUSTER_HI", 1024 * cl);
     int32_t dmax = 0;
     if (cl) G2_TRY(max_out_degree(g, st, &dmax));
+    // Measured on road grids with the grid-wide loop at two CTAs per SM: hand a
+    // near round of more than 8,192 vertices to the grid (4096^2, delta 16384:
+    // 35.6 ms against 36.5 with 16,384; 1024^2: no difference down to 4,096).
+    // Graphs that fit one round of the cluster stay in it.
+    const int32_t hi = dmax <= kBoundedDegree && n > 1024 * cl ? 512 * cl : 1024 * cl;
+    c.hi = env_i32("G2_CLUSTER_HI", hi);
     c.dedup_near = !(t->symmetric && dmax <= kBoundedDegree);
     c.nq_out = a.nq[0];
     c.fq_out = a.fq[0];
@@ -1176,7 +1190,7 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     c.result = ctrs + 36;
     c.err = d_err;
     c.ctr = a.ctr;
-    a.lo_far = cl ? std::min(std::min(env_i32("G2_CLUSTER_FAR_LO", 1024 * cl), c.hi),
+    a.lo_far = cl ? std::min(std::min(env_i32("G2_CLUSTER_FAR_LO", hi), c.hi),
                              (int32_t)(kCsQf / 2 * cl))
                   : 0;
     int32_t T = (int32_t)std::min<int64_t>(delta, G2_INF32);
@@ -1218,8 +1232,12 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
             a.T0 = T;
             a.round0 = round0;
             a.epoch0 = epoch0;
+            // two CTAs per SM: the shares of a round of 10,000 vertices are one
+            // step of a warp each (4096^2, delta 16384: 38.0 ms with one, 35.6
+            // with two)
+            const int ctas = env_i32("G2_FUSED_CTAS_PER_SM", 2);
             switch (s.load_balance) {
-                case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st)); break;
+                case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st, ctas)); break;
                 case G2_LB_CM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_CM>, a, st)); break;
                 case G2_LB_ETWC: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_ETWC>, a, st)); break;
                 case G2_LB_STRICT:

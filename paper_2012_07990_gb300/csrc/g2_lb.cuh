@@ -91,7 +91,8 @@ __device__ void lb_vertex(const DevGraph &g, const FrontierIn &fin, int32_t fsiz
 }
 
 // ------------------------------------------------------------------------ WM
-// A warp takes 32 active vertices, prefix-sums their degrees with shuffles and
+// A warp takes up to 32 active vertices (fewer where the list is short: an
+// equal share for every warp), prefix-sums their degrees with shuffles and
 // walks the combined arc range 32 arcs at a time, kFlight such steps in
 // flight; each lane finds the owner of its arc by a 5-step binary search over
 // the lanes' prefix sums.
@@ -103,11 +104,12 @@ __device__ void lb_warp(const DevGraph &g, const FrontierIn &fin, int32_t fsize,
     const int lane = threadIdx.x & 31;
     const int gw = bid * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int nw = nb * (blockDim.x >> 5);
-    for (int64_t base = (int64_t)gw * 32; base < fsize; base += (int64_t)nw * 32) {
+    const int per = fsize < nw * 32 ? (fsize + nw - 1) / nw : 32;
+    for (int64_t base = (int64_t)gw * per; base < fsize; base += (int64_t)nw * per) {
         int32_t i = (int32_t)base + lane;
         int32_t u = 0, beg = 0, len = 0;
         typename Op::S s{};
-        if (i < fsize) {
+        if (lane < per && i < fsize) {
             u = fin.vertex(i);
             s = op.load(u);
             if (!op.skip(s)) {
