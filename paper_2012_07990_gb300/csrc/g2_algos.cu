@@ -78,7 +78,28 @@ __device__ __forceinline__ void cc_link(int32_t *label, int32_t u, int32_t v) {
     }
 }
 
-// link every vertex with its r-th neighbour
+// First labels and first sampling round in one: every vertex hangs under its
+// smallest neighbour where that is smaller than itself (the first of its
+// ascending list), which makes a forest of falling ids without a link.  (Where
+// the smallest neighbour is larger, the next round links that arc too.)
+__global__ void k_cc_first(const int32_t *rowptr, const int32_t *col, int32_t n, int32_t *label,
+                           unsigned long long *ctr) {
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = base + threadIdx.x;
+        bool linked = false;
+        if (v < n) {
+            const int32_t b = rowptr[v];
+            linked = rowptr[v + 1] > b;
+            const int32_t u = linked ? col[b] : (int32_t)v;
+            label[v] = u < (int32_t)v ? u : (int32_t)v;
+        }
+        count_arcs(ctr, linked);
+    }
+}
+
+// link every vertex with its r-th neighbour (r = 1: and with its first, where
+// k_cc_first did not)
 __global__ void k_cc_sample(const int32_t *rowptr, const int32_t *col, int32_t n, int32_t r,
                             int32_t *label, unsigned long long *ctr) {
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
@@ -86,8 +107,9 @@ __global__ void k_cc_sample(const int32_t *rowptr, const int32_t *col, int32_t n
         const int64_t v = base + threadIdx.x;
         bool linked = false;
         if (v < n) {
-            int32_t b = rowptr[v];
-            if (rowptr[v + 1] - b > r) {
+            const int32_t b = rowptr[v], deg = rowptr[v + 1] - b;
+            if (r == 1 && deg > 0 && col[b] > (int32_t)v) cc_link(label, (int32_t)v, col[b]);
+            if (deg > r) {
                 cc_link(label, (int32_t)v, col[b + r]);
                 linked = true;
             }
@@ -96,22 +118,55 @@ __global__ void k_cc_sample(const int32_t *rowptr, const int32_t *col, int32_t n
     }
 }
 
-// labels of a fixed pseudo-random sample of vertices
-__global__ void k_cc_probe(const int32_t *label, int32_t n, int32_t k, int32_t *out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < k) {
-        uint32_t h = (uint32_t)i * 2654435761u + 0x9E3779B9u;
-        h ^= h >> 16;
-        h *= 0x85EBCA6Bu;
-        h ^= h >> 13;
-        out[i] = label[h % (uint32_t)n];
+// The most frequent label (the smallest of those) of a fixed pseudo-random
+// sample of kCcProbe vertices to *giant: one CTA sorts the sample in shared
+// memory (it went to the host and back before: a read-back and a sort, 35 us of
+// RMAT-22's 186).
+constexpr int kCcProbe = 1024;
+__global__ void __launch_bounds__(kCcProbe) k_cc_probe(const int32_t *label, int32_t n,
+                                                       int32_t *giant) {
+    __shared__ int32_t s[kCcProbe];
+    __shared__ unsigned long long s_best;
+    const int i = threadIdx.x;
+    uint32_t h = (uint32_t)i * 2654435761u + 0x9E3779B9u;
+    h ^= h >> 16;
+    h *= 0x85EBCA6Bu;
+    h ^= h >> 13;
+    s[i] = label[h % (uint32_t)n];
+    if (i == 0) s_best = 0;
+    __syncthreads();
+    for (int k = 2; k <= kCcProbe; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            const int o = i ^ j;
+            if (o > i) {
+                const int32_t x = s[i], y = s[o];
+                if ((x > y) == ((i & k) == 0)) {
+                    s[i] = y;
+                    s[o] = x;
+                }
+            }
+            __syncthreads();
+        }
+    // the first of each run finds its end
+    if (i == 0 || s[i] != s[i - 1]) {
+        int lo = i, hi = kCcProbe;  // s[lo] == s[i], s[hi] > s[i]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) / 2;
+            if (s[mid] == s[i]) lo = mid;
+            else hi = mid;
+        }
+        // longest run, then smallest label
+        atomicMax(&s_best, (unsigned long long)(hi - i) << 32 | (unsigned)(G2_INF32 - s[i]));
     }
+    __syncthreads();
+    if (i == 0) *giant = G2_INF32 - (int32_t)(unsigned)s_best;
 }
 
 // link the remaining arcs (from position `skip` on) of every vertex outside
-// the component `giant`; a warp walks one vertex so long lists are shared
+// the component *giant_p; a warp walks one vertex so long lists are shared
 __global__ void k_cc_finish(const int32_t *rowptr, const int32_t *col, int32_t n, int32_t skip,
-                            int32_t giant, int32_t *label, unsigned long long *ctr) {
+                            const int32_t *giant_p, int32_t *label, unsigned long long *ctr) {
+    const int32_t giant = *giant_p;
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -379,39 +434,23 @@ g2_status cc_sampled(g2_graph *g, int32_t *label, cudaStream_t st, int32_t *d_er
     Topology *t = g->topo;
     const int32_t n = t->n;
     if (n == 0) return G2_OK;
-    constexpr int kSample = 2, kProbe = 1024;
+    constexpr int kSample = 2;
     const int grid = grid_for(g, n, kCta);
     // arcs linked (stats mode): one per vertex and sampling round, then the
     // remaining arcs of the vertices outside the giant component
     unsigned long long *ctr = nullptr;
     if (count_arcs_enabled()) G2_TRY(ws(g, B_ARCS, 2, &ctr));
-    k_iota<<<grid, kCta, 0, st>>>(label, n);
-    for (int r = 0; r < kSample; ++r) {
-        k_cc_sample<<<grid, kCta, 0, st>>>(t->rowptr, t->col, n, r, label, ctr);
+    int32_t *giant = d_err - 62 + 20;
+    k_cc_first<<<grid, kCta, 0, st>>>(t->rowptr, t->col, n, label, ctr);
+    for (int r = 1; r < kSample; ++r) {
         k_compress<<<grid, kCta, 0, st>>>(label, n);
+        k_cc_sample<<<grid, kCta, 0, st>>>(t->rowptr, t->col, n, r, label, ctr);
     }
-    int32_t *probe;
-    G2_TRY(ws(g, B_I1, kProbe, &probe));
-    k_cc_probe<<<(kProbe + kCta - 1) / kCta, kCta, 0, st>>>(label, n, kProbe, probe);
-    std::vector<int32_t> h(kProbe);
-    G2_CK(cudaMemcpyAsync(h.data(), probe, kProbe * 4, cudaMemcpyDeviceToHost, st));
-    G2_TRY(sync_and_check(g, st, d_err));
-    std::sort(h.begin(), h.end());
-    int32_t giant = h[0];
-    int best = 0;
-    for (int i = 0; i < kProbe;) {
-        int j = i;
-        while (j < kProbe && h[j] == h[i]) ++j;
-        if (j - i > best) {
-            best = j - i;
-            giant = h[i];
-        }
-        i = j;
-    }
-    k_cc_finish<<<grid_for(g, n, kCta), kCta, 0, st>>>(t->rowptr, t->col, n, kSample, giant, label,
-                                                        ctr);
     k_compress<<<grid, kCta, 0, st>>>(label, n);
-    stats().launches += 2 * kSample + 5;
+    k_cc_probe<<<1, kCcProbe, 0, st>>>(label, n, giant);
+    k_cc_finish<<<grid, kCta, 0, st>>>(t->rowptr, t->col, n, kSample, giant, label, ctr);
+    k_compress<<<grid, kCta, 0, st>>>(label, n);
+    stats().launches += 2 * kSample + 3;
     stats().iterations = kSample + 1;
     G2_CK(cudaGetLastError());
     return G2_OK;
