@@ -642,6 +642,7 @@ g2_status g2_bfs(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent, cons
     } else {
         G2_TRY(bfs_plain(g, src, depth, parent, h, st, d_err));
     }
+    g->settled = true;  // each of them ends by reading its counters
     return end_call(g, st, d_err);
 }
 
@@ -678,6 +679,7 @@ g2_status g2_sssp_delta(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     } else {
         G2_TRY(sssp_plain(g, src, delta, dist, h, st, d_err));
     }
+    g->settled = true;  // both end by reading their counters
     return end_call(g, st, d_err);
 }
 

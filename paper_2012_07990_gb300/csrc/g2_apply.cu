@@ -266,7 +266,12 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         if (s.frontier_creation == G2_FUSED) {
             bool dedup = s.dedup == G2_DEDUP_ENABLED;
             size_t cap = dedup ? (size_t)std::max(n, 1) : (size_t)t->m + (size_t)n + 1;
-            G2_TRY(ws(g, dedup ? B_Q3 : B_BIG, cap, &o.q));
+            // straight into the caller's list where it is not the input's and
+            // has room for every vertex
+            if (dedup && outf->format == G2_FRONTIER_SPARSE && outf != in && outf->cap >= (int32_t)cap)
+                o.q = outf->q;
+            else
+                G2_TRY(ws(g, dedup ? B_Q3 : B_BIG, cap, &o.q));
             o.rep = OUT_SPARSE;
             o.qcap = (int32_t)std::min<size_t>(cap, 2147483647u);
             o.cnt = ctrs + 61;
@@ -312,6 +317,7 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         stats().launches += 1;
         a.from = snap;
     }
+    if (outf) outf->size = 0;  // until the call has succeeded
     G2_TRY(apply_round(g, s, a, use, o, st));
     s.direction == G2_PUSH ? stats().push_rounds++ : stats().pull_rounds++;
     stats().iterations = 1;
@@ -320,17 +326,19 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
     if (outf) {
         // produced -> caller's representation
         if (produced.rep == OUT_SPARSE) {
-            G2_CK(cudaMemcpyAsync(g->h_ctr, o.cnt, 4, cudaMemcpyDeviceToHost, st));
-            G2_TRY(sync_and_check(g, st, d_err));
-            size = g->h_ctr[0];
+            if (outf->format == G2_FRONTIER_SPARSE)
+                G2_CK(cudaMemcpyAsync(outf->cnt, o.cnt, 4, cudaMemcpyDeviceToDevice, st));
+            G2_TRY(read_counters(g, o.cnt, 1, st, d_err));
         } else {
             G2_TRY(vset_count(g, produced, ctrs + 59, st));
-            G2_CK(cudaMemcpyAsync(g->h_ctr, ctrs + 59, 4, cudaMemcpyDeviceToHost, st));
-            G2_TRY(sync_and_check(g, st, d_err));
-            size = g->h_ctr[0];
+            G2_TRY(read_counters(g, ctrs + 59, 1, st, d_err));
         }
+        size = g->h_ctr[0];
         produced.size = size;
-        if (outf->format == G2_FRONTIER_SPARSE) {
+        outf->size = outf->format == G2_FRONTIER_SPARSE ? size : -1;
+        if (outf->format == G2_FRONTIER_SPARSE && o.rep == OUT_SPARSE && o.q == outf->q) {
+            g->settled = true;
+        } else if (outf->format == G2_FRONTIER_SPARSE) {
             if (size > outf->cap) {
                 dfree(outf->q, st);
                 outf->q = nullptr;
@@ -345,10 +353,8 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
                 VSet d{OUT_SPARSE, outf->q, outf->cap, outf->cnt, nullptr, nullptr, 0};
                 G2_TRY(vset_convert(g, produced, OUT_SPARSE, d, st));
             }
-            G2_CK(cudaMemcpyAsync(outf->cnt, o.rep == OUT_SPARSE ? o.cnt : &size, 4,
-                                  o.rep == OUT_SPARSE ? cudaMemcpyDeviceToDevice
-                                                      : cudaMemcpyHostToDevice,
-                                  st));
+            if (o.rep != OUT_SPARSE)
+                G2_CK(cudaMemcpyAsync(outf->cnt, &size, 4, cudaMemcpyHostToDevice, st));
         } else {
             int want = outf->format == G2_FRONTIER_BITMAP ? OUT_BITMAP : OUT_BOOLMAP;
             VSet d{want, nullptr, 0, nullptr, outf->bitmap, outf->boolmap, 0};

@@ -479,14 +479,9 @@ g2_status ws_get(g2_graph *g, Buf b, size_t bytes, void **out) {
     return G2_OK;
 }
 
-g2_status sync_and_check(g2_graph *g, cudaStream_t st, int32_t *d_err) {
-    G2_CK(cudaGetLastError());
-    if (d_err) {
-        G2_CK(cudaMemcpyAsync(g->h_ctr + 63, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-    }
-    G2_CK(cudaStreamSynchronize(st));
-    if (d_err && g->h_ctr[63] != 0) {
-        int code = g->h_ctr[63];
+// the status of a device error word
+static g2_status device_status(int32_t code) {
+    if (code != 0) {
         const char *what = code == G2_ETIMEOUT ? "device-side wait timed out"
                            : code == G2_EOVERFLOW ? "queue or value overflow on the device"
                                                   : "device error";
@@ -495,9 +490,19 @@ g2_status sync_and_check(g2_graph *g, cudaStream_t st, int32_t *d_err) {
     return G2_OK;
 }
 
+g2_status sync_and_check(g2_graph *g, cudaStream_t st, int32_t *d_err) {
+    G2_CK(cudaGetLastError());
+    if (d_err) {
+        G2_CK(cudaMemcpyAsync(g->h_ctr + 63, d_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    }
+    G2_CK(cudaStreamSynchronize(st));
+    return d_err ? device_status(g->h_ctr[63]) : G2_OK;
+}
+
 g2_status begin_call(g2_graph *g, cudaStream_t st, int32_t **d_err) {
     stats() = g2_stats{};
     g->st = st;
+    g->settled = false;
     int32_t *ctrs;
     G2_TRY(ws(g, B_CTR, 64, &ctrs));
     G2_CK(cudaMemsetAsync(ctrs, 0, 64 * sizeof(int32_t), st));
@@ -511,7 +516,8 @@ g2_status begin_call(g2_graph *g, cudaStream_t st, int32_t **d_err) {
 }
 
 g2_status end_call(g2_graph *g, cudaStream_t st, int32_t *d_err) {
-    G2_TRY(sync_and_check(g, st, d_err));
+    if (!g->settled) G2_TRY(sync_and_check(g, st, d_err));
+    g->settled = false;
     ktime_resolve();
     if (count_arcs_enabled()) {
         unsigned long long *a;
@@ -524,6 +530,16 @@ g2_status end_call(g2_graph *g, cudaStream_t st, int32_t *d_err) {
 }
 
 g2_status read_counters(g2_graph *g, const int32_t *d, int count, cudaStream_t st, int32_t *d_err) {
+    const int32_t *ctrs = d_err ? d_err - 62 : nullptr;
+    if (ctrs && d >= ctrs && d + count <= d_err) {
+        const int off = (int)(d - ctrs);
+        G2_CK(cudaGetLastError());
+        G2_CK(cudaMemcpyAsync(g->h_ctr + 64 + off, d, (size_t)(63 - off) * sizeof(int32_t),
+                              cudaMemcpyDeviceToHost, st));
+        G2_CK(cudaStreamSynchronize(st));
+        memcpy(g->h_ctr, g->h_ctr + 64 + off, (size_t)count * sizeof(int32_t));
+        return device_status(g->h_ctr[64 + 62]);
+    }
     G2_CK(cudaMemcpyAsync(g->h_ctr, d, (size_t)count * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     return sync_and_check(g, st, d_err);
 }
@@ -783,13 +799,13 @@ static g2_status finish_handle(g2_graph *g) {
         }
     }
     if (!g->h_ctr) {
-        cudaError_t e = cudaMallocHost(&g->h_ctr, 64 * sizeof(int32_t));
+        cudaError_t e = cudaMallocHost(&g->h_ctr, 128 * sizeof(int32_t));
         if (e != cudaSuccess) {
             g->h_ctr = nullptr;
             return cuda_fail(e, "cudaMallocHost counters");
         }
     }
-    memset(g->h_ctr, 0, 64 * sizeof(int32_t));
+    memset(g->h_ctr, 0, 128 * sizeof(int32_t));
     return G2_OK;
 }
 
@@ -1207,6 +1223,7 @@ g2_status g2_frontier_set(g2_frontier *f, const int32_t *verts, int32_t k, void 
         if (verts[i] < 0 || verts[i] >= n) return fail(G2_EINVAL, "vertex id out of range");
     cudaStream_t st = as_stream(stream);
     g->st = st;
+    f->size = 0;  // until the call has succeeded
     int32_t *tmp;
     G2_TRY(ws(g, B_I1, (size_t)std::max(k, 1), &tmp));
     if (k > 0) G2_CK(cudaMemcpyAsync(tmp, verts, (size_t)k * 4, cudaMemcpyHostToDevice, st));
@@ -1225,7 +1242,9 @@ g2_status g2_frontier_set(g2_frontier *f, const int32_t *verts, int32_t k, void 
                  nullptr, f->bitmap, f->boolmap, 0};
         G2_TRY(vset_convert(g, src, dst.rep, dst, st));
     }
-    return sync_and_check(g, st, nullptr);
+    G2_TRY(sync_and_check(g, st, nullptr));
+    f->size = f->format == G2_FRONTIER_SPARSE ? k : -1;
+    return G2_OK;
 }
 
 g2_status g2_frontier_size(g2_frontier *f, int32_t *size, void *stream) {
@@ -1233,6 +1252,10 @@ g2_status g2_frontier_size(g2_frontier *f, int32_t *size, void *stream) {
     g2_graph *g = f->g;
     cudaStream_t st = as_stream(stream);
     g->st = st;
+    if (f->size >= 0) {  // the last call on the frontier ended with this many
+        *size = f->size;
+        return G2_OK;
+    }
     if (f->format == G2_FRONTIER_SPARSE) {
         G2_CK(cudaMemcpyAsync(g->h_ctr, f->cnt, 4, cudaMemcpyDeviceToHost, st));
     } else {
@@ -1244,7 +1267,7 @@ g2_status g2_frontier_size(g2_frontier *f, int32_t *size, void *stream) {
         G2_CK(cudaMemcpyAsync(g->h_ctr, d + 32, 4, cudaMemcpyDeviceToHost, st));
     }
     G2_CK(cudaStreamSynchronize(st));
-    *size = g->h_ctr[0];
+    *size = f->size = g->h_ctr[0];
     return G2_OK;
 }
 

@@ -68,10 +68,11 @@ struct g2_graph {
     g2::Topology *topo;
     void *buf[g2::B_COUNT];
     size_t cap[g2::B_COUNT];
-    int32_t *h_ctr;   // pinned host mirror of B_CTR
+    int32_t *h_ctr;   // pinned: values read back ([0, 64)), mirror of B_CTR ([64, 128))
     int32_t round;    // monotonic-counter stamp (advances every apply round)
     int32_t round2;
     cudaStream_t st;  // stream of the call in progress (set at every entry)
+    bool settled;     // nothing was queued after the last read_counters of the call
 };
 
 struct g2_frontier {
@@ -82,6 +83,7 @@ struct g2_frontier {
     int32_t *cnt;     // device int32 length (SPARSE)
     uint32_t *bitmap; // BITMAP
     uint8_t *boolmap; // BOOLMAP
+    int32_t size;     // members as the host knows them (-1: to be counted on the device)
 };
 
 namespace g2 {
@@ -203,10 +205,11 @@ void ktime_end(KTime &k, cudaStream_t st);
 // Start of a public call: reset the thread's stats, zero the device error
 // word (returned in *d_err, B_CTR slot 62) and the arc counter.
 g2_status begin_call(g2_graph *g, cudaStream_t st, int32_t **d_err);
-// End of a public call: synchronise, report device errors, collect counters.
+// End of a public call: synchronise and report device errors (unless the call
+// said with g->settled that its last read_counters did both), collect counters.
 g2_status end_call(g2_graph *g, cudaStream_t st, int32_t *d_err);
 // Read `count` device int32 counters into g->h_ctr (synchronises) and check
-// the error word.
+// the error word: one copy where the counters lie before it in B_CTR.
 g2_status read_counters(g2_graph *g, const int32_t *d, int count, cudaStream_t st, int32_t *d_err);
 
 // Small host values stored to device memory by a one-warp kernel that takes
