@@ -32,9 +32,11 @@ namespace g2 {
 // Items 0..count-1 with keys vals[i] / div in [0, nkeys) get positions such
 // that the items of key k occupy [start_k, start_k + size_k) in index order,
 // and start_k = the sum over j < k of size_j rounded up to a multiple of pad.
-// A warp owns a tile of kPartTile consecutive items and walks it 32 at a
-// time; counts live in the warp's slice of shared memory (nkeys ints).
+// A warp owns a tile of consecutive items (kPartTile of the arcs, kPartTileV of
+// the vertices) and walks it 32 at a time; counts live in the warp's slice of shared memory (nkeys ints).
 constexpr int kPartTile = 2048;
+constexpr int kPartTileV = 512;  // of the vertices' partition: a warp each for 0.2M vertices already
+                                 // (700K vertices: 342 tiles of 2,048 kept 342 warps busy for 83 us)
 constexpr int kPartMaxKeys = 1024;
 constexpr int kPartCta = 256;
 
@@ -49,7 +51,8 @@ __device__ __forceinline__ int32_t div_floor(int32_t x, int32_t d, float inv) {
 
 __global__ void __launch_bounds__(kPartCta) k_part_count(const int32_t *vals, int32_t div,
                                                          int64_t count, int32_t nkeys,
-                                                         int32_t ntiles, int32_t *counts) {
+                                                         int32_t ntiles, int32_t per,
+                                                         int32_t *counts) {
     extern __shared__ int32_t s_part[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int32_t *c = s_part + wid * nkeys;
@@ -57,12 +60,23 @@ __global__ void __launch_bounds__(kPartCta) k_part_count(const int32_t *vals, in
     for (int32_t tile = blockIdx.x * wpc + wid; tile < ntiles; tile += gridDim.x * wpc) {
         for (int k = lane; k < nkeys; k += 32) c[k] = 0;
         __syncwarp();
-        const int64_t base = (int64_t)tile * kPartTile;
+        const int64_t base = (int64_t)tile * per;
         const float inv = 1.0f / (float)div;
-#pragma unroll 8
-        for (int s = 0; s < kPartTile / 32; ++s) {
-            const int64_t i = base + s * 32 + lane;
-            if (i < count) atomicAdd(&c[div_floor(vals[i], div, inv)], 1);
+        // one atomic per key of a step (a third of a power-law graph's vertices
+        // have the key of no arcs), eight steps side by side
+        constexpr int kB = 8;
+        for (int s0 = 0; s0 < per / 32; s0 += kB) {
+            int key[kB];
+#pragma unroll
+            for (int j = 0; j < kB; ++j) {
+                const int64_t i = base + (s0 + j) * 32 + lane;
+                key[j] = i < count ? div_floor(vals[i], div, inv) : -1;
+            }
+#pragma unroll
+            for (int j = 0; j < kB; ++j) {
+                const unsigned peers = __match_any_sync(G2_FULL, key[j]);
+                if (key[j] >= 0 && lane == __ffs(peers) - 1) atomicAdd(&c[key[j]], __popc(peers));
+            }
         }
         __syncwarp();
         for (int k = lane; k < nkeys; k += 32) counts[(int64_t)k * ntiles + tile] = c[k];
@@ -70,49 +84,78 @@ __global__ void __launch_bounds__(kPartCta) k_part_count(const int32_t *vals, in
     }
 }
 
-// scan = exclusive scan of counts (key-major); one CTA: padded key starts,
-// shift[k] = padded start - unpadded start, pstart[nkeys] = padded total
-__global__ void k_part_starts(const int32_t *scan, int32_t ntiles, int32_t nkeys, int32_t pad,
-                              int32_t *shift, int32_t *pstart, int32_t *total) {
-    __shared__ int32_t s_beg[kPartMaxKeys + 1];
-    for (int k = threadIdx.x; k <= nkeys; k += blockDim.x) s_beg[k] = scan[(int64_t)k * ntiles];
+// scan = exclusive scan of counts (key-major); one CTA, a key per thread:
+// padded key starts, shift[k] = padded start - unpadded start, pstart[nkeys] =
+// padded total (a serial loop over 256 keys with its divisions took 28 us)
+__global__ void __launch_bounds__(kPartMaxKeys) k_part_starts(const int32_t *scan, int32_t ntiles,
+                                                              int32_t nkeys, int32_t pad,
+                                                              int32_t *shift, int32_t *pstart,
+                                                              int32_t *total) {
+    __shared__ int32_t s_warp[kPartMaxKeys / 32];
+    const int k = threadIdx.x, lane = k & 31, wid = k >> 5;
+    int32_t beg = 0, size = 0;
+    if (k < nkeys) {
+        beg = scan[(int64_t)k * ntiles];
+        // (the padded total fits int32: pr_blk_applies)
+        size = (int32_t)(((int64_t)scan[(int64_t)(k + 1) * ntiles] - beg + pad - 1) / pad * pad);
+    }
+    int32_t incl = warp_incl_scan(size);
+    if (lane == 31) s_warp[wid] = incl;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t acc = 0;
-        for (int k = 0; k < nkeys; ++k) {
-            const int64_t size = s_beg[k + 1] - s_beg[k];
-            pstart[k] = (int32_t)acc;
-            shift[k] = (int32_t)(acc - s_beg[k]);
-            acc += (size + pad - 1) / pad * pad;
-        }
-        pstart[nkeys] = (int32_t)acc;
-        *total = (int32_t)acc;
+    if (wid == 0) s_warp[lane] = warp_incl_scan(s_warp[lane]);
+    __syncthreads();
+    if (wid) incl += s_warp[wid - 1];
+    if (k < nkeys) {
+        pstart[k] = incl - size;
+        shift[k] = incl - size - beg;
+    }
+    if (k == nkeys - 1) {
+        pstart[nkeys] = incl;
+        *total = incl;
     }
 }
 
+// Positions of the items, eight steps' claims side by side (see k_blk_place:
+// the first lane of each key's group claims the group's positions with one
+// shared atomic; a warp's claims to a counter are served in order).
 __global__ void __launch_bounds__(kPartCta) k_part_pos(const int32_t *vals, int32_t div,
                                                        int64_t count, int32_t nkeys, int32_t ntiles,
-                                                       const int32_t *scan, const int32_t *shift,
-                                                       int32_t *pos) {
+                                                       int32_t per, const int32_t *scan,
+                                                       const int32_t *shift, int32_t *pos) {
     extern __shared__ int32_t s_part[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
     int32_t *c = s_part + wid * nkeys;
     const int32_t wpc = kPartCta / 32;
+    const float inv = 1.0f / (float)div;
     for (int32_t tile = blockIdx.x * wpc + wid; tile < ntiles; tile += gridDim.x * wpc) {
         for (int k = lane; k < nkeys; k += 32) c[k] = scan[(int64_t)k * ntiles + tile] + shift[k];
         __syncwarp();
-        const int64_t base = (int64_t)tile * kPartTile;
-        for (int s = 0; s < kPartTile / 32; ++s) {
-            const int64_t i = base + s * 32 + lane;
-            const int key = i < count ? vals[i] / div : -1;
-            const unsigned peers = __match_any_sync(G2_FULL, key);
-            const int r = __popc(peers & lt);
-            if (key >= 0) pos[i] = c[key] + r;
-            __syncwarp();
-            if (key >= 0 && r == 0) c[key] += __popc(peers);
-            __syncwarp();
+        const int64_t base = (int64_t)tile * per;
+        constexpr int kB = 8;
+        for (int s0 = 0; s0 < per / 32; s0 += kB) {
+            int key[kB], got[kB], who[kB];
+#pragma unroll
+            for (int j = 0; j < kB; ++j) {
+                const int64_t i = base + (s0 + j) * 32 + lane;
+                key[j] = i < count ? div_floor(vals[i], div, inv) : -1;
+            }
+#pragma unroll
+            for (int j = 0; j < kB; ++j) {
+                const unsigned peers = __match_any_sync(G2_FULL, key[j]);
+                const int lead = __ffs(peers) - 1;
+                got[j] = 0;
+                if (key[j] >= 0 && lane == lead) got[j] = atomicAdd(&c[key[j]], __popc(peers));
+                who[j] = (lead << 8) | __popc(peers & lt);
+            }
+#pragma unroll
+            for (int j = 0; j < kB; ++j) {
+                const int64_t i = base + (s0 + j) * 32 + lane;
+                const int32_t p = __shfl_sync(G2_FULL, got[j], who[j] >> 8) + (who[j] & 0xFF);
+                if (key[j] >= 0) pos[i] = p;
+            }
         }
+        __syncwarp();  // the tile's claims are done before the counters are reset
     }
 }
 
@@ -567,9 +610,9 @@ struct PartTable {
 
 // The tables of a stable partition of count items into nkeys keys, and the
 // launch shape of its count and position passes.
-static g2_status partition_alloc(g2_graph *g, int64_t count, int32_t nkeys, PartTable *pt,
-                                 cudaStream_t st) {
-    pt->ntiles = (int32_t)std::max<int64_t>(1, (count + kPartTile - 1) / kPartTile);
+static g2_status partition_alloc(g2_graph *g, int64_t count, int32_t nkeys, int32_t per,
+                                 PartTable *pt, cudaStream_t st) {
+    pt->ntiles = (int32_t)std::max<int64_t>(1, (count + per - 1) / per);
     const int64_t cells = (int64_t)nkeys * pt->ntiles;
     if (cells >= 2147483647LL) return fail(G2_EUNSUPPORTED, "partition table too large");
     G2_CK(dmalloc(&pt->counts, (size_t)(cells + 1) * 4, st));
@@ -589,31 +632,26 @@ static g2_status partition_starts(g2_graph *g, int32_t nkeys, int32_t pad, int32
     G2_TRY(exclusive_scan_i32(g, pt->counts, pt->scan, (int32_t)((int64_t)nkeys * pt->ntiles), st));
     k_part_starts<<<1, 1024, 0, st>>>(pt->scan, pt->ntiles, nkeys, pad, pt->shift, pstart, d_total);
     G2_CK(cudaGetLastError());
+    stats().launches += 1;
+    if (!total) return G2_OK;
     G2_CK(cudaMemcpyAsync(g->h_ctr + 50, d_total, 4, cudaMemcpyDeviceToHost, st));
     G2_CK(cudaStreamSynchronize(st));
     *total = g->h_ctr[50];
-    stats().launches += 1;
     return G2_OK;
 }
 
-static g2_status partition_table(g2_graph *g, const int32_t *vals, int32_t div, int64_t count,
-                                 int32_t nkeys, int32_t pad, int32_t *pstart, int64_t *total,
-                                 PartTable *pt, cudaStream_t st) {
-    G2_TRY(partition_alloc(g, count, nkeys, pt, st));
-    k_part_count<<<pt->grid, kPartCta, pt->smem, st>>>(vals, div, count, nkeys, pt->ntiles,
-                                                       pt->counts);
-    stats().launches += 1;
-    return partition_starts(g, nkeys, pad, pstart, total, pt, st);
-}
-
-// Positions of a stable partition: pos[i] for every item.
+// Positions of a stable partition of the vertices: pos[i] for every item.
 static g2_status stable_partition(g2_graph *g, const int32_t *vals, int32_t div, int64_t count,
                                   int32_t nkeys, int32_t pad, int32_t *pos, int32_t *pstart,
-                                  int64_t *total, cudaStream_t st) {
+                                  cudaStream_t st) {
     PartTable pt;
-    G2_TRY(partition_table(g, vals, div, count, nkeys, pad, pstart, total, &pt, st));
-    k_part_pos<<<pt.grid, kPartCta, pt.smem, st>>>(vals, div, count, nkeys, pt.ntiles, pt.scan, pt.shift,
-                                                   pos);
+    G2_TRY(partition_alloc(g, count, nkeys, kPartTileV, &pt, st));
+    k_part_count<<<pt.grid, kPartCta, pt.smem, st>>>(vals, div, count, nkeys, pt.ntiles, kPartTileV,
+                                                     pt.counts);
+    stats().launches += 1;
+    G2_TRY(partition_starts(g, nkeys, pad, pstart, nullptr, &pt, st));
+    k_part_pos<<<pt.grid, kPartCta, pt.smem, st>>>(vals, div, count, nkeys, pt.ntiles, kPartTileV,
+                                                   pt.scan, pt.shift, pos);
     G2_CK(cudaGetLastError());
     stats().launches += 1;
     pt.release(st);
@@ -662,8 +700,7 @@ g2_status ensure_blk_layout(g2_graph *g, int32_t S, cudaStream_t st) {
     G2_CK(dmalloc(&t->blk_cta, ((size_t)G + 1) * 4, st));
     // 1. vertex ranks
     k_blk_vkey<<<grid, kCta, 0, st>>>(t->rowptr, n, vkey);
-    int64_t vtotal = 0;
-    G2_TRY(stable_partition(g, vkey, 1, n, kDegBuckets, 1, rank, vstart, &vtotal, st));
+    G2_TRY(stable_partition(g, vkey, 1, n, kDegBuckets, 1, rank, vstart, st));
     // the first rank without out-arcs (bucket 0 is ranked last)
     G2_CK(cudaMemcpyAsync(g->h_ctr + 52, vstart + (kDegBuckets - 1), 4, cudaMemcpyDeviceToHost, st));
     k_blk_order<<<grid, kCta, 0, st>>>(t->rowptr, rank, n, t->blk_order, t->blk_deg);
@@ -684,7 +721,7 @@ g2_status ensure_blk_layout(g2_graph *g, int32_t S, cudaStream_t st) {
         G2_CK(dmalloc(&srank, (size_t)m * 4, st));
         G2_CK(dmalloc(&drank, (size_t)m * 4, st));
         PartTable pt;
-        G2_TRY(partition_alloc(g, m, nb, &pt, st));
+        G2_TRY(partition_alloc(g, m, nb, kPartTile, &pt, st));
         k_blk_src_count<<<pt.grid, kPartCta, pt.smem, st>>>(t->ccol, rank, S, m, nb, pt.ntiles,
                                                              srank, pt.counts);
         {
