@@ -155,6 +155,72 @@ __device__ bool fused_strict_scan(const DevGraph &g, const int32_t *q, int32_t s
     return grid_sync(bar, err, limit_ns);
 }
 
+// A PULL level of the fused hybrid: every vertex without a depth looks for its
+// first in-neighbour in the frontier `cur` of level d; the vertices found are
+// the next level's bitmap (a word is stored by the one warp that owns it), their
+// number, in lane 0, the result.  The chain of depth, row offsets, id and frontier
+// bit is what bounds it, so a warp takes W words at once and a lane has W of them
+// in flight: the whole search of RMAT-22 from the hub 191 us with one, 173 with
+// two, 156 with four, 177 with eight (registers).  Taking one at a time where
+// there are fewer than four words per warp gains nothing in the same kernel
+// (RMAT-14: 63 us both ways).
+__device__ __forceinline__ int32_t pull_level(const FusedDoBfsArgs &a, const uint32_t *cur, int d,
+                                              int64_t gwarp, int64_t nwarps) {
+    constexpr int W = 4;
+    const int lane = threadIdx.x & 31;
+    const int32_t n = a.g.n;
+    uint32_t *next = a.bm[(d + 1) & 1];
+    int32_t found = 0;
+    for (int64_t base = gwarp * 32 * W; base < n; base += nwarps * 32 * W) {
+        int32_t e[W], e1[W], acc[W];
+        int scanned = 0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const int64_t v = base + 32 * j + lane;
+            const bool open = v < n && a.depth[v] == -1;
+            e[j] = open ? a.g.crowptr[v] : 0;
+            e1[j] = open ? a.g.crowptr[v + 1] : 0;
+            acc[j] = -1;
+        }
+        for (;;) {
+            bool more = false;
+            int32_t u[W];
+            uint32_t bits[W];
+#pragma unroll
+            for (int j = 0; j < W; ++j) u[j] = e[j] < e1[j] ? a.g.ccol[e[j]] : -1;
+#pragma unroll
+            for (int j = 0; j < W; ++j) bits[j] = u[j] >= 0 ? cur[u[j] >> 5] >> (u[j] & 31) : 0u;
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                if (u[j] < 0) continue;
+                ++scanned;
+                ++e[j];
+                if (bits[j] & 1u) {
+                    acc[j] = u[j];  // ascending in-list: the first hit is the smallest
+                    e[j] = e1[j];
+                }
+                more |= e[j] < e1[j];
+            }
+            if (!more) break;
+        }
+        count_arcs(a.ctr, scanned);
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            const int64_t v0 = base + 32 * j;
+            if (acc[j] >= 0) {
+                a.depth[v0 + lane] = d + 1;
+                if (a.parent) a.parent[v0 + lane] = acc[j];
+            }
+            const unsigned mask = __ballot_sync(G2_FULL, acc[j] >= 0);
+            if (lane == 0 && v0 < n) {
+                next[v0 >> 5] = mask;
+                found += __popc(mask);
+            }
+        }
+    }
+    return found;
+}
+
 // CTAs per SM of the fused STRICT kernels (64 registers; a fifth gains BFS 3%
 // on RMAT-22 and costs RMAT-14 and delta-stepping 4-5%).
 constexpr int kFusedStrictCtas = 4;
@@ -178,7 +244,6 @@ __device__ __forceinline__ bool fused_strict(const DevGraph &g, const FrontierIn
 template <int LB>
 __global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 1) k_bfs_fused_do(FusedDoBfsArgs a) {
     OpBFS op{a.depth, a.parent};
-    PullBFS pop{a.depth, a.parent};
     const int lane = threadIdx.x & 31;
     const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nt = (int64_t)gridDim.x * blockDim.x;
@@ -270,35 +335,7 @@ __global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             }
             // bottom-up over every vertex; the next level as a bitmap
-            Member mem{MEM_BITMAP, cur, nullptr};
-            uint32_t *next = a.bm[(d + 1) & 1];
-            int32_t found = 0;
-            for (int64_t base = gwarp * 32; base < n; base += nwarps * 32) {
-                const int64_t v = base + lane;
-                int code = 0, scanned = 0;
-                if (v < n) {
-                    const int32_t c = pop.ctx((int32_t)v);
-                    if (pop.filter(c)) {
-                        int32_t acc = pop.identity();
-                        const int32_t e1 = a.g.crowptr[v + 1];
-                        for (int32_t e = a.g.crowptr[v]; e < e1; ++e) {
-                            const int32_t u = a.g.ccol[e];
-                            ++scanned;
-                            if (mem.has(u)) {
-                                acc = u;  // ascending in-list: the first hit is the smallest
-                                break;
-                            }
-                        }
-                        code = pop.finish((int32_t)v, c, acc);
-                    }
-                }
-                count_arcs(a.ctr, scanned);
-                const unsigned mask = __ballot_sync(G2_FULL, code & 1);
-                if (lane == 0) {
-                    next[base >> 5] = mask;
-                    found += __popc(mask);
-                }
-            }
+            const int32_t found = pull_level(a, cur, d, gwarp, nwarps);
             if (lane == 0 && found) atomicAdd(a.bcnt + (d + 1) % 3, found);
             if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             sparse = false;
