@@ -259,12 +259,13 @@ g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, void *vdata, 
  * grid-wide kernel (back below half that size), one launch per hand-over.
  * A hybrid with kernel fusion on both schedules and s2 VERTEX_BASED PULL over
  * a bitmap runs in one cooperative kernel too, choosing the direction per
- * level; its PUSH half is VERTEX_BASED, WM, CM, ETWC (CTA-stage entries of
- * 4096 arcs or more go to a grid-wide pass inside the launch) or STRICT (the
- * prefix sum of the level's degrees taken over the grid inside the launch).
+ * level; its PUSH half is VERTEX_BASED, WM, CM, ETWC (CTA-stage entries go to
+ * a grid-wide pass inside the launch, in pieces) or STRICT (the prefix sum of
+ * the level's degrees taken over the grid inside the launch).
  * NULL schedule: that fused direction-optimising hybrid, STRICT PUSH below 2%
- * of n, VERTEX_BASED PULL over a bitmap otherwise; on a bounded-degree graph
- * (largest out-degree <= 32: road networks, meshes) fused WM PUSH instead. */
+ * of n and up to a sixteenth of the arcs, VERTEX_BASED PULL over a bitmap
+ * otherwise; on a bounded-degree graph (largest out-degree <= 32: road
+ * networks, meshes) fused WM PUSH instead. */
 g2_status g2_bfs(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
                  const g2_hybrid *sched, void *stream);
 
@@ -285,9 +286,11 @@ g2_status g2_cc(g2_graph *g, int32_t *label, const g2_hybrid *sched, void *strea
  * G2_EOVERFLOW if a distance would reach INT32_MAX.  With kernel fusion and
  * WM, buckets run inside one thread-block cluster (near lists and far piles in
  * shared memory) while near rounds hold at most 1,024 vertices per cluster CTA,
- * and in the grid-wide kernel otherwise (back at a bucket boundary with a
- * small far pile), one launch per hand-over.  NULL schedule: STRICT PUSH
- * in one cooperative launch; fused WM PUSH on a bounded-degree graph (largest out-degree <= 32). */
+ * (512 on a bounded-degree graph of more than 16,384 vertices) and in the
+ * grid-wide kernel otherwise (back at a bucket boundary with a small far
+ * pile), one launch per hand-over.  NULL schedule: STRICT PUSH in one
+ * cooperative launch; fused WM PUSH on a bounded-degree graph (largest
+ * out-degree <= 32). */
 g2_status g2_sssp_delta(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
                         const g2_hybrid *sched, void *stream);
 
@@ -318,9 +321,9 @@ g2_status g2_pagerank(g2_graph *g, float damping, int32_t iters, float *rank,
  * bounded-degree graph the levels of at most 256 vertices per cluster CTA run
  * inside one thread-block cluster (forward and backward), the larger ones in
  * the grid-wide kernel.  NULL schedule: the
- * direction-optimising hybrid as per-level launches (STRICT PUSH below 2% of
- * n, VERTEX_BASED PULL); fused WM PUSH on a bounded-degree graph (largest
- * out-degree <= 32). */
+ * direction-optimising hybrid (STRICT PUSH below 2% of n, VERTEX_BASED PULL)
+ * as per-level launches, or with several sources g2_bfs's one launch per
+ * source; fused WM PUSH on a bounded-degree graph (largest out-degree <= 32). */
 g2_status g2_bc(g2_graph *g, const int32_t *srcs, int32_t k, double *bc,
                 const g2_hybrid *sched, void *stream);
 
@@ -349,8 +352,8 @@ g2_status g2_bfs_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dep
  * fusion with WM PUSH (the whole loop in one cooperative kernel).  NULL
  * schedule: the distances of a vertex from all sources relaxed together as one
  * row, in rounds over the vertices whose row changed (delta is not used), or
- * STRICT PUSH where that has not ended after 32 rounds; on a bounded-degree graph (largest out-degree <= 32)
- * the sources run as single-source fused WM queries, about one per 19 SMs at
+ * STRICT PUSH where that has not ended after 32 rounds; on a bounded-degree
+ * graph (largest out-degree <= 32) the sources run as single-source fused WM queries, about one per 19 SMs at
  * a time, as g2_bfs_batch does (G2_BATCH_SPLIT_WORKERS = 0: the fused
  * multi-source loop). */
 g2_status g2_sssp_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t delta,
@@ -417,8 +420,8 @@ typedef struct {
     int32_t iterations;     /* frontier rounds (or PR rounds, CC rounds, buckets) */
     int32_t push_rounds;    /* rounds run PUSH */
     int32_t pull_rounds;    /* rounds run PULL */
-    int32_t launches;       /* kernels launched (not counting the one-warp kernels that
-                               store a call's few host-side values, e.g. the source) */
+    int32_t launches;       /* kernels launched (not counting those that only store a
+                               call's initial values, e.g. the source) */
     int64_t arcs_examined;  /* arcs read by the traversal (0 unless counted) */
     int32_t barriers;       /* grid or cluster barriers passed in fused kernels */
     int32_t reserved;

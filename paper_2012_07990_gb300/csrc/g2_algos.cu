@@ -17,7 +17,7 @@ namespace g2 {
 g2_status bfs_fused(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
                     const g2_schedule &s, cudaStream_t st, int32_t *d_err);
 g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
-                       const g2_hybrid &h, cudaStream_t st, int32_t *d_err);
+                       const g2_hybrid &h, bool by_arcs, cudaStream_t st, int32_t *d_err);
 g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
                      const g2_schedule &s, cudaStream_t st, int32_t *d_err);
 
@@ -583,10 +583,10 @@ static bool bounded_degree(g2_graph *g, cudaStream_t st) {
 // Tuned schedule for BFS when the caller passes none (measured on GB300 with
 // RMAT-21 and RMAT-22): the direction-optimising hybrid fused into one
 // launch, STRICT PUSH on a sparse queue while the frontier holds < 2% of the
-// vertices, else VERTEX_BASED PULL over a bitmap.  Against the same hybrid
-// as per-level launches it is faster from every source measured (RMAT-22,
-// the hub and 8 random sources: 5.7 ms against 6.9 ms in all; from the hub
-// 0.26 against 0.35 ms): no frontier size goes back to the host per level.
+// vertices and at most a sixteenth of the arcs (kPushArcsPart), else
+// VERTEX_BASED PULL over a bitmap.  Against the same hybrid as per-level
+// launches it is faster from every source measured (RMAT-22 from the hub 0.16
+// against 0.34 ms): no frontier size goes back to the host per level.
 // STRICT divides a level's arcs evenly over the persistent grid where ETWC's
 // stages leave it unbalanced behind hub arcs (fused ETWC: 20.8 ms over the
 // same sources).  On a bounded-degree graph: fused WM PUSH (measured on a
@@ -636,7 +636,7 @@ g2_status g2_bfs(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent, cons
         if (h.criteria != G2_CRITERIA_NONE && !h.s2.kernel_fusion)
             return fail(G2_EUNSUPPORTED, "kernel fusion must be set on both hybrid schedules");
         if (h.criteria != G2_CRITERIA_NONE && h.s2.direction == G2_PULL)
-            G2_TRY(bfs_fused_do(g, src, depth, parent, h, st, d_err));
+            G2_TRY(bfs_fused_do(g, src, depth, parent, h, !sched, st, d_err));
         else
             G2_TRY(bfs_fused(g, src, depth, parent, h.s1, st, d_err));
     } else {

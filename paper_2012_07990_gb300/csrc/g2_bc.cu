@@ -44,7 +44,7 @@
 namespace g2 {
 
 g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
-                       const g2_hybrid &h, cudaStream_t st, int32_t *d_err);
+                       const g2_hybrid &h, bool by_arcs, cudaStream_t st, int32_t *d_err);
 
 constexpr int32_t kBigDeg = 4096;    // a CTA per vertex from this many arcs
 constexpr int32_t kThreadDeg = 32;   // a thread per vertex below this many arcs
@@ -842,7 +842,7 @@ static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h,
         const int32_t it = stats().iterations, push = stats().push_rounds, pull = stats().pull_rounds;
         // the hybrid's counters, zero at the start of a call, lie in ctrs[20, 56)
         G2_CK(cudaMemsetAsync(d_err - 62 + 20, 0, 36 * 4, st));
-        G2_TRY(bfs_fused_do(g, s.src, s.depth, nullptr, h, st, d_err));
+        G2_TRY(bfs_fused_do(g, s.src, s.depth, nullptr, h, true, st, d_err));
         levels = stats().iterations;
         stats().iterations += it - 1;
         stats().push_rounds += push;

@@ -100,7 +100,8 @@ struct FusedDoBfsArgs {
     int32_t *cnt;        // [3] list lengths; cnt[0] = 1 (the source) at launch, the rest 0
     uint32_t *bm[2];     // frontier bitmaps, (n + 31) / 32 words each
     int32_t *bcnt;       // [3] bitmap populations, 0 at launch
-    int32_t push_below;  // PUSH while the frontier holds fewer vertices
+    int32_t push_below;  // PUSH while the frontier holds fewer vertices ...
+    int32_t push_arcs;   // ... and (STRICT) at most this many arcs
     int32_t *scan;       // STRICT: prefix sums of a PUSH level's degrees (n + 1) ...
     int32_t *ctasum;     // ... and the slice totals of the CTAs (one per CTA)
     EtwcEntry<int32_t> *spq;  // ETWC: a level's CTA-stage pieces (room for spcap) ...
@@ -225,20 +226,23 @@ __device__ __forceinline__ int32_t pull_level(const FusedDoBfsArgs &a, const uin
 // on RMAT-22 and costs RMAT-14 and delta-stepping 4-5%).
 constexpr int kFusedStrictCtas = 4;
 
-// One STRICT round of a fused loop (no barrier after it).  False: a barrier
-// wait gave up.
+// One STRICT round of a fused loop (no barrier after it), left out in every
+// CTA if the list has more than `most` arcs.
+enum { ROUND_FAILED, ROUND_DONE, ROUND_TOO_MANY };  // failed: a barrier wait gave up
 template <class Op>
-__device__ __forceinline__ bool fused_strict(const DevGraph &g, const FrontierIn &fin, int32_t size,
-                                             const Op &op, const OutCtx &out, int32_t *scan,
-                                             int32_t *ctasum, const GridBarrier &bar, int32_t *err,
-                                             uint64_t limit_ns, unsigned long long *ctr) {
-    if (size <= kStrictSmall) {
-        lb_strict_small(g, fin, size, op, out, blockIdx.x, gridDim.x, ctr);
-        return true;
-    }
-    if (!fused_strict_scan(g, fin.q, size, scan, ctasum, bar, err, limit_ns)) return false;
+__device__ __forceinline__ int fused_strict(const DevGraph &g, const FrontierIn &fin, int32_t size,
+                                            const Op &op, const OutCtx &out, int32_t *scan,
+                                            int32_t *ctasum, const GridBarrier &bar, int32_t *err,
+                                            uint64_t limit_ns, unsigned long long *ctr,
+                                            int32_t most = 0x7fffffff) {
+    if (size <= kStrictSmall)
+        return lb_strict_small(g, fin, size, op, out, blockIdx.x, gridDim.x, ctr, most)
+                   ? ROUND_DONE
+                   : ROUND_TOO_MANY;
+    if (!fused_strict_scan(g, fin.q, size, scan, ctasum, bar, err, limit_ns)) return ROUND_FAILED;
+    if (most != 0x7fffffff && scan[size] > most) return ROUND_TOO_MANY;
     lb_strict(g, fin, size, scan, op, out, blockIdx.x, gridDim.x, ctr);
-    return true;
+    return ROUND_DONE;
 }
 
 template <int LB>
@@ -266,7 +270,9 @@ __global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 
             a.bcnt[(d + 2) % 3] = 0;
             if (a.spcnt) a.spcnt[(d + 1) & 1] = 0;
         }
-        if (size < a.push_below) {
+        bool push = size < a.push_below;
+        const bool bits_of_d = !sparse;  // level d's bitmap is there
+        if (push) {
             if (!sparse) {
                 // bitmap -> list d & 1 (cnt[d % 3] is zero: cleared two levels ago)
                 const uint32_t *bm = a.bm[d & 1];
@@ -313,17 +319,19 @@ __global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 
                 }
             } else if (LB == G2_LB_STRICT) {
                 // the same number of arcs for every thread of the grid
-                if (!fused_strict(a.g, fin, size, op, out, a.scan, a.ctasum, a.bar, a.err, a.limit_ns,
-                                  a.ctr))
-                    return;
-                if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
+                const int r = fused_strict(a.g, fin, size, op, out, a.scan, a.ctasum, a.bar, a.err,
+                                           a.limit_ns, a.ctr, a.push_arcs);
+                if (r == ROUND_FAILED) return;
+                push = r == ROUND_DONE;
+                if (push && !grid_sync(a.bar, a.err, a.limit_ns)) return;
             } else {
                 run_lb<LB>(a.g, fin, size, op, out, a.ctr);
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             }
-        } else {
+        }
+        if (!push) {
             uint32_t *cur = a.bm[d & 1];
-            if (sparse) {
+            if (!bits_of_d) {
                 // list d & 1 -> bitmap: clear it, then set the list's bits
                 for (int64_t w = gt; w < words; w += nt) cur[w] = 0u;
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
@@ -1085,8 +1093,18 @@ __global__ void k_bfs_do_init(int32_t *depth, int32_t *parent, int32_t n, int32_
 // PUSH schedule (a load balancing of the fused loops), h.s2 VERTEX_BASED
 // PULL over a bitmap; PUSH while the frontier holds fewer than threshold * n
 // vertices.
+// The tuned hybrid's second line (`by_arcs`): a list of few vertices but more
+// than a sixteenth of the graph's arcs (hubs) is not pushed either; STRICT's
+// prefix sum has the number.  The push of such a level reads every one of its
+// arcs, the pull ends each list at its first hit.  RMAT-22, the hub and 12
+// random sources: 4.01 ms without the line, 2.52 with it at an eighth, 2.53 at a
+// sixteenth, 2.75 at a 32nd, 3.01 at a fourth or a 64th (most levels lie well to
+// one side); RMAT-21 2.05 -> 1.76 ms.  Below 2^18 arcs a push takes about as long as
+// making the bitmap (RMAT-14: the same with and without).
+constexpr int32_t kPushArcsPart = 16, kPushArcsLeast = 1 << 18;
+
 g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent,
-                       const g2_hybrid &h, cudaStream_t st, int32_t *d_err) {
+                       const g2_hybrid &h, bool by_arcs, cudaStream_t st, int32_t *d_err) {
     // the PUSH half: a load balancing of the fused loops, or STRICT (its
     // prefix sum taken inside the launch)
     if (h.s1.load_balance == G2_LB_STRICT) {
@@ -1132,6 +1150,7 @@ g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent
     }
     const double pb = (double)h.threshold * (double)n;
     a.push_below = (int32_t)std::min<double>(std::max<double>(pb, 0.0), 2147483647.0);
+    a.push_arcs = by_arcs ? std::max(t->m / kPushArcsPart, kPushArcsLeast) : 0x7fffffff;
     a.result = ctrs + 24;
     a.bar = GridBarrier{reinterpret_cast<unsigned long long *>(ctrs + 28)};
     a.err = d_err;

@@ -352,12 +352,14 @@ __device__ void lb_strict(const DevGraph &g, const FrontierIn &fin, int32_t fsiz
 // STRICT for a list of up to kStrictSmall entries in a fused loop, without a
 // scan of the whole grid before it: every CTA scans the list's degrees itself
 // (1 us, against two grid barriers and a pass over the list) and takes every
-// nb-th tile of its arcs.
+// nb-th tile of its arcs.  False, in every CTA, and nothing done if there are
+// more than `most` arcs.
 constexpr int kStrictSmall = 4 * kCta;
 
 template <class Op>
-__device__ void lb_strict_small(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
-                                const OutCtx &out, int bid, int nb, unsigned long long *ctr) {
+__device__ bool lb_strict_small(const DevGraph &g, const FrontierIn &fin, int32_t fsize, const Op &op,
+                                const OutCtx &out, int bid, int nb, unsigned long long *ctr,
+                                int32_t most = 0x7fffffff) {
     typedef typename Op::S S;
     constexpr int N = Op::kFlight, kTile = kCta * N, kPer = kStrictSmall / kCta;
     Stage st = stage_begin();
@@ -386,6 +388,7 @@ __device__ void lb_strict_small(const DevGraph &g, const FrontierIn &fin, int32_
     }
     int total;
     int at = block_incl_scan(sum, s_warp, &total) - sum;
+    if (total > most) return false;  // the same in every CTA
 #pragma unroll
     for (int j = 0; j < kPer; ++j) {
         const int i = tid * kPer + j;
@@ -426,6 +429,7 @@ __device__ void lb_strict_small(const DevGraph &g, const FrontierIn &fin, int32_
     }
     stage_end(out, st);
     __syncthreads();  // the next call writes the arrays
+    return true;
 }
 
 // ---------------------------------------------------------------------- ETWC
