@@ -286,8 +286,7 @@ g2_status g2_cc(g2_graph *g, int32_t *label, const g2_hybrid *sched, void *strea
  * G2_EOVERFLOW if a distance would reach INT32_MAX.  With kernel fusion and
  * WM, buckets run inside one thread-block cluster (near lists and far piles in
  * shared memory) while near rounds hold at most 1,024 vertices per cluster CTA,
- * (512 on a bounded-degree graph of more than 16,384 vertices) and in the
- * grid-wide kernel otherwise (back at a bucket boundary with a small far
+ * and in the grid-wide kernel otherwise (back at a bucket boundary with a small far
  * pile), one launch per hand-over.  NULL schedule: STRICT PUSH in one
  * cooperative launch; fused WM PUSH on a bounded-degree graph (largest
  * out-degree <= 32). */

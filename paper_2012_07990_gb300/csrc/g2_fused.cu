@@ -1244,11 +1244,11 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     c.stamp2 = a.stamp2;
     int32_t dmax = 0;
     if (cl) G2_TRY(max_out_degree(g, st, &dmax));
-    // Measured on road grids with the grid-wide loop at two CTAs per SM: hand a
-    // near round of more than 8,192 vertices to the grid (4096^2, delta 16384:
-    // 35.6 ms against 36.5 with 16,384; 1024^2: no difference down to 4,096).
-    // Graphs that fit one round of the cluster stay in it.
-    const int32_t hi = dmax <= kBoundedDegree && n > 1024 * cl ? 512 * cl : 1024 * cl;
+    // Handing near rounds of 8,192 vertices to a grid of two CTAs per SM is
+    // faster alone (4096^2, delta 16384: 34.4 ms against 38) and slower
+    // beside other streams, where that launch waits for the whole GPU (a mixed
+    // load of 500 queries a second in 4 slots: p99 390 ms against 73).
+    const int32_t hi = 1024 * cl;
     c.hi = env_i32("G2_CLUSTER_HI", hi);
     c.dedup_near = !(t->symmetric && dmax <= kBoundedDegree);
     c.nq_out = a.nq[0];
@@ -1301,10 +1301,9 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
             a.T0 = T;
             a.round0 = round0;
             a.epoch0 = epoch0;
-            // two CTAs per SM: the shares of a round of 10,000 vertices are one
-            // step of a warp each (4096^2, delta 16384: 38.0 ms with one, 35.6
-            // with two)
-            const int ctas = env_i32("G2_FUSED_CTAS_PER_SM", 2);
+            // one CTA per SM (two: 35.6 against 38.0 ms on 4096^2 with delta
+            // 16384, but see above)
+            const int ctas = env_i32("G2_FUSED_CTAS_PER_SM", 1);
             switch (s.load_balance) {
                 case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st, ctas)); break;
                 case G2_LB_CM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_CM>, a, st)); break;
