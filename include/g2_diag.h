@@ -1,7 +1,8 @@
 /*
- * g2_diag.h — measurement probes of libg2.so that are not part of the
- * traversal library: they time access patterns of its kernels on their own,
- * to find the floor a kernel runs against.  Same conventions as g2.h.
+ * g2_diag.h — probes of libg2.so that are not part of the traversal library:
+ * one times access patterns of its kernels on their own, to find the floor a
+ * kernel runs against; one lets a test meet a device without room.  Same
+ * conventions as g2.h.
  */
 #ifndef G2_DIAG_H
 #define G2_DIAG_H
@@ -27,6 +28,12 @@ extern "C" {
  * arc sweep on that index order.  Synchronises `stream` before returning. */
 g2_status g2_diag_gather(const int32_t *idx, int64_t m, const float *x, int32_t n, int32_t mode,
                          float *out, int32_t grid, float *ms, void *stream);
+
+/* Test aid: of the calling thread's next device allocations of at least
+ * min_bytes, the nth (1 = the first; 0 = none) fails as on a device without
+ * room, once.  *left (host, may be NULL) receives what was left to count of
+ * the request before: 0 if its failure has happened (or none was asked for). */
+g2_status g2_diag_fail_alloc(int32_t nth, int64_t min_bytes, int32_t *left);
 
 #ifdef __cplusplus
 }

@@ -10,6 +10,9 @@
 // atomics: a floor for the sweep on that order of indices.  mode 1 streams
 // idx alone (the column bytes, no gather).  The indices are checked in a
 // separate pass first; the pass that is timed loads without checks.
+//
+// g2_diag_fail_alloc: an allocation that fails on request, for tests of what
+// a call does when the device has no room.
 #include <cuda_runtime.h>
 
 #include "g2_diag.h"
@@ -52,6 +55,13 @@ __global__ void __launch_bounds__(256) k_diag_gather(const int32_t *__restrict__
 }  // namespace g2
 
 using namespace g2;
+
+extern "C" g2_status g2_diag_fail_alloc(int32_t nth, int64_t min_bytes, int32_t *left) {
+    if (nth < 0 || min_bytes < 0) return fail(G2_EINVAL, "bad g2_diag_fail_alloc arguments");
+    const int32_t before = fail_alloc(nth, (size_t)min_bytes);
+    if (left) *left = before;
+    return G2_OK;
+}
 
 extern "C" g2_status g2_diag_gather(const int32_t *idx, int64_t m, const float *x, int32_t n,
                                     int32_t mode, float *out, int32_t grid, float *ms,

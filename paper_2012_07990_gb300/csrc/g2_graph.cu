@@ -30,6 +30,10 @@ g2_status fail(g2_status st, const std::string &msg) {
 }
 g2_status cuda_fail(cudaError_t e, const char *what) {
     t_err = std::string(what) + ": " + cudaGetErrorString(e);
+    // reported here: it must not be found again by the check after a later
+    // launch (a failed allocation would fail the next call too, or the form
+    // that a call falls back to)
+    cudaGetLastError();
     if (e == cudaErrorMemoryAllocation) return G2_ENOMEM;
     return G2_ECUDA;
 }
@@ -444,9 +448,23 @@ cudaMemPool_t current_pool() {
 }
 }  // namespace
 
+// g2_diag_fail_alloc: which of this thread's next allocations of at least
+// t_fail_bytes fails (0: none does)
+static thread_local int32_t t_fail_nth = 0;
+static thread_local size_t t_fail_bytes = 0;
+
+int32_t fail_alloc(int32_t nth, size_t bytes) {
+    const int32_t left = t_fail_nth;
+    t_fail_nth = nth;
+    t_fail_bytes = bytes;
+    return left;
+}
+
 cudaError_t dmalloc_bytes(void **p, size_t bytes, cudaStream_t st) {
     *p = nullptr;
     if (bytes < 16) bytes = 16;
+    // more than any device has, so that CUDA's allocator itself refuses
+    if (t_fail_nth > 0 && bytes >= t_fail_bytes && --t_fail_nth == 0) bytes = (size_t)1 << 50;
     cudaMemPool_t pool = current_pool();
     if (!pool) return cudaMalloc(p, bytes);
     return cudaMallocFromPoolAsync(p, bytes, pool, st);

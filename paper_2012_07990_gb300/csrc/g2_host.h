@@ -172,6 +172,7 @@ struct Topology {
 //  dfree:   the release is ordered after the work already queued on `st`;
 //           the block must not be in use by work on any other stream.
 cudaError_t dmalloc_bytes(void **p, size_t bytes, cudaStream_t st);
+int32_t fail_alloc(int32_t nth, size_t bytes);  // g2_diag_fail_alloc
 void dfree(void *p, cudaStream_t st);
 template <class T>
 inline cudaError_t dmalloc(T **p, size_t bytes, cudaStream_t st) {

@@ -93,6 +93,7 @@ _SIGS = {
     "g2_last_error": [],
     "g2_selftest_wait_timeout": [I64, P],
     "g2_diag_gather": [P, I64, P, I32, I32, P, I32, ctypes.POINTER(F32), P],
+    "g2_diag_fail_alloc": [I32, I64, ctypes.POINTER(I32)],
     "g2_bfs_csr_static": [I32, I64, P, P, I32, P, P, P],
     "g2_sssp_async": [P, I32, I32, P, P],
     "g2_bfs_async": [P, I32, I32, P, P, P],
@@ -369,6 +370,16 @@ def g2_diag_gather(idx, x, mode, out, grid, stream=None) -> float:
     _check(_lib.g2_diag_gather(_ptr(idx), int(idx.numel()), _ptr(x), n, int(mode), _ptr(out),
                                int(grid), ctypes.byref(ms), _stream(stream)), "g2_diag_gather")
     return ms.value
+
+
+def g2_diag_fail_alloc(nth: int, min_bytes: int = 0) -> int:
+    """Test aid (see include/g2_diag.h): the nth device allocation of at least
+    min_bytes from now on fails, once.  Returns what was left to count of the
+    request before (0: it has happened)."""
+    left = I32()
+    _check(_lib.g2_diag_fail_alloc(int(nth), int(min_bytes), ctypes.byref(left)),
+           "g2_diag_fail_alloc")
+    return left.value
 
 
 # ------------------------------------------------------------- schedules

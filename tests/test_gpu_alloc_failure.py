@@ -1,0 +1,52 @@
+"""Calls on a device without room: each allocation of a call fails in turn.
+The call reports G2_ENOMEM or goes on without that buffer, and the next call on
+the same handle is right."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2012_07990_gb300 import graphgen as gg
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def g2():
+    from paper_2012_07990_gb300 import g2 as m
+    return m
+
+
+def fail_each(g2, dg, call, min_bytes=0):
+    """call(handle) with the first, second, ... of its allocations failing, on a
+    handle of its own each time; yields the handle and whether the call got by."""
+    for nth in range(1, 100):
+        view = dg.view()
+        g2.g2_diag_fail_alloc(nth, min_bytes)
+        status = g2.G2_OK
+        try:
+            call(view)
+        except g2.G2Error as e:
+            status = e.status
+        if g2.g2_diag_fail_alloc(0):        # it makes fewer allocations
+            assert status == g2.G2_OK and nth > 1
+            return
+        assert status in (g2.G2_OK, g2.G2_ENOMEM)
+        yield view, status == g2.G2_OK
+    pytest.fail("a call with 100 allocations")
+
+
+def test_next_call_is_right(g2):
+    g = gg.rmat(10, seed=2)
+    want = oracle.bfs(g.n, g.rowptr, g.col, 3, False)[0]
+    dg = g2.load_graph(g)
+    depth = torch.empty(g.n, dtype=torch.int32, device="cuda")
+
+    def bfs(h):
+        g2.g2_bfs(h, 3, depth, None, g2.schedule("STRICT"))
+
+    for view, ok in fail_each(g2, dg, bfs):
+        if not ok:
+            depth.fill_(-9)
+            bfs(view)
+        assert np.array_equal(depth.cpu().numpy(), want)
