@@ -335,16 +335,10 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         }
         size = g->h_ctr[0];
         produced.size = size;
-        outf->size = outf->format == G2_FRONTIER_SPARSE ? size : -1;
         if (outf->format == G2_FRONTIER_SPARSE && o.rep == OUT_SPARSE && o.q == outf->q) {
             g->settled = true;
         } else if (outf->format == G2_FRONTIER_SPARSE) {
-            if (size > outf->cap) {
-                dfree(outf->q, st);
-                outf->q = nullptr;
-                G2_CK(dmalloc(&outf->q, (size_t)size * 4, st));
-                outf->cap = size;
-            }
+            G2_TRY(frontier_reserve(outf, size, st));
             if (produced.rep == OUT_SPARSE) {
                 if (size > 0)
                     G2_CK(cudaMemcpyAsync(outf->q, produced.q, (size_t)size * 4,
@@ -371,6 +365,7 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         }
     }
     G2_TRY(end_call(g, st, d_err));
+    if (outf) outf->size = outf->format == G2_FRONTIER_SPARSE ? size : -1;
     if (out_size) *out_size = size;
     return G2_OK;
 }

@@ -905,6 +905,18 @@ g2_status pr_prepare_wait(Topology *t) {
     return G2_OK;
 }
 
+g2_status frontier_reserve(g2_frontier *f, int32_t k, cudaStream_t st) {
+    if (k <= f->cap) return G2_OK;
+    // the old list's block goes back first: it may be what the new one needs
+    dfree(f->q, st);
+    f->q = nullptr;
+    f->cap = 0;
+    f->size = 0;
+    G2_CK(dmalloc(&f->q, (size_t)k * 4, st));
+    f->cap = k;
+    return G2_OK;
+}
+
 }  // namespace g2
 
 using namespace g2;
@@ -1247,12 +1259,7 @@ g2_status g2_frontier_set(g2_frontier *f, const int32_t *verts, int32_t k, void 
     if (k > 0) G2_CK(cudaMemcpyAsync(tmp, verts, (size_t)k * 4, cudaMemcpyHostToDevice, st));
     VSet src{OUT_SPARSE, tmp, k, nullptr, nullptr, nullptr, k};
     if (f->format == G2_FRONTIER_SPARSE) {
-        if (k > f->cap) {
-            dfree(f->q, st);
-            f->q = nullptr;
-            G2_CK(dmalloc(&f->q, (size_t)k * 4, st));
-            f->cap = k;
-        }
+        G2_TRY(frontier_reserve(f, k, st));
         if (k > 0) G2_CK(cudaMemcpyAsync(f->q, tmp, (size_t)k * 4, cudaMemcpyDeviceToDevice, st));
         G2_TRY(put_i32(st, {{f->cnt, src.size}}));
     } else {

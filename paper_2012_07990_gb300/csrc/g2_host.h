@@ -316,6 +316,10 @@ struct VSet {
 // Convert a vertexset to the representation `rep` using buffers `dst`
 // (which must not alias the source's live buffer).
 g2_status vset_convert(g2_graph *g, const VSet &src, int rep, VSet &dst, cudaStream_t st);
+// Room for k entries in a SPARSE frontier's list (old contents are not kept
+// when it grows).  Where there is none the frontier is left empty, without a
+// list: its capacity never outlives the list it belongs to.
+g2_status frontier_reserve(g2_frontier *f, int32_t k, cudaStream_t st);
 // Exact member count of a bitmap / boolmap on the device into *d_out.
 g2_status vset_count(g2_graph *g, const VSet &v, int32_t *d_out, cudaStream_t st);
 
