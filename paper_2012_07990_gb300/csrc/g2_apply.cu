@@ -226,7 +226,7 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         G2_TRY(g2_frontier_size(in, &sz, stream));
         vin.size = sz;
         if (in->format == G2_FRONTIER_SPARSE) {
-            vin.rep = OUT_SPARSE; vin.q = in->q; vin.qcap = in->cap; vin.cnt = in->cnt;
+            vin.rep = OUT_SPARSE; vin.q = in->q; vin.qcap = in->cap;
         } else if (in->format == G2_FRONTIER_BITMAP) {
             vin.rep = OUT_BITMAP; vin.bitmap = in->bitmap;
         } else {
@@ -266,12 +266,7 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         if (s.frontier_creation == G2_FUSED) {
             bool dedup = s.dedup == G2_DEDUP_ENABLED;
             size_t cap = dedup ? (size_t)std::max(n, 1) : (size_t)t->m + (size_t)n + 1;
-            // straight into the caller's list where it is not the input's and
-            // has room for every vertex
-            if (dedup && outf->format == G2_FRONTIER_SPARSE && outf != in && outf->cap >= (int32_t)cap)
-                o.q = outf->q;
-            else
-                G2_TRY(ws(g, dedup ? B_Q3 : B_BIG, cap, &o.q));
+            G2_TRY(ws(g, dedup ? B_Q3 : B_BIG, cap, &o.q));
             o.rep = OUT_SPARSE;
             o.qcap = (int32_t)std::min<size_t>(cap, 2147483647u);
             o.cnt = ctrs + 61;
@@ -317,7 +312,6 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         stats().launches += 1;
         a.from = snap;
     }
-    if (outf) outf->size = 0;  // until the call has succeeded
     G2_TRY(apply_round(g, s, a, use, o, st));
     s.direction == G2_PUSH ? stats().push_rounds++ : stats().pull_rounds++;
     stats().iterations = 1;
@@ -325,9 +319,8 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
     int32_t size = 0;
     if (outf) {
         // produced -> caller's representation
+        // (a round that fails leaves `out` as it was, also where it is `in`)
         if (produced.rep == OUT_SPARSE) {
-            if (outf->format == G2_FRONTIER_SPARSE)
-                G2_CK(cudaMemcpyAsync(outf->cnt, o.cnt, 4, cudaMemcpyDeviceToDevice, st));
             G2_TRY(read_counters(g, o.cnt, 1, st, d_err));
         } else {
             G2_TRY(vset_count(g, produced, ctrs + 59, st));
@@ -335,10 +328,18 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
         }
         size = g->h_ctr[0];
         produced.size = size;
-        if (outf->format == G2_FRONTIER_SPARSE && o.rep == OUT_SPARSE && o.q == outf->q) {
+        if (outf->format == G2_FRONTIER_SPARSE && o.rep == OUT_SPARSE && o.q == g->buf[B_Q3]) {
+            // the workspace list, with room for every vertex, becomes the
+            // frontier's and the frontier's old one the workspace's: no copy
+            const size_t bytes = (size_t)outf->cap * 4;
+            g->buf[B_Q3] = outf->q;
+            outf->q = o.q;
+            outf->cap = (int32_t)(g->cap[B_Q3] / 4);
+            g->cap[B_Q3] = bytes;
             g->settled = true;
         } else if (outf->format == G2_FRONTIER_SPARSE) {
             G2_TRY(frontier_reserve(outf, size, st));
+            outf->size = 0;
             if (produced.rep == OUT_SPARSE) {
                 if (size > 0)
                     G2_CK(cudaMemcpyAsync(outf->q, produced.q, (size_t)size * 4,
@@ -347,8 +348,6 @@ extern "C" g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, vo
                 VSet d{OUT_SPARSE, outf->q, outf->cap, outf->cnt, nullptr, nullptr, 0};
                 G2_TRY(vset_convert(g, produced, OUT_SPARSE, d, st));
             }
-            if (o.rep != OUT_SPARSE)
-                G2_CK(cudaMemcpyAsync(outf->cnt, &size, 4, cudaMemcpyHostToDevice, st));
         } else {
             int want = outf->format == G2_FRONTIER_BITMAP ? OUT_BITMAP : OUT_BOOLMAP;
             VSet d{want, nullptr, 0, nullptr, outf->bitmap, outf->boolmap, 0};

@@ -1253,15 +1253,14 @@ g2_status g2_frontier_set(g2_frontier *f, const int32_t *verts, int32_t k, void 
         if (verts[i] < 0 || verts[i] >= n) return fail(G2_EINVAL, "vertex id out of range");
     cudaStream_t st = as_stream(stream);
     g->st = st;
-    f->size = 0;  // until the call has succeeded
     int32_t *tmp;
     G2_TRY(ws(g, B_I1, (size_t)std::max(k, 1), &tmp));
+    f->size = 0;  // from here until the call has succeeded
     if (k > 0) G2_CK(cudaMemcpyAsync(tmp, verts, (size_t)k * 4, cudaMemcpyHostToDevice, st));
     VSet src{OUT_SPARSE, tmp, k, nullptr, nullptr, nullptr, k};
     if (f->format == G2_FRONTIER_SPARSE) {
         G2_TRY(frontier_reserve(f, k, st));
         if (k > 0) G2_CK(cudaMemcpyAsync(f->q, tmp, (size_t)k * 4, cudaMemcpyDeviceToDevice, st));
-        G2_TRY(put_i32(st, {{f->cnt, src.size}}));
     } else {
         VSet dst{f->format == G2_FRONTIER_BITMAP ? (int)OUT_BITMAP : (int)OUT_BOOLMAP, nullptr, 0,
                  nullptr, f->bitmap, f->boolmap, 0};
@@ -1281,16 +1280,12 @@ g2_status g2_frontier_size(g2_frontier *f, int32_t *size, void *stream) {
         *size = f->size;
         return G2_OK;
     }
-    if (f->format == G2_FRONTIER_SPARSE) {
-        G2_CK(cudaMemcpyAsync(g->h_ctr, f->cnt, 4, cudaMemcpyDeviceToHost, st));
-    } else {
-        VSet v{f->format == G2_FRONTIER_BITMAP ? (int)OUT_BITMAP : (int)OUT_BOOLMAP, nullptr, 0,
-               nullptr, f->bitmap, f->boolmap, 0};
-        int32_t *d;
-        G2_TRY(ws(g, B_CTR, 64, &d));
-        G2_TRY(vset_count(g, v, d + 32, st));
-        G2_CK(cudaMemcpyAsync(g->h_ctr, d + 32, 4, cudaMemcpyDeviceToHost, st));
-    }
+    VSet v{f->format == G2_FRONTIER_BITMAP ? (int)OUT_BITMAP : (int)OUT_BOOLMAP, nullptr, 0, nullptr,
+           f->bitmap, f->boolmap, 0};
+    int32_t *d;
+    G2_TRY(ws(g, B_CTR, 64, &d));
+    G2_TRY(vset_count(g, v, d + 32, st));
+    G2_CK(cudaMemcpyAsync(g->h_ctr, d + 32, 4, cudaMemcpyDeviceToHost, st));
     G2_CK(cudaStreamSynchronize(st));
     *size = f->size = g->h_ctr[0];
     return G2_OK;

@@ -80,10 +80,10 @@ struct g2_frontier {
     int32_t format;
     int32_t *q;       // SPARSE: list (capacity cap)
     int32_t cap;
-    int32_t *cnt;     // device int32 length (SPARSE)
+    int32_t *cnt;     // SPARSE: device counter of a conversion into the list
     uint32_t *bitmap; // BITMAP
     uint8_t *boolmap; // BOOLMAP
-    int32_t size;     // members as the host knows them (-1: to be counted on the device)
+    int32_t size;     // members; -1: to be counted on the device (never for SPARSE)
 };
 
 namespace g2 {
