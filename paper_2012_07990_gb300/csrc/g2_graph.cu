@@ -479,14 +479,18 @@ void dfree(void *p, cudaStream_t st) {
     cudaFreeAsync(p, st);
 }
 
+void ws_release(g2_graph *g, Buf b) {
+    // the block may still be read by work queued on g->st: its release is
+    // ordered after that work
+    dfree(g->buf[b], g->st);
+    g->buf[b] = nullptr;
+    g->cap[b] = 0;
+}
+
 g2_status ws_get(g2_graph *g, Buf b, size_t bytes, void **out) {
     if (bytes == 0) bytes = 16;
     if (g->cap[b] < bytes) {
-        // the old block may still be read by work queued on g->st: its
-        // release is ordered after that work
-        if (g->buf[b]) dfree(g->buf[b], g->st);
-        g->buf[b] = nullptr;
-        g->cap[b] = 0;
+        ws_release(g, b);
         void *p = nullptr;
         cudaError_t e = dmalloc_bytes(&p, bytes, g->st);
         if (e != cudaSuccess) return cuda_fail(e, "workspace allocation");

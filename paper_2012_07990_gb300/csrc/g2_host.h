@@ -188,6 +188,9 @@ inline g2_status ws(g2_graph *g, Buf b, size_t count, T **out) {
     return ws_get(g, b, count * sizeof(T), reinterpret_cast<void **>(out));
 }
 
+// Slot b's buffer back to the pool (ordered on g->st).
+void ws_release(g2_graph *g, Buf b);
+
 // Stream helpers.
 inline cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 g2_status sync_and_check(g2_graph *g, cudaStream_t st, int32_t *d_err);

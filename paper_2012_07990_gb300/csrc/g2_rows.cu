@@ -353,14 +353,16 @@ static g2_status max_weight(g2_graph *g, int32_t *d_tmp, cudaStream_t st, int32_
 }
 
 template <int K>
-static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist, int32_t *D,
+static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist,
                           cudaStream_t st, int32_t *d_err, bool *done) {
     Topology *t = g->topo;
     const int32_t n = t->n, m = t->m;
     const int32_t words = (n + 31) / 32, cap = std::max(n / 32, 1);
     int32_t *ctrs = d_err - 62;
     uint32_t *flags[2];
-    int32_t *list, *deg, *scan, *dsrc;
+    int32_t *D, *list, *deg, *scan, *dsrc;
+    G2_TRY(ws(g, B_ROWS, (size_t)n * K, &D));
+    G2_TRY(ensure_coo(g, st));
     G2_TRY(ws(g, B_BM0, (size_t)words + 1, &flags[0]));
     G2_TRY(ws(g, B_BM1, (size_t)words + 1, &flags[1]));
     G2_TRY(ws(g, B_Q0, (size_t)n, &list));
@@ -383,11 +385,7 @@ static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *
         G2_TRY(read_counters(g, ctrs, 1, st, d_err));
         const int32_t size = g->h_ctr[0];
         if (size == 0) break;
-        if (stats().iterations == kRowRounds) {
-            G2_CK(cudaMemsetAsync(ctrs, 0, 4, st));
-            stats().iterations = stats().push_rounds = 0;
-            return G2_OK;
-        }
+        if (stats().iterations == kRowRounds) return G2_OK;
         // the line: a sweep reads the source id of every arc (RMAT-21: 0.36 ms
         // with 8% of the vertices flagged), a list of fewer than 1/32 of the
         // vertices takes 0.05 ms, 0.25 ms where it holds the hubs
@@ -421,24 +419,21 @@ static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *
 }
 
 // Shortest distances of k sources over rows; *done is false where the form
-// does not apply (no arcs, no memory for the rows and the arcs' source ids
-// beside what the device already holds, or more than kRowRounds rounds).
+// does not apply (no arcs, no memory for the rows, the arcs' source ids or the
+// lists beside what the device already holds, or more than kRowRounds rounds).
+// The rows' memory is given back then: what runs instead needs its own.
 g2_status sssp_batch_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist,
                           cudaStream_t st, int32_t *d_err, bool *done) {
-    Topology *t = g->topo;
     *done = false;
-    if (t->m == 0) return G2_OK;
-    const int K = k <= 8 ? 8 : k <= 16 ? 16 : 32;
-    int32_t *D;
-    const g2_status have = ws(g, B_ROWS, (size_t)t->n * K, &D);
-    if (have == G2_ENOMEM) return G2_OK;
-    G2_TRY(have);
-    const g2_status coo = ensure_coo(g, st);
-    if (coo == G2_ENOMEM) return G2_OK;
-    G2_TRY(coo);
-    return K == 8    ? run_rows<8>(g, srcs, k, dist, D, st, d_err, done)
-           : K == 16 ? run_rows<16>(g, srcs, k, dist, D, st, d_err, done)
-                     : run_rows<32>(g, srcs, k, dist, D, st, d_err, done);
+    if (g->topo->m == 0) return G2_OK;
+    const g2_status r = k <= 8    ? run_rows<8>(g, srcs, k, dist, st, d_err, done)
+                        : k <= 16 ? run_rows<16>(g, srcs, k, dist, st, d_err, done)
+                                  : run_rows<32>(g, srcs, k, dist, st, d_err, done);
+    if (*done || (r != G2_OK && r != G2_ENOMEM)) return r;
+    ws_release(g, B_ROWS);
+    G2_CK(cudaMemsetAsync(d_err - 62, 0, 4, st));  // the counter that run_rows used
+    stats().iterations = stats().push_rounds = 0;
+    return G2_OK;
 }
 
 }  // namespace g2

@@ -50,3 +50,28 @@ def test_next_call_is_right(g2):
             depth.fill_(-9)
             bfs(view)
         assert np.array_equal(depth.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("k", [1, 9, 32])
+def test_sssp_batch_goes_on_without_rows(g2, k):
+    """The tuned multi-source SSSP survives each single failed allocation: it
+    goes on without the distance rows."""
+    g = gg.rmat(10, seed=3)
+    w = gg.pair_weights(g, 255, seed=1)
+    srcs = np.random.default_rng(k).integers(0, g.n, k).astype(np.int32)
+    want = np.stack([oracle.sssp(g.n, g.rowptr, g.col, w, int(s)) for s in srcs])
+    dist = torch.empty((k, g.n), dtype=torch.int32, device="cuda")
+    failed = []
+    for nth in range(1, 40):
+        dg = g2.load_graph(g, w)
+        dist.fill_(-9)
+        g2.g2_diag_fail_alloc(nth)
+        g2.g2_sssp_batch(dg, srcs, 64, dist)
+        left = g2.g2_diag_fail_alloc(0)
+        assert np.array_equal(dist.cpu().numpy(), want), nth
+        if left:
+            break
+        failed.append(nth)
+        g2.g2_sssp_batch(dg, srcs, 64, dist)
+        assert np.array_equal(dist.cpu().numpy(), want), nth
+    assert len(failed) >= 8       # counters, rows, sources of the arcs, flags, list, degrees, scan
