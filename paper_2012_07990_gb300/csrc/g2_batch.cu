@@ -53,7 +53,8 @@ struct OpMsBfs {
 // that a round writes 8 bytes a plane and vertex, and k_ms_out writes every
 // depth once, in order.  (Written to depth[b][v] round by round, the 64 arrays
 // took 446 us of RMAT-21's rounds in part lines, beside 80 us to clear them.)
-// A search of more levels goes on writing its depths directly.
+// A search of more levels goes on writing its depths directly, and so does one
+// without room for the planes.
 constexpr int kMsPlanes = 5;  // depths up to 31
 struct MsLevels {
     u64 *plane[kMsPlanes];
@@ -461,17 +462,19 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
     G2_CK(cudaMemsetAsync(F[0], 0, (size_t)n * 8, st));
     G2_CK(cudaMemsetAsync(F[1], 0, (size_t)n * 8, st));
     MsLevels lv;
-    u64 *planes;
-    G2_TRY(ws(g, B_ROWS, (size_t)kMsPlanes * std::max(n, 1), &planes));
+    u64 *planes = nullptr;
+    const g2_status room = ws(g, B_ROWS, (size_t)kMsPlanes * std::max(n, 1), &planes);
+    if (room != G2_ENOMEM) G2_TRY(room);
     for (int j = 0; j < kMsPlanes; ++j) lv.plane[j] = planes + (size_t)j * n;
-    lv.depth = nullptr;
+    lv.depth = planes ? nullptr : depth;  // without room for planes: written directly
+    if (lv.depth) G2_CK(cudaMemsetAsync(depth, 0xFF, (size_t)k * n * 4, st));
     lv.n = n;
     int nplanes = 0;  // cleared so far
     G2_TRY(put_array(dsrc, srcs, k, st));
     // ctrs: [0..1] list lengths, [2] big vertices, [3] a pull's rest, [8..11] active masks of the
     // even and odd levels (all zero at the start of the call)
     u64 *active[2] = {reinterpret_cast<u64 *>(ctrs + 8), reinterpret_cast<u64 *>(ctrs + 10)};
-    k_ms_seed<<<1, 64, 0, st>>>(dsrc, k, visit, F[0], nullptr, n, list[0], ctrs + 0);
+    k_ms_seed<<<1, 64, 0, st>>>(dsrc, k, visit, F[0], lv.depth, n, list[0], ctrs + 0);
     const u64 full = k == 64 ? ~0ull : ((1ull << k) - 1);
     G2_TRY(put_i32(st, {{ctrs + 8, (int32_t)(uint32_t)full}, {ctrs + 9, (int32_t)(uint32_t)(full >> 32)}}));
     stats().launches += 1;

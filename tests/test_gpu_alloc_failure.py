@@ -75,3 +75,17 @@ def test_sssp_batch_goes_on_without_rows(g2, k):
         g2.g2_sssp_batch(dg, srcs, 64, dist)
         assert np.array_equal(dist.cpu().numpy(), want), nth
     assert len(failed) >= 8       # counters, rows, sources of the arcs, flags, list, degrees, scan
+
+
+@pytest.mark.parametrize("k", [1, 33, 64])
+def test_bfs_batch_goes_on_without_planes(g2, k):
+    g = gg.rmat(10, seed=3)
+    srcs = np.random.default_rng(k).integers(0, g.n, k).astype(np.int32)
+    want = np.stack([oracle.bfs(g.n, g.rowptr, g.col, int(s), False)[0] for s in srcs])
+    dg = g2.load_graph(g)
+    depth = torch.empty((k, g.n), dtype=torch.int32, device="cuda")
+    depth.fill_(-9)
+    g2.g2_diag_fail_alloc(1, 40 * g.n)       # the planes: no other buffer is as large
+    g2.g2_bfs_batch(dg, srcs, depth)
+    assert g2.g2_diag_fail_alloc(0) == 0
+    assert np.array_equal(depth.cpu().numpy(), want)
