@@ -138,7 +138,7 @@ __global__ void __launch_bounds__(kCta) k_rows_sweep(const int32_t *__restrict__
                                                      const int32_t *__restrict__ col,
                                                      const int32_t *__restrict__ w, int32_t m,
                                                      int32_t *D, const uint32_t *__restrict__ cur,
-                                                     uint32_t *next) {
+                                                     uint32_t *next, unsigned long long *ctr) {
     constexpr int F = kRowFlight, G = 32 / K;
     static_assert(F == 8, "two 16-byte loads");
     const int lane = threadIdx.x & 31, sl = lane % K, gi = lane / K;
@@ -156,6 +156,7 @@ __global__ void __launch_bounds__(kCta) k_rows_sweep(const int32_t *__restrict__
         const unsigned act =
             __ballot_sync(G2_FULL, ul >= 0 && ((cur[ul >> 5] >> (ul & 31)) & 1u));
         if (act == 0) continue;
+        count_arcs(ctr, (act >> lane) & 1u);
 #pragma unroll 1
         for (int s = gi * F; s < 32; s += G * F) {
             const unsigned on = (act >> s) & 255u;
@@ -205,8 +206,8 @@ __global__ void __launch_bounds__(kCta) k_rows_sweep(const int32_t *__restrict__
 // the entry i with scan[i] <= k < scan[i + 1].
 template <int K>
 __global__ void __launch_bounds__(kCta) k_rows_push(DevGraph g, const int32_t *list, int32_t size,
-                                                    const int32_t *scan, int32_t *D,
-                                                    uint32_t *next) {
+                                                    const int32_t *scan, int32_t *D, uint32_t *next,
+                                                    unsigned long long *ctr) {
     constexpr int F = kRowFlight, G = 32 / K;
     const int lane = threadIdx.x & 31, sl = lane % K, gi = lane / K;
     const unsigned group = K == 32 ? G2_FULL : ((1u << K % 32) - 1u) << (gi * K);
@@ -216,6 +217,7 @@ __global__ void __launch_bounds__(kCta) k_rows_push(DevGraph g, const int32_t *l
     const int32_t total = scan[size];
     for (int64_t t0 = gw * kRowTile; t0 < total; t0 += nw * kRowTile) {
         const int32_t len = (int32_t)(total - t0 < kRowTile ? total - t0 : kRowTile);
+        count_arcs(ctr, lane == 0 ? len : 0);
         const int32_t own = scan_owner(scan, size, (int32_t)t0);
         if (len == kRowTile && scan[own + 1] >= t0 + kRowTile) {
             // the whole tile belongs to one vertex
@@ -375,6 +377,8 @@ static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *
     k_rows_seed<<<1, 32, 0, st>>>(dsrc, k, K, D, flags[0]);
     stats().launches += 2;
     const int sweep = grid_for(g, m, kCta);
+    unsigned long long *ctr = nullptr;
+    if (count_arcs_enabled()) G2_TRY(ws(g, B_ARCS, 2, &ctr));
     int p = 0;
     for (;; p ^= 1) {
         // (all counters are zero at the start of the call)
@@ -393,11 +397,11 @@ static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *
             k_rows_degrees<<<grid_for(g, size, kCta), kCta, 0, st>>>(t->rowptr, list, size, deg);
             G2_TRY(exclusive_scan_i32(g, deg, scan, size, st));
             k_rows_push<K><<<t->sm_count * 8, kCta, 0, st>>>(t->view(), list, size, scan, D,
-                                                           flags[p ^ 1]);
+                                                           flags[p ^ 1], ctr);
             stats().launches += 2;
         } else {
             k_rows_sweep<K><<<sweep, kCta, 0, st>>>(t->coo_src, t->col, t->w, m, D, flags[p],
-                                                 flags[p ^ 1]);
+                                                 flags[p ^ 1], ctr);
             stats().launches += 1;
         }
         stats().push_rounds++;
