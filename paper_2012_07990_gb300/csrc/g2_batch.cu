@@ -795,6 +795,32 @@ __global__ void k_msr_seed(const int32_t *srcs, int32_t k, int32_t *dist, int32_
     }
 }
 
+// Going on from distance rows: every flagged vertex waits with each source that
+// has reached it (which of them changed last is not known).
+__global__ void k_msr_resume(const uint32_t *flags, int32_t words, const int32_t *dist, int32_t n,
+                             int32_t k, unsigned *mask, int32_t *list, int32_t *cnt) {
+    const int lane = threadIdx.x & 31;
+    const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = gw; i < words; i += nw) {
+        const uint32_t x = flags[i];
+        if (x == 0) continue;
+        const int64_t v = i * 32 + lane;
+        const bool on = (x >> lane) & 1u;
+        unsigned m = 0;
+        if (on)
+            for (int32_t b = 0; b < k; ++b)
+                if (dist[(int64_t)b * n + v] != G2_INF32) m |= 1u << b;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(cnt, __popc(x));
+        base = __shfl_sync(G2_FULL, base, 0);
+        if (on) {
+            mask[v] = m;
+            list[base + __popc(x & lanemask_lt())] = (int32_t)v;
+        }
+    }
+}
+
 __global__ void k_msr_clear(const int32_t *list, int32_t cnt, unsigned *m) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
          i += (int64_t)gridDim.x * blockDim.x)
@@ -855,8 +881,11 @@ static g2_status sssp_batch_fused(g2_graph *g, const int32_t *srcs, int32_t k, i
     return G2_OK;
 }
 
+// `left` (may be null): dist holds distances already, and the arcs of the
+// vertices flagged there are still to be relaxed.
 g2_status sssp_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t delta, int32_t *dist,
-                         const g2_hybrid &h, cudaStream_t st, int32_t *d_err) {
+                         const g2_hybrid &h, const uint32_t *left, cudaStream_t st,
+                         int32_t *d_err) {
     if (h.s1.kernel_fusion) {
         if (h.criteria != G2_CRITERIA_NONE && !h.s2.kernel_fusion)
             return fail(G2_EUNSUPPORTED, "kernel fusion must be set on both hybrid schedules");
@@ -878,19 +907,30 @@ g2_status sssp_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t de
     G2_CK(cudaMemsetAsync(M[0], 0, (size_t)n * 4, st));
     G2_CK(cudaMemsetAsync(M[1], 0, (size_t)n * 4, st));
     G2_CK(cudaMemsetAsync(far, 0, (size_t)n * 4, st));
-    k_fill_i32_b<<<grid_for(g, (int64_t)k * n, kCta), kCta, 0, st>>>(dist, (int64_t)k * n, G2_INF32);
-    G2_TRY(put_array(dsrc, srcs, k, st));
-    k_msr_seed<<<1, 32, 0, st>>>(dsrc, k, dist, n, M[0], nl[0], ctrs + 0);
-    stats().launches += 2;
+    const bool bucketed = delta > 0;
+    int64_t T = bucketed ? delta : (int64_t)G2_INF32;
+    // (all counters are zero here)
+    if (left) {
+        // no bucket is settled yet: what waits is the far pile, to be split at
+        // the first threshold
+        const int32_t words = (n + 31) / 32;
+        if (bucketed) T = 0;
+        k_msr_resume<<<grid_for(g, words, kWarps), kCta, 0, st>>>(
+            left, words, dist, n, k, bucketed ? far : M[0], bucketed ? fl[0] : nl[0],
+            bucketed ? ctrs + 4 : ctrs);
+        stats().launches += 1;
+    } else {
+        k_fill_i32_b<<<grid_for(g, (int64_t)k * n, kCta), kCta, 0, st>>>(dist, (int64_t)k * n,
+                                                                       G2_INF32);
+        G2_TRY(put_array(dsrc, srcs, k, st));
+        k_msr_seed<<<1, 32, 0, st>>>(dsrc, k, dist, n, M[0], nl[0], ctrs + 0);
+        stats().launches += 2;
+    }
     G2_TRY(read_counters(g, ctrs, 8, st, d_err));
     int32_t size = g->h_ctr[0];
     unsigned long long *ctr = nullptr;
     if (count_arcs_enabled()) G2_TRY(ws(g, B_ARCS, 2, &ctr));
-    const DevGraph dg = t->view();
-    const bool bucketed = delta > 0;
-    int64_t T = bucketed ? delta : (int64_t)G2_INF32;
     int p = 0, fp = 0;
-    G2_CK(cudaMemsetAsync(ctrs + 4, 0, 8, st));
     for (;;) {
         while (size > 0) {
             const g2_schedule &s = pick_schedule(h, size, n);
@@ -910,8 +950,10 @@ g2_status sssp_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t de
             out.err = d_err;
             G2_CK(cudaMemsetAsync(ctrs + q, 0, 4, st));
             VSet in{OUT_SPARSE, nl[p], n, ctrs + p, nullptr, nullptr, size};
+            // distances that rows left may still fall: the overflow rule is
+            // applied to the final ones (sssp_batch_check)
             OpMsRelax op{dist, t->w, M[p], M[q], far, n, (int32_t)std::min<int64_t>(T, G2_INF32),
-                         d_err};
+                         left ? nullptr : d_err};
             G2_TRY(push_round(g, s, op, in, out, ctr, st));
             k_msr_clear<<<grid_for(g, size, kCta), kCta, 0, st>>>(nl[p], size, M[p]);
             stats().launches += 2;
@@ -1125,11 +1167,16 @@ g2_status g2_sssp_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t del
     if (!sched && !h.s1.kernel_fusion) {
         // rows of distances (RMAT-21, 32 sources: 8.2 ms against 42.7 ms for
         // STRICT delta-stepping over stacked arrays)
-        bool done = false;
-        G2_TRY(sssp_batch_rows(g, srcs, k, dist, st, d_err, &done));
-        if (done) return end_call(g, st, d_err);
+        int how;
+        const uint32_t *left;
+        G2_TRY(sssp_batch_rows(g, srcs, k, dist, st, d_err, &how, &left));
+        if (how == ROWS_LEFT) {
+            G2_TRY(sssp_batch_run(g, srcs, k, delta, dist, h, left, st, d_err));
+            G2_TRY(sssp_batch_check(g, dist, k, st, d_err));
+        }
+        if (how != ROWS_NONE) return end_call(g, st, d_err);
     }
-    G2_TRY(sssp_batch_run(g, srcs, k, delta, dist, h, st, d_err));
+    G2_TRY(sssp_batch_run(g, srcs, k, delta, dist, h, nullptr, st, d_err));
     return end_call(g, st, d_err);
 }
 

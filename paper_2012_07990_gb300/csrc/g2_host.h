@@ -249,10 +249,14 @@ g2_status pagerank_blk_run(g2_graph *g, float damping, int32_t iters, float *ran
 g2_status pr_prepare_start(g2_graph *g, cudaStream_t load_stream);
 g2_status pr_prepare_wait(Topology *t);
 
-// Multi-source SSSP over distance rows (g2_rows.cu); *done tells whether the
-// form applied.
+// Multi-source SSSP over distance rows (g2_rows.cu); *how tells what is left to
+// do, *left where to go on.
+enum { ROWS_DONE, ROWS_NONE, ROWS_LEFT };
 g2_status sssp_batch_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist,
-                          cudaStream_t st, int32_t *d_err, bool *done);
+                          cudaStream_t st, int32_t *d_err, int *how, const uint32_t **left);
+// The overflow rule on the distances of a batch that went on from rows.
+g2_status sssp_batch_check(g2_graph *g, const int32_t *dist, int32_t k, cudaStream_t st,
+                           int32_t *d_err);
 
 // Largest out-degree of the graph (computed on the device once, then kept).
 g2_status max_out_degree(g2_graph *g, cudaStream_t st, int32_t *out);

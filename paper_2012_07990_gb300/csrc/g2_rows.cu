@@ -40,8 +40,9 @@ namespace g2 {
 constexpr int kRowTile = 128;   // arcs of a list that a warp takes at a time
 constexpr int kRowFlight = 8;   // rows in flight per lane
 // Rounds without buckets repeat work where paths are long (a road network with
-// a hub): power-law graphs take 12-15 rounds, and a batch that has not ended
-// after this many starts over with the near/far queue.
+// a hub): power-law graphs take 12-15 rounds.  A batch that has not ended after
+// this many goes on with the near/far queue, from the distances found so far
+// and the vertices that are flagged.
 constexpr int kRowRounds = 32;
 
 __global__ void k_rows_fill(int32_t *D, int64_t count4) {
@@ -317,23 +318,24 @@ __global__ void __launch_bounds__(kCta) k_rows_out(const int32_t *__restrict__ D
 }
 
 // error G2_EOVERFLOW if an arc out of a reached vertex leads to INT32_MAX or beyond
-template <int K>
-__global__ void k_rows_check(const int32_t *row, const int32_t *w, int32_t m, const int32_t *D,
-                             int32_t *err) {
-    const int64_t total = (int64_t)m * K;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t e = i / K;
-        const int32_t d = D[(int64_t)row[e] * K + i % K];
-        if (d != G2_INF32 && (int64_t)d + w[e] >= G2_INF32) set_error(err, G2_EOVERFLOW);
-    }
+__global__ void k_rows_check(const int32_t *row, const int32_t *w, int32_t m, const int32_t *dist,
+                             int32_t n, int32_t k, int32_t *err) {
+    for (int32_t i = 0; i < k; ++i)
+        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+             e += (int64_t)gridDim.x * blockDim.x) {
+            const int32_t d = dist[(int64_t)i * n + row[e]];
+            if (d != G2_INF32 && (int64_t)d + w[e] >= G2_INF32) set_error(err, G2_EOVERFLOW);
+        }
 }
 
-__global__ void k_max_i32(const int32_t *a, int32_t n, int32_t *out) {
+// the largest of a[0, n) that is not `skip`
+__global__ void k_max_i32(const int32_t *a, int64_t n, int32_t skip, int32_t *out) {
     int32_t best = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        best = max(best, a[i]);
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t x = a[i];
+        if (x != skip) best = max(best, x);
+    }
     best = __reduce_max_sync(G2_FULL, best);
     if ((threadIdx.x & 31) == 0 && best > 0) atomicMax(out, best);
 }
@@ -345,7 +347,7 @@ static g2_status max_weight(g2_graph *g, int32_t *d_tmp, cudaStream_t st, int32_
     std::lock_guard<std::recursive_mutex> lk(t->layout_mu);
     if (t->max_w < 0) {
         G2_CK(cudaMemsetAsync(d_tmp, 0, 4, st));
-        k_max_i32<<<grid_for(g, t->m, kCta * 4), kCta, 0, st>>>(t->w, t->m, d_tmp);
+        k_max_i32<<<grid_for(g, t->m, kCta * 4), kCta, 0, st>>>(t->w, t->m, -1, d_tmp);
         stats().launches += 1;
         G2_TRY(read_counters(g, d_tmp, 1, st, d_err));
         t->max_w = g->h_ctr[0];
@@ -354,9 +356,36 @@ static g2_status max_weight(g2_graph *g, int32_t *d_tmp, cudaStream_t st, int32_
     return G2_OK;
 }
 
+// The overflow rule on final distances, the largest finite of which is dmax.
+static g2_status check_overflow(g2_graph *g, const int32_t *dist, int32_t k, int32_t dmax,
+                                int32_t wmax, cudaStream_t st, int32_t *d_err) {
+    Topology *t = g->topo;
+    if ((int64_t)dmax + wmax < G2_INF32) return G2_OK;
+    k_rows_check<<<grid_for(g, t->m, kCta), kCta, 0, st>>>(t->coo_src, t->w, t->m, dist, t->n, k, d_err);
+    G2_CK(cudaGetLastError());
+    stats().launches += 1;
+    return G2_OK;
+}
+
+// For a batch that went on from rows: they drop a distance of INT32_MAX or
+// beyond without a word, so the rule is applied to what the batch ended with.
+g2_status sssp_batch_check(g2_graph *g, const int32_t *dist, int32_t k, cudaStream_t st,
+                           int32_t *d_err) {
+    const int64_t count = (int64_t)k * g->topo->n;
+    int32_t *ctrs = d_err - 62, wmax = 0;
+    G2_TRY(max_weight(g, ctrs + 1, st, d_err, &wmax));
+    G2_CK(cudaMemsetAsync(ctrs + 1, 0, 4, st));
+    k_max_i32<<<grid_for(g, count, kCta * 4), kCta, 0, st>>>(dist, count, G2_INF32, ctrs + 1);
+    stats().launches += 1;
+    G2_TRY(read_counters(g, ctrs + 1, 1, st, d_err));
+    return check_overflow(g, dist, k, g->h_ctr[0], wmax, st, d_err);
+}
+
+// *left: null where the batch ended, else the flags of the vertices whose arcs
+// are still to be relaxed from the distances in dist.
 template <int K>
 static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist,
-                          cudaStream_t st, int32_t *d_err, bool *done) {
+                          cudaStream_t st, int32_t *d_err, const uint32_t **left) {
     Topology *t = g->topo;
     const int32_t n = t->n, m = t->m;
     const int32_t words = (n + 31) / 32, cap = std::max(n / 32, 1);
@@ -389,7 +418,10 @@ static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *
         G2_TRY(read_counters(g, ctrs, 1, st, d_err));
         const int32_t size = g->h_ctr[0];
         if (size == 0) break;
-        if (stats().iterations == kRowRounds) return G2_OK;
+        if (stats().iterations == kRowRounds) {
+            *left = flags[p];
+            break;
+        }
         // the line: a sweep reads the source id of every arc (RMAT-21: 0.36 ms
         // with 8% of the vertices flagged), a list of fewer than 1/32 of the
         // vertices takes 0.05 ms, 0.25 ms where it holds the hubs
@@ -408,35 +440,42 @@ static g2_status run_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *
         stats().iterations++;
     }
     int32_t wmax = 0;
-    G2_TRY(max_weight(g, ctrs + 1, st, d_err, &wmax));
+    if (!*left) G2_TRY(max_weight(g, ctrs + 1, st, d_err, &wmax));
     G2_CK(cudaMemsetAsync(ctrs + 1, 0, 4, st));
     k_rows_out<K><<<grid_for(g, n, kCta), kCta, 0, st>>>(D, n, k, dist, ctrs + 1);
     stats().launches += 1;
     G2_TRY(read_counters(g, ctrs + 1, 1, st, d_err));
-    if ((int64_t)g->h_ctr[0] + wmax >= G2_INF32) {
-        k_rows_check<K><<<grid_for(g, (int64_t)m * K, kCta), kCta, 0, st>>>(t->coo_src, t->w, m, D,
-                                                                         d_err);
-        stats().launches += 1;
-    }
-    *done = true;
-    return G2_OK;
+    return *left ? G2_OK : check_overflow(g, dist, k, g->h_ctr[0], wmax, st, d_err);
 }
 
-// Shortest distances of k sources over rows; *done is false where the form
-// does not apply (no arcs, no memory for the rows, the arcs' source ids or the
-// lists beside what the device already holds, or more than kRowRounds rounds).
-// The rows' memory is given back then: what runs instead needs its own.
+// Shortest distances of k sources over rows.  *how says what is left to do:
+// nothing (ROWS_DONE); everything, where the form does not apply (ROWS_NONE: no
+// arcs, or no memory for the rows, the arcs' source ids or the lists beside
+// what the device already holds); or the rest, after kRowRounds rounds
+// (ROWS_LEFT: dist holds distances, and the arcs of the vertices flagged in
+// *left are still to be relaxed).  The rows' memory is given back unless the
+// batch is done: what runs next needs its own.
 g2_status sssp_batch_rows(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dist,
-                          cudaStream_t st, int32_t *d_err, bool *done) {
-    *done = false;
+                          cudaStream_t st, int32_t *d_err, int *how, const uint32_t **left) {
+    *how = ROWS_NONE;
+    *left = nullptr;
     if (g->topo->m == 0) return G2_OK;
-    const g2_status r = k <= 8    ? run_rows<8>(g, srcs, k, dist, st, d_err, done)
-                        : k <= 16 ? run_rows<16>(g, srcs, k, dist, st, d_err, done)
-                                  : run_rows<32>(g, srcs, k, dist, st, d_err, done);
-    if (*done || (r != G2_OK && r != G2_ENOMEM)) return r;
+    const g2_status r = k <= 8    ? run_rows<8>(g, srcs, k, dist, st, d_err, left)
+                        : k <= 16 ? run_rows<16>(g, srcs, k, dist, st, d_err, left)
+                                  : run_rows<32>(g, srcs, k, dist, st, d_err, left);
+    if (r == G2_OK && !*left) {
+        *how = ROWS_DONE;
+        return G2_OK;
+    }
+    if (r != G2_OK && r != G2_ENOMEM) return r;
     ws_release(g, B_ROWS);
-    G2_CK(cudaMemsetAsync(d_err - 62, 0, 4, st));  // the counter that run_rows used
-    stats().iterations = stats().push_rounds = 0;
+    G2_CK(cudaMemsetAsync(d_err - 62, 0, 8, st));  // the counters that run_rows used
+    if (r == G2_OK) {
+        *how = ROWS_LEFT;
+    } else {
+        *left = nullptr;
+        stats().iterations = stats().push_rounds = 0;
+    }
     return G2_OK;
 }
 
