@@ -126,3 +126,16 @@ def test_overflow_is_told_in_either_form(g2, tail, last, over, delta):
         want[[0, 1, 40]] = [1, 0, last + 1]
         want[41:] = 2 + np.arange(tail)
         assert np.array_equal(dist.cpu().numpy()[0], want)
+
+
+@pytest.mark.parametrize("k", [1, 5, 32])
+@pytest.mark.parametrize("delta", [0, 300])
+def test_frontier_that_does_not_fall(g2, k, delta):
+    """A band 50 hops across: given up at the look, with most vertices flagged."""
+    rng = np.random.default_rng(6)
+    i = np.repeat(np.arange(4000), 20)
+    j = i + rng.integers(1, 80, i.size)
+    g = gg.from_arcs(4000, i[j < 4000], j[j < 4000])
+    srcs = rng.integers(0, g.n, k).astype(np.int32)
+    srcs[0] = 0
+    run(g2, g, gg.pair_weights(g, 255, seed=2), srcs, delta)
