@@ -162,12 +162,15 @@ __device__ bool fused_strict_scan(const DevGraph &g, const int32_t *q, int32_t s
 // number, in lane 0, the result.  The chain of depth, row offsets, id and frontier
 // bit is what bounds it, so a warp takes W words at once and a lane has W of them
 // in flight: the whole search of RMAT-22 from the hub 191 us with one, 173 with
-// two, 156 with four, 177 with eight (registers).  Taking one at a time where
-// there are fewer than four words per warp gains nothing in the same kernel
-// (RMAT-14: 63 us both ways).
+// two, 156 with four, 177 with eight (registers).  The grid's warps take turns
+// across the CTAs, so that a graph of fewer words than the warps could take
+// keeps every SM at work, and such a graph is taken one word at a time: 100,000
+// vertices of out-degree about 48, 60 hops across, 0.64 ms; 0.90 with four, 2.26 with
+// four and neighbouring shares in one CTA, 0.77 with one and those.
+template <int W>
 __device__ __forceinline__ int32_t pull_level(const FusedDoBfsArgs &a, const uint32_t *cur, int d,
-                                              int64_t gwarp, int64_t nwarps) {
-    constexpr int W = 4;
+                                              int64_t nwarps) {
+    const int64_t gwarp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const int lane = threadIdx.x & 31;
     const int32_t n = a.g.n;
     uint32_t *next = a.bm[(d + 1) & 1];
@@ -343,7 +346,8 @@ __global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             }
             // bottom-up over every vertex; the next level as a bitmap
-            const int32_t found = pull_level(a, cur, d, gwarp, nwarps);
+            const int32_t found = words < 4 * nwarps ? pull_level<1>(a, cur, d, nwarps)
+                                                     : pull_level<4>(a, cur, d, nwarps);
             if (lane == 0 && found) atomicAdd(a.bcnt + (d + 1) % 3, found);
             if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             sparse = false;
