@@ -36,16 +36,21 @@ __global__ void __launch_bounds__(kCta) k_push_etwc_spill(DevGraph g,
                                                           OutCtx out) {
     lb_etwc_spill(g, spill, op, out, blockIdx.x, gridDim.x);
 }
-// (an update of one arc in flight needs the warps: eight CTAs per SM, 32
-// registers; 32 sources of RMAT-20 16.9 ms against 23.9 with 40 registers)
 template <class Op>
-__global__ void __launch_bounds__(kCta, Op::kFlight == 1 ? 8 : 1)
-    k_push_strict(DevGraph g, FrontierIn fin, int32_t fsize, const int32_t *scan, Op op, OutCtx out,
-                  unsigned long long *ctr) {
-    if constexpr (Op::kFlight == 1)
-        lb_strict_single(g, fin, fsize, scan, op, out, blockIdx.x, gridDim.x, ctr);
-    else
-        lb_strict(g, fin, fsize, scan, op, out, blockIdx.x, gridDim.x, ctr);
+__global__ void __launch_bounds__(kCta) k_push_strict(DevGraph g, FrontierIn fin, int32_t fsize,
+                                                      const int32_t *scan, Op op, OutCtx out,
+                                                      unsigned long long *ctr) {
+    lb_strict(g, fin, fsize, scan, op, out, blockIdx.x, gridDim.x, ctr);
+}
+// An update of one arc in flight needs the warps: eight CTAs per SM, 32
+// registers; 32 sources of RMAT-20 16.9 ms against 23.9 with 40 registers.
+// (A bound of one CTA on the kernel above gives its updates 16 to 24 registers
+// more: 64 BFS sources of RMAT-20 1.85 ms against 1.74.)
+template <class Op>
+__global__ void __launch_bounds__(kCta, 8) k_push_strict_single(DevGraph g, FrontierIn fin, int32_t fsize,
+                                                                const int32_t *scan, Op op, OutCtx out,
+                                                                unsigned long long *ctr) {
+    lb_strict_single(g, fin, fsize, scan, op, out, blockIdx.x, gridDim.x, ctr);
 }
 template <class Op>
 __global__ void __launch_bounds__(kCta) k_twc_classify(DevGraph g, FrontierIn fin, int32_t fsize,
@@ -133,7 +138,10 @@ inline g2_status push_round(g2_graph *g, const g2_schedule &s, const Op &op, con
             // delta-stepping rounds: 2,876 us with a serial owner search per
             // tile, one arc in flight per thread and an append per 32 arcs;
             // 1,529 us so (latency: 4 CTAs per SM, L2 22%, DRAM 11%)
-            k_push_strict<<<t->sm_count * 8, kCta, 0, st>>>(dg, fin, fsize, scan, op, out, ctr);
+            if constexpr (Op::kFlight == 1)
+                k_push_strict_single<<<t->sm_count * 8, kCta, 0, st>>>(dg, fin, fsize, scan, op, out, ctr);
+            else
+                k_push_strict<<<t->sm_count * 8, kCta, 0, st>>>(dg, fin, fsize, scan, op, out, ctr);
             stats().launches += 1;
             break;
         }
