@@ -54,8 +54,10 @@ struct OpMsBfs {
 // depth once, in order.  (Written to depth[b][v] round by round, the 64 arrays
 // took 446 us of RMAT-21's rounds in part lines, beside 80 us to clear them.)
 // A search of more levels goes on writing its depths directly, and so does one
-// without room for the planes.
-constexpr int kMsPlanes = 5;  // depths up to 31
+// without room for the planes or of few sources (12 sources: 0.36 against 0.37 ms
+// on RMAT-14, 0.40 against 0.43 on 300,001 vertices, 0.63 against 0.67 on RMAT-20).
+constexpr int kMsPlanes = 5;   // depths up to 31
+constexpr int kMsDirect = 16;  // sources whose depths are written directly
 struct MsLevels {
     u64 *plane[kMsPlanes];
     int32_t *depth;  // null while the planes are used
@@ -111,25 +113,34 @@ __device__ __forceinline__ void ms_note_active(u64 *active, u64 nm) {
 // whose frontier is not empty (`active`; a source in a small component ends
 // after a level or two, and waiting for its bit made every vertex read its
 // whole list).  Three kernels by the length of the list: k_ms_pull_pieces for
-// kMsPiece arcs and more, k_ms_pull for the first kMsThread arcs of the rest, a
-// thread each, k_ms_pull_rest for what those threads leave, a warp each from a
-// list (left to the warp that found them, the low ids of a power-law graph
-// held it for half a millisecond).  They only collect fnext; k_ms_commit_all
-// then passes over the vertices in order.  RMAT-21, 64 sources: the four pull
-// rounds took 1.99 ms with a thread per vertex waiting for every source (6 ms
-// where one source lay in a small component), 0.35 ms so, 0.15 ms to commit.
+// kMsPiece arcs and more (where the graph has such a vertex), k_ms_pull for the
+// first kMsThread arcs of the rest, a thread each, k_ms_pull_rest for what those
+// threads leave, a warp each from a list (left to the warp that found them, the
+// low ids of a power-law graph held it for half a millisecond; not launched where
+// no list is longer).  A vertex's new bits become visited, its level noted and
+// the vertex listed in k_ms_pull, for the pieces' vertices too, and those of
+// the rest in k_ms_pull_end, a lane each (by the warps of k_ms_pull_rest, a
+// vertex each: RMAT-20 5% slower; 32 vertices a warp there: 26%).  64 sources:
+// RMAT-21, the whole tuned search 1.10 ms (with a thread per vertex waiting for
+// every source 3.7, 6 where one source lay in a small component).
 struct MsPullArgs {
     DevGraph g;
-    const u64 *visit;
+    u64 *visit;
     const u64 *fcur;
     u64 *fnext;
     const u64 *active;  // sources with a frontier
+    u64 *active_next;
+    MsLevels l;
+    int32_t level;
+    int32_t *q, *q_cnt;  // the vertices with new bits
     int32_t *rest, *rest_cnt;
+    int32_t alone;       // arcs a thread walks before it leaves the rest
     int32_t *err;
     unsigned long long *ctr;
 };
 
-constexpr int32_t kMsThread = 32;   // arcs a thread walks alone
+constexpr int32_t kMsThread = 32;   // arcs a thread walks alone ...
+constexpr int32_t kMsAlone = 128;   // ... or the whole list where none is longer than this
 constexpr int32_t kMsPiece = 2048;  // arcs of a big vertex a CTA takes
 
 // the OR of up to four masks, in flight together, at arcs e, e + step, ...
@@ -144,42 +155,61 @@ __device__ __forceinline__ u64 ms_gather(const MsPullArgs &a, int64_t e, int ste
     return m;
 }
 
+__device__ __forceinline__ OutCtx ms_out(const MsPullArgs &a) {
+    OutCtx out;
+    memset(&out, 0, sizeof(out));
+    out.mode = OUT_SPARSE;
+    out.q = a.q;
+    out.cnt = a.q_cnt;
+    out.cap = out.cap2 = a.g.n;
+    out.q2 = a.rest;
+    out.cnt2 = a.rest_cnt;
+    out.err = a.err;
+    return out;
+}
+
 __global__ void __launch_bounds__(kCta) k_ms_pull(MsPullArgs a) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const u64 active = *a.active;
     const int32_t n = a.g.n;
-    OutCtx out;
-    memset(&out, 0, sizeof(out));
-    out.mode = OUT_SPARSE;
-    out.q = a.rest;
-    out.cnt = a.rest_cnt;
-    out.cap = n;
-    out.err = a.err;
+    const OutCtx out = ms_out(a);
     Stage st = stage_begin();
     for (int64_t base = gw * 32; base < n; base += nw * 32) {
         const int64_t v = base + lane;
-        u64 need = v < n ? active & ~a.visit[v] : 0, acc = 0;
+        const u64 seen = v < n ? a.visit[v] : ~0ull;
+        const u64 need = active & ~seen;
+        u64 nm = 0;
         int32_t b = 0, e = 0;
         int cnt = 0;
+        bool more = false;
         if (need) {
             b = a.g.crowptr[v];
             e = a.g.crowptr[v + 1];
             if (e - b < kMsPiece) {
-                const int32_t e1 = e - b > kMsThread ? b + kMsThread : e;
-                for (; b < e1 && (acc & need) != need; b += 4) {
-                    acc |= ms_gather(a, b, 1, e1);
+                const int32_t e1 = e - b > a.alone ? b + a.alone : e;
+                for (; b < e1 && (nm & need) != need; b += 4) {
+                    nm |= ms_gather(a, b, 1, e1);
                     cnt += e1 - b < 4 ? e1 - b : 4;
                 }
-                if (acc & need) a.fnext[v] = acc & need;
+                nm &= need;
+                more = b < e && nm != need;
+                if (nm) a.fnext[v] = nm;
             } else {
-                b = e;
+                nm = a.fnext[v];  // the pieces' result
             }
         }
         count_arcs(a.ctr, cnt);
+        if (more) nm = 0;  // k_ms_pull_rest goes on from fnext
+        const bool found = nm != 0;
+        if (__any_sync(G2_FULL, found)) {
+            if (found) a.visit[v] = seen | nm;
+            ms_set_level(a.l, (int32_t)v, nm, a.level);
+            ms_note_active(a.active_next, nm);
+        }
         const int32_t vs[1] = {(int32_t)v};
-        const int code[1] = {b < e && (acc & need) != need};
+        const int code[1] = {found ? 1 : more ? 2 : 0};
         emit_n<1>(out, st, vs, code);
     }
     stage_end(out, st);
@@ -238,36 +268,6 @@ __global__ void __launch_bounds__(kCta) k_ms_pull_pieces(MsPullArgs a, const int
     }
 }
 
-// The new masks of all vertices become visited, depths written, and the
-// vertices with one the new frontier.
-__global__ void __launch_bounds__(kCta) k_ms_commit_all(u64 *visit, const u64 *fnext, MsLevels l,
-                                                        int32_t level, u64 *active_next, int32_t *q,
-                                                        int32_t *qcnt, int32_t *err) {
-    const int lane = threadIdx.x & 31;
-    const int32_t n = l.n;
-    OutCtx out;
-    memset(&out, 0, sizeof(out));
-    out.mode = OUT_SPARSE;
-    out.q = q;
-    out.cnt = qcnt;
-    out.cap = n;
-    out.err = err;
-    Stage st = stage_begin();
-    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; base < n;
-         base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t v = base + lane;
-        const u64 nm = v < n ? fnext[v] : 0;
-        if (!__any_sync(G2_FULL, nm != 0)) continue;
-        if (nm) visit[v] |= nm;
-        ms_set_level(l, (int32_t)v, nm, level);
-        ms_note_active(active_next, nm);
-        const int32_t vs[1] = {(int32_t)v};
-        const int code[1] = {nm != 0};
-        emit_n<1>(out, st, vs, code);
-    }
-    stage_end(out, st);
-}
-
 // the vertices of at least `big` in-arcs, and their numbers of pieces
 __global__ void k_ms_big(const int32_t *crowptr, int32_t n, int32_t big, int32_t *list, int32_t *np,
                          int32_t *cnt) {
@@ -303,10 +303,50 @@ __global__ void k_ms_commit(const int32_t *touched, const int32_t *cnt_ptr, u64 
     }
 }
 
-__global__ void k_ms_clear(const int32_t *list, int32_t cnt, u64 *f) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt;
+// The end of a level: the masks of the spent frontier back to zero, and with
+// them what the next levels count in.
+struct MsEnd {
+    const int32_t *list;  // the spent frontier
+    int32_t cnt;
+    u64 *f;
+    int32_t *next_cnt, *next_rest;
+    u64 *active;
+};
+
+__device__ __forceinline__ void ms_end(const MsEnd &z) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *z.next_cnt = 0;
+        *z.next_rest = 0;
+        *z.active = 0;
+    }
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < z.cnt;
          i += (int64_t)gridDim.x * blockDim.x)
-        f[list[i]] = 0ull;
+        z.f[z.list[i]] = 0ull;
+}
+
+__global__ void k_ms_end(MsEnd z) { ms_end(z); }
+
+// ... and what k_ms_pull_rest found becomes visited.
+__global__ void __launch_bounds__(kCta) k_ms_pull_end(MsPullArgs a, MsEnd z) {
+    const int lane = threadIdx.x & 31;
+    const int32_t cnt = *a.rest_cnt;
+    OutCtx out = ms_out(a);
+    out.q2 = nullptr;
+    Stage st = stage_begin();
+    for (int64_t base = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31LL; base < cnt;
+         base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t i = base + lane;
+        const int32_t v = i < cnt ? a.rest[i] : 0;
+        const u64 nm = i < cnt ? a.fnext[v] : 0;
+        if (nm) a.visit[v] |= nm;
+        ms_set_level(a.l, v, nm, a.level);
+        ms_note_active(a.active_next, nm);
+        const int32_t vs[1] = {v};
+        const int code[1] = {nm != 0};
+        emit_n<1>(out, st, vs, code);
+    }
+    stage_end(out, st);
+    ms_end(z);
 }
 
 __global__ void k_ms_seed(const int32_t *srcs, int32_t k, u64 *visit, u64 *fcur, int32_t *depth,
@@ -463,16 +503,18 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
     G2_CK(cudaMemsetAsync(F[1], 0, (size_t)n * 8, st));
     MsLevels lv;
     u64 *planes = nullptr;
-    const g2_status room = ws(g, B_ROWS, (size_t)kMsPlanes * std::max(n, 1), &planes);
-    if (room != G2_ENOMEM) G2_TRY(room);
+    if (k > kMsDirect) {
+        const g2_status room = ws(g, B_ROWS, (size_t)kMsPlanes * std::max(n, 1), &planes);
+        if (room != G2_ENOMEM) G2_TRY(room);
+    }
     for (int j = 0; j < kMsPlanes; ++j) lv.plane[j] = planes + (size_t)j * n;
-    lv.depth = planes ? nullptr : depth;  // without room for planes: written directly
+    lv.depth = planes ? nullptr : depth;
     if (lv.depth) G2_CK(cudaMemsetAsync(depth, 0xFF, (size_t)k * n * 4, st));
     lv.n = n;
     int nplanes = 0;  // cleared so far
     G2_TRY(put_array(dsrc, srcs, k, st));
-    // ctrs: [0..1] list lengths, [2] big vertices, [3] a pull's rest, [8..11] active masks of the
-    // even and odd levels (all zero at the start of the call)
+    // ctrs: [0..1] list lengths, [2] big vertices, [3..4] a pull's rest by level parity, [8..11]
+    // active masks of the even and odd levels (all zero at the start of the call)
     u64 *active[2] = {reinterpret_cast<u64 *>(ctrs + 8), reinterpret_cast<u64 *>(ctrs + 10)};
     k_ms_seed<<<1, 64, 0, st>>>(dsrc, k, visit, F[0], lv.depth, n, list[0], ctrs + 0);
     const u64 full = k == 64 ? ~0ull : ((1ull << k) - 1);
@@ -483,7 +525,13 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
     int32_t nbig = 0;
     const bool pulls = h.s1.direction == G2_PULL ||
                        (h.criteria == G2_INPUT_VERTEXSET_SIZE && h.s2.direction == G2_PULL);
+    bool long_lists = true;  // in-lists that a thread leaves to a warp
     if (pulls) {
+        if (t->symmetric) {
+            int32_t dmax = 0;
+            G2_TRY(max_out_degree(g, st, &dmax));
+            long_lists = dmax > kMsAlone;
+        }
         int32_t *np;
         const size_t room = (size_t)t->m / kMsPiece + 1;  // vertices of kMsPiece arcs or more
         G2_TRY(ws(g, B_F0, room, &big));
@@ -509,8 +557,10 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
         G2_TRY(batch_lb(s));
         int q = 1 - p;
         u64 *act = active[(level - 1) & 1], *act_next = active[level & 1];
-        G2_CK(cudaMemsetAsync(ctrs + q, 0, 4, st));
-        G2_CK(cudaMemsetAsync(act_next, 0, 8, st));
+        int32_t *rest_cnt = ctrs + 3 + (level & 1);
+        // (the masks of the level's frontier become the all-zero array of the
+        // level after the next)
+        const MsEnd end{list[p], size, F[p], ctrs + p, ctrs + 3 + (1 - (level & 1)), act};
         if (!lv.depth && level == 1 << nplanes) {
             if (nplanes < kMsPlanes) {
                 G2_CK(cudaMemsetAsync(lv.plane[nplanes++], 0, (size_t)n * 8, st));
@@ -532,26 +582,30 @@ g2_status bfs_batch_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *de
             G2_TRY(push_round(g, s, OpMsBfs{visit, F[p], F[q]}, in, out, ctr, st));
             k_ms_commit<<<t->sm_count * 8, kCta, 0, st>>>(list[q], ctrs + q, visit, F[q], lv, level,
                                                         act_next);
+            k_ms_end<<<grid_for(g, size, kCta), kCta, 0, st>>>(end);
             stats().push_rounds++;
             stats().launches += 2;
         } else {
-            // (the schedule's VERTEX_BASED and WM run the same kernel)
-            MsPullArgs a{t->view(), visit, F[p], F[q], act, rest, ctrs + 3, d_err, ctr};
-            G2_CK(cudaMemsetAsync(ctrs + 3, 0, 4, st));
-            if (nbig > 0)
+            // (the schedule's VERTEX_BASED and WM run the same kernels)
+            MsPullArgs a{t->view(), visit, F[p], F[q], act, act_next, lv, level, list[q], ctrs + q, rest,
+                         rest_cnt, long_lists ? kMsThread : kMsAlone, d_err, ctr};
+            if (nbig > 0) {
                 k_ms_pull_pieces<<<grid_for(g, (int64_t)t->m / kMsPiece + nbig, 1), kCta, 0, st>>>(
                     a, big, nbig, piece);
+                stats().launches += 1;
+            }
             k_ms_pull<<<grid_for(g, n, kCta), kCta, 0, st>>>(a);
-            k_ms_pull_rest<<<t->sm_count * 16, kCta, 0, st>>>(a);
-            k_ms_commit_all<<<grid_for(g, n, kCta), kCta, 0, st>>>(visit, F[q], lv, level, act_next,
-                                                                 list[q], ctrs + q, d_err);
+            if (long_lists) {
+                k_ms_pull_rest<<<t->sm_count * 16, kCta, 0, st>>>(a);
+                k_ms_pull_end<<<std::max(t->sm_count * 8, grid_for(g, size, kCta)), kCta, 0, st>>>(a, end);
+                stats().launches += 1;
+            } else {
+                k_ms_end<<<grid_for(g, size, kCta), kCta, 0, st>>>(end);
+            }
             G2_CK(cudaGetLastError());
             stats().pull_rounds++;
-            stats().launches += nbig > 0 ? 4 : 3;
+            stats().launches += 2;
         }
-        // the current frontier masks become the (all-zero) next-next array
-        k_ms_clear<<<grid_for(g, size, kCta), kCta, 0, st>>>(list[p], size, F[p]);
-        stats().launches += 1;
         G2_TRY(read_counters(g, ctrs, 4, st, d_err));
         size = g->h_ctr[q];
         p = q;
