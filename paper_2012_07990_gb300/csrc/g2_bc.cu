@@ -711,9 +711,10 @@ __global__ void __launch_bounds__(kClCta, 1) k_bc_cluster(ClusterBcArgs a) {
 }
 
 // ------------------------------------------------------------------- host
-// The source's depths by one edgeset.apply round per level.  *levels: how many.
-static g2_status bc_depths(g2_graph *g, const BcState &s, const g2_hybrid &h, int32_t *levels,
-                           cudaStream_t st, int32_t *d_err) {
+// The source's depths by one edgeset.apply round per level.  Level L's vertices
+// are s.lvl[starts[L], starts[L + 1]).
+static g2_status bc_depths(g2_graph *g, const BcState &s, const g2_hybrid &h,
+                           std::vector<int32_t> &starts, cudaStream_t st, int32_t *d_err) {
     Topology *t = g->topo;
     const int32_t n = t->n;
     int32_t *ctrs = d_err - 62;
@@ -722,7 +723,9 @@ static g2_status bc_depths(g2_graph *g, const BcState &s, const g2_hybrid &h, in
     G2_TRY(ws(g, B_BM0, (size_t)(n + 31) / 32 + 1, &bm));
     G2_TRY(ws(g, B_BOOL0, (size_t)std::max(n, 1), &bo));
     int32_t b = 0, e = 1;
-    for (int d = 0;; ++d) {
+    starts.assign(1, 0);
+    for (;;) {
+        starts.push_back(e);
         const int32_t size = e - b;
         const g2_schedule &sc = pick_schedule(h, size, n);
         G2_TRY(check_schedule(g, sc, K_BFS, false));
@@ -753,10 +756,7 @@ static g2_status bc_depths(g2_graph *g, const BcState &s, const g2_hybrid &h, in
         sc.direction == G2_PUSH ? stats().push_rounds++ : stats().pull_rounds++;
         G2_TRY(read_counters(g, ctrs, 4, st, d_err));
         const int32_t nn = g->h_ctr[3];
-        if (nn == 0) {
-            *levels = d + 1;
-            return G2_OK;
-        }
+        if (nn == 0) return G2_OK;
         stats().iterations++;
         b = e;
         e += nn;
@@ -850,10 +850,22 @@ static g2_status bc_one_plain(g2_graph *g, const BcState &s, const g2_hybrid &h,
         k_bc_init_rec<<<grid_for(g, n, kCta), kCta, 0, st>>>(s, n);
     } else {
         k_bc_init<<<grid_for(g, n, kCta), kCta, 0, st>>>(s, n, nullptr);
-        G2_TRY(bc_depths(g, s, h, &levels, st, d_err));
+        G2_TRY(bc_depths(g, s, h, gr.off, st, d_err));
+        levels = (int32_t)gr.off.size() - 1;
     }
     stats().launches += 1;
-    G2_TRY(bc_group(g, s, s.g.crowptr, levels, gr, st, d_err));
+    if (!fused_depths && s.per_thread) {
+        // short lists: the levels as they were found, a thread per vertex (all
+        // of class 0; sorting each source's vertices by degree costs a 64 x 64
+        // grid 4% of the call)
+        gr.levels = levels;
+        gr.off.resize((size_t)4 * levels + 1, gr.off.back());
+        gr.piece = nullptr;
+        gr.done = nullptr;
+        gr.part = nullptr;
+    } else {
+        G2_TRY(bc_group(g, s, s.g.crowptr, levels, gr, st, d_err));
+    }
     for (int32_t L = 1; L < levels; ++L) launch_level<true>(g, s, gr, L, L - 1, false, st);
     if (!t->symmetric) G2_TRY(bc_group(g, s, s.g.rowptr, levels, gr, st, d_err));
     for (int32_t L = levels - 1; L >= 0; --L)
