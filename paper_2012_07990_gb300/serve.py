@@ -165,11 +165,14 @@ class GpuExecutor:
         self.streams = [torch.cuda.Stream() for _ in range(slots)]
         self.views = [{name: g.handle.view() for name, g in pool.graphs.items()} for _ in range(slots)]
         self.fused = g2.schedule("WM", kernel_fusion=True)
-        # A single BFS or SSSP on a power-law graph: with several slots, the
-        # tuned schedules as launches per level or round, whose small kernels
-        # interleave with the other slots' work (the fused form's cooperative
-        # launch needs every SM at once, so the slots' launches would run one
-        # at a time); with one slot, the library's tuned schedule (NULL).
+        # A single BFS or SSSP, or BC from several sources, on a power-law
+        # graph: with several slots, the tuned schedules as launches per level
+        # or round, whose small kernels interleave with the other slots' work
+        # (the fused form's cooperative launch needs every SM at once, so it
+        # waits for the other slots and they for it: 3,000 queries a second on
+        # two power-law graphs and a grid, half of them BC in batches of up to
+        # 8, p99 18-30 ms with the library's BC, 8 ms by rounds); with one slot,
+        # the library's tuned schedule (NULL).
         self.powerlaw_bfs = self.powerlaw_sssp = None
         if slots > 1:
             pull = g2.schedule("VERTEX_BASED", direction=g2.G2_PULL, pull_frontier=g2.G2_BITMAP,
@@ -204,7 +207,7 @@ class GpuExecutor:
                     g2.g2_sssp_batch(view, srcs, pg.spec.delta, out, None)
             else:
                 out = torch.empty(n, dtype=torch.float64, device="cuda")
-                g2.g2_bc(view, srcs, out, single)
+                g2.g2_bc(view, srcs, out, single if pg.spec.road or k == 1 else self.powerlaw_bfs)
             if self.keep_results:
                 host = out.cpu().numpy()
                 rows = host.reshape(k, n) if r0.kind != "bc" else host.reshape(1, n)
