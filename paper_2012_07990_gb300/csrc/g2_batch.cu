@@ -361,17 +361,6 @@ __global__ void k_ms_seed(const int32_t *srcs, int32_t k, u64 *visit, u64 *fcur,
     }
 }
 
-template <class Op>
-__global__ void __launch_bounds__(kCta) k_ms_push(DevGraph g, FrontierIn fin, int32_t fsize, Op op,
-                                                  OutCtx out, int lb, unsigned long long *ctr) {
-    switch (lb) {
-        case G2_LB_WM: lb_warp(g, fin, fsize, op, out, blockIdx.x, gridDim.x, ctr); break;
-        case G2_LB_CM: lb_cta(g, fin, fsize, op, out, blockIdx.x, gridDim.x, ctr); break;
-        case G2_LB_ETWC: lb_etwc(g, fin, fsize, op, out, blockIdx.x, gridDim.x, ctr); break;
-        default: lb_vertex(g, fin, fsize, op, out, blockIdx.x, gridDim.x, ctr); break;
-    }
-}
-
 // ------------------------------------------- multi-source BFS, fused
 // The whole multi-source loop in one cooperative kernel (kernel fusion for
 // the batch): per level a WM PUSH over the list of vertices whose frontier

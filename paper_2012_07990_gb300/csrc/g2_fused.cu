@@ -1252,8 +1252,7 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     // faster alone (4096^2, delta 16384: 34.4 ms against 38) and slower
     // beside other streams, where that launch waits for the whole GPU (a mixed
     // load of 500 queries a second in 4 slots: p99 390 ms against 73).
-    const int32_t hi = 1024 * cl;
-    c.hi = env_i32("G2_CLUSTER_HI", hi);
+    c.hi = env_i32("G2_CLUSTER_HI", 1024 * cl);
     c.dedup_near = !(t->symmetric && dmax <= kBoundedDegree);
     c.nq_out = a.nq[0];
     c.fq_out = a.fq[0];
@@ -1263,7 +1262,7 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     c.result = ctrs + 36;
     c.err = d_err;
     c.ctr = a.ctr;
-    a.lo_far = cl ? std::min(std::min(env_i32("G2_CLUSTER_FAR_LO", hi), c.hi),
+    a.lo_far = cl ? std::min(std::min(env_i32("G2_CLUSTER_FAR_LO", 1024 * cl), c.hi),
                              (int32_t)(kCsQf / 2 * cl))
                   : 0;
     int32_t T = (int32_t)std::min<int64_t>(delta, G2_INF32);
@@ -1305,11 +1304,9 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
             a.T0 = T;
             a.round0 = round0;
             a.epoch0 = epoch0;
-            // one CTA per SM (two: 35.6 against 38.0 ms on 4096^2 with delta
-            // 16384, but see above)
-            const int ctas = env_i32("G2_FUSED_CTAS_PER_SM", 1);
+            // (one CTA per SM: see above)
             switch (s.load_balance) {
-                case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st, ctas)); break;
+                case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st)); break;
                 case G2_LB_CM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_CM>, a, st)); break;
                 case G2_LB_ETWC: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_ETWC>, a, st)); break;
                 case G2_LB_STRICT:
