@@ -211,6 +211,11 @@ g2_status g2_frontier_list(g2_frontier *f, int32_t *verts, int32_t cap, int32_t 
  *                   Output: v whose dist decreased.
  *  G2_OP_LABEL_MIN  vdata int32 label[n].  label[v] = min(label[v], label[u]).
  *                   Output: v whose label decreased.
+ *                   In both, a PUSH round takes dist[u] / label[u] from before
+ *                   the round; a PULL round reads them as they are, so a value
+ *                   may travel over several arcs in one PULL round and which
+ *                   do depends on what runs first.  Loops that go on until
+ *                   nothing decreases end with the same values either way.
  *  G2_OP_PR_ADD     vdata float contrib[n] (per source), vdata2 float acc[n].
  *                   acc[v] += contrib[u].  No output frontier (out must be NULL).
  *  G2_OP_BC_SIGMA   vdata int32 depth[n] (read only), vdata2 double sigma[n].
@@ -240,7 +245,8 @@ typedef enum {
  *   vdata/2   device arrays, typed by op (above)
  *   sched     schedule (NULL = defaults); a hybrid picks s1/s2 by |in|
  *   out       output vertexset (applyModified), or NULL (apply).  Its
- *             previous contents are replaced.
+ *             previous contents are replaced; a call that fails before or in
+ *             its round leaves them as they were.  May be `in`.
  *   out_size  host int32 receiving |out| (nullable) */
 g2_status g2_edgeset_apply(g2_graph *g, g2_op op, g2_frontier *in, void *vdata, void *vdata2,
                            const g2_hybrid *sched, g2_frontier *out, int32_t *out_size,
@@ -330,7 +336,8 @@ g2_status g2_bc(g2_graph *g, const int32_t *srcs, int32_t k, double *bc,
  * queries of the serving path): k <= 64 sources (host int32[k]) in one traversal, one bit
  * per source in per-vertex 64-bit visit/frontier masks.  depth int32[k][n]
  * device (row i = BFS from srcs[i]).  Schedules: PUSH with any frontier load
- * balancing but EDGE_ONLY, PULL with VERTEX_BASED or WM, or kernel fusion with
+ * balancing but EDGE_ONLY, PULL with VERTEX_BASED or WM (one form: a thread, a
+ * warp or CTAs per vertex by the length of its list), or kernel fusion with
  * WM PUSH (the whole loop in one cooperative kernel).  NULL schedule: the
  * direction-optimising hybrid (STRICT PUSH below 2% of n, VERTEX_BASED PULL);
  * on a bounded-degree graph (largest out-degree <= 32) the sources run as
@@ -350,10 +357,12 @@ g2_status g2_bfs_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t *dep
  * Schedules: PUSH with any frontier load balancing but EDGE_ONLY, or kernel
  * fusion with WM PUSH (the whole loop in one cooperative kernel).  NULL
  * schedule: the distances of a vertex from all sources relaxed together as one
- * row, in rounds over the vertices whose row changed (delta is not used), or
- * STRICT PUSH where that has not ended after 32 rounds; on a bounded-degree
- * graph (largest out-degree <= 32) the sources run as single-source fused WM queries, about one per 19 SMs at
- * a time, as g2_bfs_batch does (G2_BATCH_SPLIT_WORKERS = 0: the fused
+ * row, in rounds over the vertices whose row changed (delta is not used), and
+ * from there STRICT PUSH over the near/far queue where that has not ended after
+ * 32 rounds (16, if as many vertices still change as ever), or STRICT PUSH
+ * from the start where there is no memory for the rows (up to 128 bytes a
+ * vertex); on a bounded-degree graph (largest out-degree <= 32) the sources run
+ * as single-source fused WM queries, about one per 19 SMs at a time, as g2_bfs_batch does (G2_BATCH_SPLIT_WORKERS = 0: the fused
  * multi-source loop). */
 g2_status g2_sssp_batch(g2_graph *g, const int32_t *srcs, int32_t k, int32_t delta,
                         int32_t *dist, const g2_hybrid *sched, void *stream);

@@ -85,7 +85,7 @@ def sample_schedule(algo: str, rng: random.Random) -> dict:
         return {"criteria": 0, "threshold": 0.0, "s1": s, "s2": s}
     if algo == "bfs_batch":
         push = _simple(lb=rng.choice(PUSH_FRONTIER_LBS))
-        pull = _simple(lb=rng.choice(["VERTEX_BASED", "WM"]), direction=1)
+        pull = _simple(lb="VERTEX_BASED", direction=1)   # WM runs the same kernels
         return {"criteria": 1, "threshold": rng.choice([0.0, 0.005, 0.02, 0.05, 1e9]), "s1": push,
                 "s2": pull}
     raise ValueError(f"unknown algorithm {algo}")

@@ -26,11 +26,12 @@
 // one launch of the fused hybrid when there are several sources), then the
 // reached vertices are grouped by level and degree, and sigma and delta are
 // pulled level by level over the groups: a thread, eight lanes, a warp or a
-// CTA per vertex by its degree.  With kernel fusion the whole source runs in
-// one persistent cooperative kernel with one grid barrier per level and pass;
-// there the pulls give a warp to every vertex and a whole CTA to the vertices
-// with at least kBigDeg arcs, or a thread to every vertex on a symmetric
-// bounded-degree graph.
+// CTA per piece of a vertex by its degree (on a symmetric bounded-degree graph a
+// thread per vertex over the levels as found).  With kernel fusion the whole
+// source runs in one persistent cooperative kernel with one grid barrier per
+// level and pass; there the pulls give a thread to the vertices below
+// kThreadDeg arcs, a warp to those below kBigDeg and a whole CTA to the rest,
+// or a thread to every vertex on a symmetric bounded-degree graph.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -117,9 +118,9 @@ struct BcState {
     double *bc;
     int32_t *lvl;  // all levels, in order
     int32_t src;
-    // fused kernels' granularity: one thread per vertex on a symmetric
-    // bounded-degree graph (every list short), else one warp per vertex and,
-    // when some vertex may have kBigDeg or more arcs (`big`), one CTA for those
+    // granularity: one thread per vertex on a symmetric bounded-degree graph
+    // (every list short), else by degree (fused kernels: threads, warps and,
+    // when some vertex may have kBigDeg or more arcs (`big`), CTAs for those)
     int32_t per_thread;
     int32_t big;
 };
@@ -390,11 +391,11 @@ struct BcLevel {
 };
 
 // sigma of the vertices at level d + 1 (SIGMA), or delta of those at level d.
-// The largest first, each class by the whole grid.  Bound: one L1 tag look-up
-// per gathered record (84% of L1's peak with two 8-byte loads a record).  Six
-// CTAs per SM: delta's pass needs 70 registers unbounded (17.4 ms for 16
-// sources of RMAT-21 against 19.4, 17.7 with five, 18.9 with eight); two
-// records in flight per lane instead of four 18.9 ms.
+// The largest first, each class by the whole grid.  Bound: the gathered records
+// through L1 (66% of its peak on RMAT-20's largest levels) and L2 (45%).  Six
+// CTAs per SM, though delta's pass spills 104 bytes at its 40 registers: it
+// needs 70 unbounded (17.4 ms for 16 sources of RMAT-21 against 19.4, 17.7 with
+// five, 18.9 with eight); two records in flight per lane instead of four 18.9 ms.
 template <bool SIGMA>
 __global__ void __launch_bounds__(kCta, 6) k_bc_level(BcState s, BcLevel l, int32_t d,
                                                    int32_t deepest) {

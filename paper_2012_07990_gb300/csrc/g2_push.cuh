@@ -137,7 +137,8 @@ inline g2_status push_round(g2_graph *g, const g2_schedule &s, const Op &op, con
             // CTAs and stride.  RMAT of 1,300,003 vertices, 107M arcs over 29
             // delta-stepping rounds: 2,876 us with a serial owner search per
             // tile, one arc in flight per thread and an append per 32 arcs;
-            // 1,529 us so (latency: 4 CTAs per SM, L2 22%, DRAM 11%)
+            // 1,529 us so (latency: 4 CTAs per SM; RMAT-20's largest round L2
+            // 24% and DRAM 12% of their peaks)
             if constexpr (Op::kFlight == 1)
                 k_push_strict_single<<<t->sm_count * 8, kCta, 0, st>>>(dg, fin, fsize, scan, op, out, ctr);
             else

@@ -21,10 +21,11 @@
 // in L1, and relaxes kRowFlight arcs at once.  A round with fewer takes the
 // flagged vertices as a list, their arcs divided evenly by a prefix sum.
 //
-// Bound: the latency of the row reads, at 37 warps per SM with 8 rows each in
-// flight (half of them hit L1; L2 21%, DRAM 13% of peak).  RMAT-21, 32 sources,
-// weights 1-255: a sweep with every vertex flagged 1.4 ms, the whole call 8.2
-// ms, against 42.7 ms for STRICT delta-stepping over stacked arrays.  Measured
+// Bound: the row reads through L1 (57% of its peak, a quarter of the sectors
+// hit; issue 48%, L2 26%, DRAM 13%; 36 warps per SM with 8 rows each in flight).
+// RMAT-21, 32 sources, weights 1-255: a sweep with every vertex flagged 1.4 ms,
+// the whole call 8.1-8.4 ms, against 40-43 ms for STRICT delta-stepping over
+// stacked arrays when the rows replaced it (33.8 ms since).  Measured
 // and rejected: the arcs held a lane each and handed out by shuffles (36
 // instructions an arc, 2.5 ms a sweep), fewer registers for more warps (6 CTAs
 // per SM 13.0 ms, 8 CTAs 19.7 ms: spills).
