@@ -162,11 +162,13 @@ __device__ bool fused_strict_scan(const DevGraph &g, const int32_t *q, int32_t s
 // number, in lane 0, the result.  The chain of depth, row offsets, id and frontier
 // bit is what bounds it, so a warp takes W words at once and a lane has W of them
 // in flight: the whole search of RMAT-22 from the hub 191 us with one, 173 with
-// two, 156 with four, 177 with eight (registers).  The grid's warps take turns
-// across the CTAs, so that a graph of fewer words than the warps could take
-// keeps every SM at work, and such a graph is taken one word at a time: 100,000
+// two, 156 with four, 177 with eight (registers).  The shares go round the CTAs,
+// so that every SM is at work where there are fewer words than that for every
+// warp, and where there is one for a warp at most, it takes one: 100,000
 // vertices of out-degree about 48, 60 hops across, 0.64 ms; 0.90 with four, 2.26 with
-// four and neighbouring shares in one CTA, 0.77 with one and those.
+// four and neighbouring shares in one CTA, 0.77 with one and those.  (With more
+// words than warps four are better: the same graph with CM PUSH, two CTAs per SM,
+// 0.85 against 0.88 ms, with ETWC PUSH, one CTA, 0.63 against 0.79.)
 template <int W>
 __device__ __forceinline__ int32_t pull_level(const FusedDoBfsArgs &a, const uint32_t *cur, int d,
                                               int64_t nwarps) {
@@ -346,8 +348,8 @@ __global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 
                 if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             }
             // bottom-up over every vertex; the next level as a bitmap
-            const int32_t found = words < 4 * nwarps ? pull_level<1>(a, cur, d, nwarps)
-                                                     : pull_level<4>(a, cur, d, nwarps);
+            const int32_t found = words <= nwarps ? pull_level<1>(a, cur, d, nwarps)
+                                                  : pull_level<4>(a, cur, d, nwarps);
             if (lane == 0 && found) atomicAdd(a.bcnt + (d + 1) % 3, found);
             if (!grid_sync(a.bar, a.err, a.limit_ns)) return;
             sparse = false;

@@ -1,6 +1,7 @@
 """The fused hybrid's PULL levels about the line between one and four bitmap
-words a warp (4,865 words with one CTA per SM on 152 SMs), and a band whose
-levels leave most lists without a hit; bit-exact against the oracle."""
+words a warp (1,216 words with one CTA per SM on 152 SMs), where four fill
+every warp (4,864), and on a band whose levels leave most lists without a hit;
+bit-exact against the oracle."""
 import numpy as np
 import pytest
 
@@ -10,7 +11,7 @@ from paper_2012_07990_gb300 import graphgen as gg
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-LINE = 4 * 152 * 8 * 32
+LINE = 152 * 8 * 32
 
 
 def _check(g, src):
@@ -30,7 +31,7 @@ def _check(g, src):
     assert np.array_equal(parent.cpu().numpy(), want_parent)
 
 
-@pytest.mark.parametrize("n", [LINE - 64, LINE - 31, LINE, LINE + 1, LINE + 97])
+@pytest.mark.parametrize("n", [line + d for line in (LINE, 4 * LINE) for d in (-64, -31, 0, 1, 97)])
 def test_about_the_line(monkeypatch, n):
     monkeypatch.setenv("G2_FUSED_DO_CTAS_PER_SM", "1")
     r = np.random.default_rng(n)
