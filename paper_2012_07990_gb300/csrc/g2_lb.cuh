@@ -241,10 +241,11 @@ __device__ __forceinline__ StrictOwners<Op> &strict_owners() {
 // STRICT for an update of one arc in flight (it loops over sources for every
 // arc, and lives on what L1 keeps of their distances): the tiles' owners would
 // be shared memory taken from L1, and tiles of kCta arcs.  A warp takes
-// kStrictWarp arcs, and a lane searches the scan itself, between the owners of
-// the first and the last.  32 sources of RMAT-20, weights 1-255: 16.9 ms, 27.7
-// with owners in shared memory in tiles of kCta arcs, 23.9 in tiles of 4 kCta,
-// 19.8 with 512 arcs a warp.
+// kStrictWarp arcs (32 where there are not as many for every warp), and a lane
+// searches the scan itself, between the owners of the first and the last.  32
+// sources of RMAT-20, weights 1-255: 16.9 ms, 27.7 with owners in shared memory
+// in tiles of kCta arcs, 23.9 in tiles of 4 kCta, 19.8 with 512 arcs a warp.
+// RMAT-14: 3.7 ms, 4.4 with 128 arcs for every warp; 400 x 400 grid 26.9 and 32.2.
 constexpr int kStrictWarp = 128;
 
 template <class Op>
@@ -255,8 +256,9 @@ __device__ void lb_strict_single(const DevGraph &g, const FrontierIn &fin, int32
     const int lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)bid * kWarps + (threadIdx.x >> 5), nw = (int64_t)nb * kWarps;
     const int32_t total = scan[fsize];
-    for (int64_t t0 = gw * kStrictWarp; t0 < total; t0 += nw * kStrictWarp) {
-        const int64_t t1 = t0 + kStrictWarp < total ? t0 + kStrictWarp : total;
+    const int share = total < nw * kStrictWarp ? 32 : kStrictWarp;
+    for (int64_t t0 = gw * share; t0 < total; t0 += nw * share) {
+        const int64_t t1 = t0 + share < total ? t0 + share : total;
         const int32_t own0 = scan_owner(scan, fsize, (int32_t)t0);
         const int32_t own1 = scan_owner(scan, fsize, (int32_t)(t1 - 1));
         count_arcs(ctr, lane == 0 ? (int)(t1 - t0) : 0);
