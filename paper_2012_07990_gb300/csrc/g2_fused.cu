@@ -393,8 +393,14 @@ struct FusedSsspArgs {
 // threshold go to the next near list, the rest to the far pile); then the
 // smallest live far distance picks the next bucket and the far pile is split
 // (stale entries, already settled, are dropped).
-template <int LB>
-__global__ void __launch_bounds__(kCta, LB == G2_LB_STRICT ? kFusedStrictCtas : 1) k_sssp_fused(FusedSsspArgs a) {
+// CTAS: how many CTAs' registers fit on an SM.  One query alone runs one (WM
+// then takes 96 registers).  Beside the other queries of a batch, each with a
+// launch of one CTA per SM, as many queries run at once as fit: with 40
+// registers six, 32 sources on the 4096^2 grid, delta 16384, 311 ms; 509 with
+// 96 registers, 355 with 64, 329 with 48.  (Alone 38.8 ms against 37.6.)
+constexpr int kSsspBeside = 6;
+template <int LB, int CTAS = LB == G2_LB_STRICT ? kFusedStrictCtas : 1>
+__global__ void __launch_bounds__(kCta, CTAS) k_sssp_fused(FusedSsspArgs a) {
     const int32_t n = a.g.n;
     int64_t T = a.T0;
     int d = 0, fp = 0, epoch = 0, buckets = 0, handover = 0;
@@ -1308,7 +1314,10 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
             a.epoch0 = epoch0;
             // (one CTA per SM: see above)
             switch (s.load_balance) {
-                case G2_LB_WM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st)); break;
+                case G2_LB_WM:
+                    if (g->beside) G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM, kSsspBeside>, a, st, 1));
+                    else G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st));
+                    break;
                 case G2_LB_CM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_CM>, a, st)); break;
                 case G2_LB_ETWC: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_ETWC>, a, st)); break;
                 case G2_LB_STRICT:

@@ -804,6 +804,8 @@ static g2_graph *new_handle(Topology *t) {
     g->round = 0;
     g->round2 = 0;
     g->st = nullptr;
+    g->settled = false;
+    g->beside = false;
     return g;
 }
 

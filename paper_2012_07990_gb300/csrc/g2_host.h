@@ -73,6 +73,7 @@ struct g2_graph {
     int32_t round2;
     cudaStream_t st;  // stream of the call in progress (set at every entry)
     bool settled;     // nothing was queued after the last read_counters of the call
+    bool beside;      // its calls run at the same time as others' (a batch's workers)
 };
 
 struct g2_frontier {
