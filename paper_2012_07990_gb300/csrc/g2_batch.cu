@@ -1095,10 +1095,10 @@ namespace g2 {
 // graph (its own workspace) and a stream of its own, driven by a host thread.
 // A single-source fused loop keeps most levels of a road graph inside one
 // 16-CTA thread-block cluster, so about nine of them fit on the GPU at once;
-// on the 4096^2 road grid 64 BFS sources take 178 ms this way against 475 ms
-// in one multi-source traversal (whose 64 wavefronts rarely meet, so it does
-// the same vertex work with wider masks), and 32 SSSP sources 447 ms against
-// 512 ms.  Outputs are row i of the caller's k x n array, as in the batched
+// on the 4096^2 road grid 64 BFS sources take 156-166 ms this way against 286
+// ms in one multi-source traversal (whose 64 wavefronts rarely meet, so it does
+// the same vertex work with wider masks), and 32 SSSP sources 291 ms against
+// 376 ms.  Outputs are row i of the caller's k x n array, as in the batched
 // traversal.
 static int split_workers(g2_graph *g, int32_t k, int per_sm_default) {
     int w = std::max(1, g->topo->sm_count / per_sm_default);
