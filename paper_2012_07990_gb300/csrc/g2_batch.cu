@@ -1116,7 +1116,6 @@ static g2_status split_run(g2_graph *g, const int32_t *srcs, int32_t k, int32_t 
     g2_status made = G2_OK;
     for (int i = 0; i < workers && made == G2_OK; ++i) {
         made = g2_graph_view(g, &views[i]);
-        if (made == G2_OK) views[i]->beside = true;
         if (made == G2_OK && cudaStreamCreateWithFlags(&streams[i], cudaStreamNonBlocking) != cudaSuccess)
             made = fail(G2_ECUDA, "stream for a split batch");
     }

@@ -394,10 +394,10 @@ struct FusedSsspArgs {
 // smallest live far distance picks the next bucket and the far pile is split
 // (stale entries, already settled, are dropped).
 // CTAS: how many CTAs' registers fit on an SM.  One query alone runs one (WM
-// then takes 96 registers).  Beside the other queries of a batch, each with a
-// launch of one CTA per SM, as many queries run at once as fit: with 40
-// registers six, 32 sources on the 4096^2 grid, delta 16384, 311 ms; 509 with
-// 96 registers, 355 with 64, 329 with 48.  (Alone 38.8 ms against 37.6.)
+// then takes 96 registers).  Where queries run side by side on a graph, each with
+// a launch of one CTA per SM, as many run at once as fit: with 40 registers
+// six, 32 sources on the 4096^2 grid, delta 16384, 311 ms; 509 with 96
+// registers, 355 with 64, 329 with 48.  (Alone 38.8 ms against 37.6.)
 constexpr int kSsspBeside = 6;
 template <int LB, int CTAS = LB == G2_LB_STRICT ? kFusedStrictCtas : 1>
 __global__ void __launch_bounds__(kCta, CTAS) k_sssp_fused(FusedSsspArgs a) {
@@ -1189,6 +1189,13 @@ g2_status bfs_fused_do(g2_graph *g, int32_t src, int32_t *depth, int32_t *parent
     return G2_OK;
 }
 
+// A call counted among those in flight while it lives.
+struct InFlight {
+    std::atomic<int> &count;
+    explicit InFlight(std::atomic<int> &c) : count(c) { ++count; }
+    ~InFlight() { --count; }
+};
+
 // (STRICT is the tuned schedule on power-law graphs; the caller checks that a
 // schedule of its user's does not ask for it.)
 g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
@@ -1197,6 +1204,7 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
     if (s.frontier_creation != G2_FUSED || s.dedup != G2_DEDUP_ENABLED)
         return fail(G2_EUNSUPPORTED, "the fused near/far queue uses FUSED lists with deduplication");
     Topology *t = g->topo;
+    const InFlight counted(t->near_far);
     const int32_t n = t->n;
     int32_t *ctrs = d_err - 62;
     FusedSsspArgs a;
@@ -1315,7 +1323,7 @@ g2_status sssp_fused(g2_graph *g, int32_t src, int32_t delta, int32_t *dist,
             // (one CTA per SM: see above)
             switch (s.load_balance) {
                 case G2_LB_WM:
-                    if (g->beside) G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM, kSsspBeside>, a, st, 1));
+                    if (t->near_far > 1) G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM, kSsspBeside>, a, st, 1));
                     else G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_WM>, a, st));
                     break;
                 case G2_LB_CM: G2_TRY(launch_coop(g, k_sssp_fused<G2_LB_CM>, a, st)); break;

@@ -805,7 +805,6 @@ static g2_graph *new_handle(Topology *t) {
     g->round2 = 0;
     g->st = nullptr;
     g->settled = false;
-    g->beside = false;
     return g;
 }
 

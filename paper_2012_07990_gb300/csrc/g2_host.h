@@ -73,7 +73,6 @@ struct g2_graph {
     int32_t round2;
     cudaStream_t st;  // stream of the call in progress (set at every entry)
     bool settled;     // nothing was queued after the last read_counters of the call
-    bool beside;      // its calls run at the same time as others' (a batch's workers)
 };
 
 struct g2_frontier {
@@ -91,6 +90,7 @@ namespace g2 {
 
 struct Topology {
     std::atomic<int> refs;
+    std::atomic<int> near_far{0};  // fused near/far queries in flight, on all views
     // serialise the lazy layout builders (views on several threads share
     // the topology); recursive because one builder may call another.
     // PageRank's layouts have a lock of their own, so that building them in
