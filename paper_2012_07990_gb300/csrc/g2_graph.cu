@@ -685,29 +685,34 @@ g2_status ensure_edge_block(g2_graph *g, int32_t N, cudaStream_t st) {
     }
     G2_TRY(ensure_coo(g, st));
     int64_t runs = nseg * n;
-    int32_t *cnt = nullptr, *off = nullptr, *beg = nullptr;
-    G2_CK(dmalloc(&t->eb_src, (size_t)std::max<int64_t>(m, 1) * 4, st));
-    G2_CK(dmalloc(&t->eb_dst, (size_t)std::max<int64_t>(m, 1) * 4, st));
-    G2_CK(dmalloc(&t->eb_seg, (size_t)(nseg + 1) * 8, st));
-    G2_CK(dmalloc(&cnt, (size_t)(runs + 1) * 4, st));
-    G2_CK(dmalloc(&off, (size_t)(runs + 1) * 4, st));
-    G2_CK(dmalloc(&beg, (size_t)(runs + 1) * 4, st));
+    // the graph's only when all of it is built
+    HeldBlocks mem(st);
+    int32_t *src, *dst, *cnt, *off, *beg;
+    int64_t *seg;
+    G2_CK(mem.alloc(&src, (size_t)std::max<int64_t>(m, 1) * 4));
+    G2_CK(mem.alloc(&dst, (size_t)std::max<int64_t>(m, 1) * 4));
+    G2_CK(mem.alloc(&seg, (size_t)(nseg + 1) * 8));
+    G2_CK(mem.alloc(&cnt, (size_t)(runs + 1) * 4));
+    G2_CK(mem.alloc(&off, (size_t)(runs + 1) * 4));
+    G2_CK(mem.alloc(&beg, (size_t)(runs + 1) * 4));
     if (runs > 0) {
         k_eb_runs<<<grid_for(g, runs, kCta), kCta, 0, st>>>(t->rowptr, t->col, n, N, (int32_t)nseg,
                                                             cnt, beg);
         G2_TRY(exclusive_scan_i32(g, cnt, off, (int32_t)runs, st));
         if (m > 0)
             k_eb_scatter<<<grid_for(g, m, kCta), kCta, 0, st>>>(t->coo_src, t->col, m, n, N, off,
-                                                                beg, t->eb_src, t->eb_dst);
+                                                                beg, src, dst);
     }
-    k_eb_seg_end<<<(int)((nseg + 1 + kCta - 1) / kCta), kCta, 0, st>>>(off, n, (int32_t)nseg, m,
-                                                                       t->eb_seg);
+    k_eb_seg_end<<<(int)((nseg + 1 + kCta - 1) / kCta), kCta, 0, st>>>(off, n, (int32_t)nseg, m, seg);
     G2_CK(cudaGetLastError());
-    t->h_eb_seg = new int64_t[nseg + 1];
-    G2_CK(cudaMemcpyAsync(t->h_eb_seg, t->eb_seg, (size_t)(nseg + 1) * 8, cudaMemcpyDeviceToHost,
-                          st));
+    std::vector<int64_t> ends((size_t)nseg + 1);
+    G2_CK(cudaMemcpyAsync(ends.data(), seg, ends.size() * 8, cudaMemcpyDeviceToHost, st));
     G2_CK(cudaStreamSynchronize(st));
-    dfree(cnt, st); dfree(off, st); dfree(beg, st);
+    t->h_eb_seg = new int64_t[nseg + 1];
+    std::copy(ends.begin(), ends.end(), t->h_eb_seg);
+    t->eb_src = mem.take(src);
+    t->eb_dst = mem.take(dst);
+    t->eb_seg = mem.take(seg);
     t->eb_N = N;
     t->eb_nseg = (int32_t)nseg;
     return G2_OK;

@@ -180,6 +180,34 @@ inline cudaError_t dmalloc(T **p, size_t bytes, cudaStream_t st) {
     return dmalloc_bytes(reinterpret_cast<void **>(p), bytes, st);
 }
 
+// Blocks that a builder of a layout allocates: freed when it returns (ordered on
+// st), unless it has handed them on with take().
+class HeldBlocks {
+    cudaStream_t st;
+    void *block[8] = {};
+    int count = 0;
+
+public:
+    explicit HeldBlocks(cudaStream_t s) : st(s) {}
+    HeldBlocks(const HeldBlocks &) = delete;
+    ~HeldBlocks() {
+        while (count > 0) dfree(block[--count], st);
+    }
+    template <class T>
+    cudaError_t alloc(T **p, size_t bytes) {
+        if (count == 8) return cudaErrorInvalidValue;
+        const cudaError_t e = dmalloc(p, bytes, st);
+        if (e == cudaSuccess) block[count++] = *p;
+        return e;
+    }
+    template <class T>
+    T *take(T *p) {
+        for (int i = 0; i < count; ++i)
+            if (block[i] == p) block[i] = nullptr;
+        return p;
+    }
+};
+
 // Device buffer of at least `bytes` bytes for slot b (grown if needed; old
 // contents are NOT kept when it grows).  Allocation and release are ordered
 // on g->st, the stream of the call in progress on this handle.

@@ -89,3 +89,30 @@ def test_bfs_batch_goes_on_without_planes(g2, k):
     g2.g2_bfs_batch(dg, srcs, depth)
     assert g2.g2_diag_fail_alloc(0) == 0
     assert np.array_equal(depth.cpu().numpy(), want)
+
+
+def test_edge_blocking_is_all_or_nothing(g2):
+    """A rebuild that fails leaves no layout of another segment size behind: the
+    next request of the size before it builds, and its export is what it was."""
+    g = gg.rmat(9, seed=1)
+    dg = g2.load_graph(g)
+
+    def export():
+        ns = g2.g2_edge_block(dg, 100)
+        s, d = (torch.full((g.m,), -1, dtype=torch.int32, device="cuda") for _ in range(2))
+        seg = torch.full((ns + 1,), -1, dtype=torch.int64, device="cuda")
+        g2.g2_edge_block_export(dg, s, d, seg)
+        return [x.cpu().numpy() for x in (s, d, seg)]
+
+    want = export()
+    for nth in range(1, 20):
+        g2.g2_diag_fail_alloc(nth)
+        try:
+            g2.g2_edge_block(dg, 60)
+        except g2.G2Error as e:
+            assert e.status == g2.G2_ENOMEM
+        if g2.g2_diag_fail_alloc(0):
+            break
+        for a, b in zip(export(), want):
+            assert np.array_equal(a, b), nth
+    assert nth >= 7          # six arrays and the scan's
