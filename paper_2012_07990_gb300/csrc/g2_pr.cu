@@ -755,26 +755,32 @@ static g2_status ensure_seg_layout(g2_graph *g, cudaStream_t st) {
     const int32_t n = t->n, m = t->m;
     const size_t words = ((size_t)m + 31) / 32 + 8;
     const int64_t nchunks = ((int64_t)m + kSegArcs - 1) / kSegArcs;
-    int32_t *nz, *pos, *ccount;
+    // the graph's only when all of it is built
+    HeldBlocks mem(st);
+    uint32_t *head;
+    int32_t *nz, *pos, *ccount, *nzrow, *chunk_rank;
     G2_TRY(ws(g, B_I0, (size_t)n + 1, &nz));
     G2_TRY(ws(g, B_I1, (size_t)n + 1, &pos));
     G2_TRY(ws(g, B_TWC_S, (size_t)nchunks + 1, &ccount));
-    G2_CK(dmalloc(&t->seg_head, words * 4, st));
-    G2_CK(cudaMemsetAsync(t->seg_head, 0, words * 4, st));
-    k_seg_heads<<<grid_for(g, n, kCta), kCta, 0, st>>>(t->crowptr, n, t->seg_head, nz);
+    G2_CK(mem.alloc(&head, words * 4));
+    G2_CK(cudaMemsetAsync(head, 0, words * 4, st));
+    k_seg_heads<<<grid_for(g, n, kCta), kCta, 0, st>>>(t->crowptr, n, head, nz);
     G2_TRY(exclusive_scan_i32(g, nz, pos, n, st));
     G2_CK(cudaMemcpyAsync(g->h_ctr + 60, pos + n, 4, cudaMemcpyDeviceToHost, st));
     G2_CK(cudaStreamSynchronize(st));
     const int32_t nnz = g->h_ctr[60];
-    G2_CK(dmalloc(&t->seg_nzrow, ((size_t)nnz + 1) * 4, st));
-    k_seg_nzrow<<<grid_for(g, n, kCta), kCta, 0, st>>>(nz, pos, n, t->seg_nzrow);
-    G2_CK(dmalloc(&t->seg_chunk_rank, ((size_t)nchunks + 1) * 4, st));
+    G2_CK(mem.alloc(&nzrow, ((size_t)nnz + 1) * 4));
+    k_seg_nzrow<<<grid_for(g, n, kCta), kCta, 0, st>>>(nz, pos, n, nzrow);
+    G2_CK(mem.alloc(&chunk_rank, ((size_t)nchunks + 1) * 4));
     if (nchunks > 0) {
-        k_seg_chunk_heads<<<grid_for(g, nchunks, kCta), kCta, 0, st>>>(t->seg_head, nchunks, ccount);
-        G2_TRY(exclusive_scan_i32(g, ccount, t->seg_chunk_rank, (int32_t)nchunks, st));
+        k_seg_chunk_heads<<<grid_for(g, nchunks, kCta), kCta, 0, st>>>(head, nchunks, ccount);
+        G2_TRY(exclusive_scan_i32(g, ccount, chunk_rank, (int32_t)nchunks, st));
     }
     G2_CK(cudaGetLastError());
     G2_CK(cudaStreamSynchronize(st));
+    t->seg_head = mem.take(head);
+    t->seg_nzrow = mem.take(nzrow);
+    t->seg_chunk_rank = mem.take(chunk_rank);
     t->seg_nnzrow = nnz;
     return G2_OK;
 }

@@ -116,3 +116,26 @@ def test_edge_blocking_is_all_or_nothing(g2):
         for a, b in zip(export(), want):
             assert np.array_equal(a, b), nth
     assert nth >= 7          # six arrays and the scan's
+
+
+@pytest.mark.parametrize("kernel", ["seg", "blk", "merge"])
+def test_pagerank_layouts_are_all_or_nothing(g2, monkeypatch, kernel):
+    """PageRank on a graph whose layout could not be built builds it on the next
+    call."""
+    monkeypatch.setenv("G2_PR_KERNEL", kernel)
+    g = gg.rmat(9, seed=1)
+    want = oracle.pagerank_graph(g, 0.85, 5)
+    rank = torch.empty(g.n, dtype=torch.float32, device="cuda")
+    for nth in range(1, 60):
+        dg = g2.load_graph(g)
+        g2.g2_diag_fail_alloc(nth)
+        try:
+            g2.g2_pagerank(dg, 0.85, 5, rank)
+        except g2.G2Error as e:
+            assert e.status == g2.G2_ENOMEM
+        if g2.g2_diag_fail_alloc(0):
+            break
+        rank.fill_(-1)
+        g2.g2_pagerank(dg, 0.85, 5, rank)
+        assert np.abs(rank.cpu().numpy().astype(np.float64) - want).sum() <= 1e-5, nth
+    assert nth > 4
